@@ -102,6 +102,7 @@ int apply_H_internal(hub_t h, int spin, const void* X, int ld, void* Y, int ncol
     }
     a.center = alpha * (-0.5 * c0 * inv2 - shift);
     a.alpha = alpha;
+    a.shift = shift;
     a.beta = beta;
     a.coef = coef_dev;
     if ((rc = launch_stencil(h, a))) return rc;
@@ -188,7 +189,7 @@ int hub_create_grid(hub_t* out, int n1, int n2, int n3, double L1, double L2, do
     if (e == cudaSuccess) e = cudaMalloc((void**)&h->d_bar, 4 * sizeof(unsigned int));
     if (e == cudaSuccess) e = cudaMalloc((void**)&h->d_scal, 4096 * sizeof(double));
     if (e == cudaSuccess) e = cudaMalloc((void**)&h->d_tcmax, 4 * sizeof(unsigned));
-    if (e == cudaSuccess) e = cudaMalloc(&h->d_veff, (size_t)h->Nd * h->esize);
+    if (e == cudaSuccess) e = cudaMalloc(&h->d_veff, veff_bytes(h));
     if (e == cudaSuccess) e = cudaMemset(h->d_flags, 0, 8 * sizeof(int));
     if (e == cudaSuccess) e = cudaMemset(h->d_scal, 0, 4096 * sizeof(double));
     if (e != cudaSuccess) {
@@ -205,7 +206,7 @@ int hub_destroy(hub_t h) {
     for (auto& e : h->prof) { cudaEventDestroy(e.a); cudaEventDestroy(e.b); }
     free_table(h->proj);
     void* ptrs[] = {h->d_veff, h->d_work, h->d_work2, h->d_part, h->d_C, h->d_W, h->d_small,
-                    h->d_gpart, h->d_bf16, h->d_aux, h->d_flags, h->d_bar, h->d_scal, h->d_tcmax, h->d_dens,
+                    h->d_gpart, h->d_bf16, h->d_aux, h->d_flags, h->d_bar, h->d_scal, h->d_tcmax, h->d_cmax, h->d_dens,
                     h->d_veff_spin[0], h->d_veff_spin[1], h->d_rho_ws, h->d_vloc};
     for (void* p : ptrs)
         if (p) cudaFree(p);
@@ -808,7 +809,7 @@ static int density_setup(hub_t h, ScfState& st) {
     }
     for (int s = 0; s < ns; ++s)
         if (!h->d_veff_spin[s])
-            HUB_CUDA_TRY(h, cudaMalloc(&h->d_veff_spin[s], Nd * h->esize));
+            HUB_CUDA_TRY(h, cudaMalloc(&h->d_veff_spin[s], veff_bytes(h)));
     const double vol = h->dV * (double)h->Nd;
     for (int s = 0; s < ns; ++s)
         if ((rc = density_fill(h, st.rho_in[s], st.p.n_elec / ns / vol))) return rc;

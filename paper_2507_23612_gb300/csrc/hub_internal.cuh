@@ -175,6 +175,7 @@ struct hub_ctx {
     int* d_flags = nullptr;       // [8] device error flags (0..5), Jacobi sweep count (6)
     unsigned int* d_bar = nullptr;  // [4] grid-barrier state
     double* d_scal = nullptr;     // [256] device scalars (Lanczos, reductions)
+    unsigned* d_cmax = nullptr;   size_t cmax_bytes = 0;    // column maxima of the FP64 stencil's input
     unsigned* d_tcmax = nullptr;  // [4] max |x| bit patterns of the FP16 operands (scales)
 
     hub::ScfState* scf = nullptr;
@@ -238,6 +239,7 @@ struct StencilArgs {
     int n1, n2, n3, ld, ncol;
     double w[3][kMaxHalf];  // alpha * (-1/2) c_p / h_a^2
     double center;          // alpha * ((-1/2) c0 sum_a h_a^-2 - shift)
+    double shift;
     double alpha;           // multiplies V
     double beta;
     int n0;
@@ -247,6 +249,14 @@ struct StencilArgs {
 };
 int launch_stencil(hub_t h, const StencilArgs& a);
 int stencil_variants(hub_t h);
+// stencil_fx.cu: the real FP64 stencil in fixed point.  A potential of Nd doubles is followed
+// by its fixed-point form (fx_veff_bytes bytes), written by launch_fx_veff
+int launch_stencil_fx(hub_t h, const StencilArgs& a);
+size_t fx_veff_bytes(int64_t Nd);
+int launch_fx_veff(hub_t h, const void* V);
+inline size_t veff_bytes(const hub_ctx* h) {
+    return (size_t)h->Nd * h->esize + (h->esize == 8 && !h->cplx ? fx_veff_bytes(h->Nd) : 0);
+}
 
 // projectors.cu
 int build_tables(hub_t h, int natoms, const double* pos, const int* kb_nchan, const int* kb_l,

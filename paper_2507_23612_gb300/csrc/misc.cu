@@ -164,11 +164,13 @@ int lanczos_t(hub_t h, int spin, int steps, const void* v0, double* lo, double* 
 
 int launch_copy_convert_veff(hub_t h, const double* src, void* dst) {
     const unsigned nb = (unsigned)((h->Nd + 255) / 256);
-    ProfScope ps(h, HUB_K_COPY);
-    if (h->esize == 8) k_convert<double><<<nb, 256, 0, h->stream>>>(src, (double*)dst, h->Nd);
-    else k_convert<float><<<nb, 256, 0, h->stream>>>(src, (float*)dst, h->Nd);
+    {
+        ProfScope ps(h, HUB_K_COPY);
+        if (h->esize == 8) k_convert<double><<<nb, 256, 0, h->stream>>>(src, (double*)dst, h->Nd);
+        else k_convert<float><<<nb, 256, 0, h->stream>>>(src, (float*)dst, h->Nd);
+    }
     HUB_CUDA_TRY(h, cudaGetLastError());
-    return HUB_OK;
+    return h->esize == 8 && !h->cplx ? launch_fx_veff(h, dst) : HUB_OK;
 }
 
 int launch_copy_block(hub_t h, const void* src, int lds, void* dst, int ldd, int ncol) {

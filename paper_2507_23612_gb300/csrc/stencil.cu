@@ -1516,7 +1516,7 @@ int launch_fd_gradient(hub_t h, const void* X, int ld, int ncol, int axis, const
 int stencil_variants(hub_t h) {
     const int es = h->esize * (h->cplx ? 2 : 1);
     if (h->esize == 4) return h->cplx ? 6 : 9;   // float real (packed) / float complex (packed, vector)
-    return es == 16 ? 2 : 3;              // double complex / double real (scalar pipeline)
+    return es == 16 ? 2 : 3;              // double complex (scalar pipeline) / double real (fixed point)
 }
 
 int launch_stencil(hub_t h, const StencilArgs& a) {
@@ -1555,11 +1555,7 @@ int launch_stencil(hub_t h, const StencilArgs& a) {
     // FP64 is bound by the FP64 pipe: a short ring keeps two CTAs per SM
     if (h->esize == 8) {
         if (h->cplx) return v == 1 ? run_cfg<double, true, 32, 4, 2>(h, a) : run_cfg<double, true, 32, 8, 2>(h, a);
-        switch (v) {
-            case 1: return run_cfg<double, false, 32, 4, 4>(h, a);
-            case 2: return run_cfg<double, false, 64, 4, 2>(h, a);
-            default: return run_cfg<double, false, 32, 8, 2>(h, a);
-        }
+        return launch_stencil_fx(h, a);
     }
     return h->cplx ? run_cfg<float, true, 32, 8, 2>(h, a) : run_cfg<float, false, 32, 8, 4>(h, a);
 }
