@@ -105,6 +105,7 @@ int apply_H_internal(hub_t h, int spin, const void* X, int ld, void* Y, int ncol
     a.shift = shift;
     a.beta = beta;
     a.coef = coef_dev;
+    a.cmax_ready = h->proj.nsites > 0 && gather_digits(h, ncol);
     if ((rc = launch_stencil(h, a))) return rc;
     if (h->proj.nsites > 0)
         if ((rc = launch_scatter(h, Y, ncol, ld, alpha, coef_dev))) return rc;
@@ -206,7 +207,7 @@ int hub_destroy(hub_t h) {
     for (auto& e : h->prof) { cudaEventDestroy(e.a); cudaEventDestroy(e.b); }
     free_table(h->proj);
     void* ptrs[] = {h->d_veff, h->d_work, h->d_work2, h->d_part, h->d_C, h->d_W, h->d_small,
-                    h->d_gpart, h->d_bf16, h->d_aux, h->d_flags, h->d_bar, h->d_scal, h->d_tcmax, h->d_cmax, h->d_dens,
+                    h->d_gpart, h->d_bf16, h->d_aux, h->d_flags, h->d_bar, h->d_scal, h->d_tcmax, h->d_cmax, h->d_wmax, h->d_dens,
                     h->d_veff_spin[0], h->d_veff_spin[1], h->d_rho_ws, h->d_vloc};
     for (void* p : ptrs)
         if (p) cudaFree(p);
@@ -528,7 +529,7 @@ int hub_expand(hub_t h, const double* W_host, int ncol, void* Y, int ld, double 
         HUB_CUDA_TRY(h, cudaMemcpyAsync(h->d_W, wf.data(), n * sizeof(float), cudaMemcpyHostToDevice, h->stream));
         HUB_CUDA_TRY(h, cudaStreamSynchronize(h->stream));     // wf goes out of scope
     }
-    return launch_scatter(h, Y, ncol, ld, alpha);
+    return launch_scatter(h, Y, ncol, ld, alpha, nullptr, false);
 }
 
 int hub_hubbard_forces(hub_t h, int spin, const void* X, int ncol, int ld, const double* f_host,

@@ -96,6 +96,20 @@ struct Table {
     int* d_frow = nullptr;            // [npart_rows] global projector row (-1: padding)
     int* d_roff = nullptr;            // [nproj + 1] partial rows of each projector row (CSR)
     int* d_rent = nullptr;
+    // digit form of the bricks (projectors_oz.cu): FP64 and complex blocks, and real float ones
+    // without the brick tables above.  A function has one slot (real) or two (complex)
+    int oz = 0;                       // 1 when the arrays below are built
+    int oz_ngroups = 0, oz_nbricks = 0;
+    long oz_npart = 0;                // (function, brick) pairs: partial rows of the gather
+    int4* d_ozg = nullptr;            // per group: brick, slots, 16-byte offset of its values, first slot
+    int2* d_ozg_row = nullptr;        // per slot: partial row (x slots per function; -1 padding), exponent
+    uint4* d_ozg_val = nullptr;
+    int4* d_ozb = nullptr;            // per brick: brick, slots, 16-byte offset of its values, first slot
+    int2* d_ozb_row = nullptr;        // per slot: real row of W (-1 padding), exponent
+    uint4* d_ozb_val = nullptr;
+    int* d_oz_exp = nullptr;          // [nproj] biased exponent of each function's largest value
+    int* d_oz_roff = nullptr;         // [nproj + 1] partial rows of each projector row (CSR)
+    int* d_oz_rent = nullptr;
     // tensor-core form of the brick gather (built with the bricks when n1 % 4 == 0): the
     // entries of each brick packed into groups of at most 64 functions, per group its values
     // in the 128-byte-swizzled K-major layout of tcgen05 operands, split as TF32 hi + lo,
@@ -175,7 +189,8 @@ struct hub_ctx {
     int* d_flags = nullptr;       // [8] device error flags (0..5), Jacobi sweep count (6)
     unsigned int* d_bar = nullptr;  // [4] grid-barrier state
     double* d_scal = nullptr;     // [256] device scalars (Lanczos, reductions)
-    unsigned* d_cmax = nullptr;   size_t cmax_bytes = 0;    // column maxima of the FP64 stencil's input
+    unsigned* d_cmax = nullptr;   size_t cmax_bytes = 0;    // column maxima (colmax.cu)
+    int* d_wmax = nullptr;        size_t wmax_bytes = 0;    // column maxima of W (projectors_oz.cu)
     unsigned* d_tcmax = nullptr;  // [4] max |x| bit patterns of the FP16 operands (scales)
 
     hub::ScfState* scf = nullptr;
@@ -245,10 +260,23 @@ struct StencilArgs {
     int n0;
     double phase[3][2];     // exp(i k_a L_a) (re, im), complex only
     const double* coef;     // device {alpha, beta, shift} or nullptr (then w/center/alpha/beta)
+    bool cmax_ready;        // d_cmax holds the column maxima of Y
     double wbase[3][kMaxHalf];  // (-1/2) c_p / h_a^2 (alpha = 1)
 };
 int launch_stencil(hub_t h, const StencilArgs& a);
 int stencil_variants(hub_t h);
+// colmax.cu: h->d_cmax[col * kColParts + i], the largest leading word of |x| over slice i of
+// each column (biased exponent on top)
+constexpr int kColParts = 8;
+int launch_colmax(hub_t h, const void* X, int ncol, int ld);
+#ifdef __CUDACC__
+__device__ __forceinline__ unsigned column_max(const unsigned* cmax, int col) {
+    unsigned m = 0;
+#pragma unroll
+    for (int i = 0; i < kColParts; ++i) m = max(m, cmax[(size_t)col * kColParts + i]);
+    return m;
+}
+#endif
 // stencil_fx.cu: the real FP64 stencil in fixed point.  A potential of Nd doubles is followed
 // by its fixed-point form (fx_veff_bytes bytes), written by launch_fx_veff
 int launch_stencil_fx(hub_t h, const StencilArgs& a);
@@ -269,7 +297,8 @@ void free_table(Table& t);
 int launch_gather(hub_t h, const void* X, int ncol, int ld, int spin, bool want_W);
 // Y[g, n] += alpha * sum_e vals_e . W[rows_e, n]   (W from the last launch_gather); with
 // alpha_dev != nullptr alpha is read on the device
-int launch_scatter(hub_t h, void* Y, int ncol, int ld, double alpha, const double* alpha_dev = nullptr);
+int launch_scatter(hub_t h, void* Y, int ncol, int ld, double alpha, const double* alpha_dev = nullptr,
+                   bool w_from_gather = true);
 // D per Hubbard atom (double, [nhub*50] re/im pairs) and E_U into d_scal[0] from the C of
 // the last launch_gather; f_dev [ncol] double.
 int launch_occupation(hub_t h, int ncol, const double* f_dev, double kweight, double* D_dev);
@@ -285,6 +314,15 @@ int build_tc_tables(hub_t h, Table& t);
 int launch_gather_tc(hub_t h, const void* X, int ncol, int ld);
 // Y += alpha Phi W (W of the last launch_gather) in the tensor-core brick form
 int launch_scatter_tc(hub_t h, void* Y, int ncol, int ld, double alpha, const double* alpha_dev);
+
+// projectors_oz.cu: digit form of the gather and scatter; launch_gather and launch_scatter take it
+// where these say so.  site_pts: grid points of each site, ascending
+bool gather_digits(hub_t h, int ncol);
+bool scatter_digits(hub_t h, int ncol);
+int build_oz_tables(hub_t h, Table& t, const std::vector<std::vector<int>>& site_pts);
+int launch_gather_oz(hub_t h, const void* X, int ncol, int ld, int spin, bool want_W);
+// wmax_ready: d_wmax holds the maxima of W (both written by launch_gather_oz)
+int launch_scatter_oz(hub_t h, void* Y, int ncol, int ld, double alpha, const double* alpha_dev, bool wmax_ready);
 
 // Moment integrals of the stress: Gm_b = dV <(x - R_image)_b phi_m | G> for the Hubbard rows
 // (layout of d_C: [nproj x ncol] doubles, x2 complex; other rows untouched), b = x, y, z

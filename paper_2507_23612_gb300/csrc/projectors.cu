@@ -20,6 +20,7 @@
 
 #include "hub_internal.cuh"
 #include "cplx.cuh"
+#include "site_transform.cuh"
 
 namespace hub {
 
@@ -213,37 +214,6 @@ k_gather(const typename VT<R, CPLX>::T* __restrict__ X, int ld, int ncol,
         case 8: gather_body<T, D, 8, NC, PTS>(X, ld, nc, c0, idx, vp0, first, cnt, lane, part, pbase, ncol); break;
         case 9: gather_body<T, D, 9, NC, PTS>(X, ld, nc, c0, idx, vp0, first, cnt, lane, part, pbase, ncol); break;
         default: break;   // build_tables rejects sites with more than kMaxProj functions
-    }
-}
-
-// W row of a site from its inner products c (KB: gamma C; Hubbard: M C, Eq. DerED)
-template <typename R, bool CPLX>
-__device__ __forceinline__ void site_transform(const SiteDev& S, const typename VT<double, CPLX>::T* c,
-                                               const double* __restrict__ gamma, const double* __restrict__ M,
-                                               typename VT<R, CPLX>::T* __restrict__ W, int n, int ncol) {
-    using D = typename VT<double, CPLX>::T;
-    using T = typename VT<R, CPLX>::T;
-    for (int p = 0; p < S.nproj; ++p) {
-        D w = zero_of(D());
-        if (S.kind == 0) {
-            w = mulr(gamma[S.proj_off + p], c[p]);
-        } else {
-            // coefficient of phi_p: sum_m M[p][m] C_m  (M = (U/2)(I - 2D))
-            for (int m = 0; m < S.nproj; ++m) {
-                D mm;
-                if constexpr (CPLX) {
-                    const double* Mi = M + (size_t)S.hub_index * 50;
-                    mm = make_double2(Mi[2 * (p * 5 + m)], Mi[2 * (p * 5 + m) + 1]);
-                } else {
-                    mm = M[(size_t)S.hub_index * 25 + p * 5 + m];
-                }
-                w = cfma(mm, c[m], w);
-            }
-        }
-        T wv;
-        if constexpr (CPLX) wv = T{(R)w.x, (R)w.y};
-        else wv = (R)w;
-        W[(size_t)(S.proj_off + p) * ncol + n] = wv;
     }
 }
 
@@ -777,7 +747,8 @@ void free_table(Table& t) {
                     t.d_csr_ent, t.d_order, t.d_gamma, t.d_hub_sites, t.d_U,
                     t.d_M[0], t.d_M[1], t.d_bent, t.d_bfirst, t.d_phi, t.d_frow, t.d_roff,
                     t.d_rent, t.d_tcg, t.d_tcg_row, t.d_tchi, t.d_tclo, t.d_tcs_brick, t.d_tcs_frow, t.d_tcs_hi,
-                    t.d_tcs_lo};
+                    t.d_tcs_lo, t.d_ozg, t.d_ozg_row, t.d_ozg_val, t.d_ozb, t.d_ozb_row, t.d_ozb_val, t.d_oz_exp,
+                    t.d_oz_roff, t.d_oz_rent};
     for (void* p : ptrs)
         if (p) cudaFree(p);
     t = Table();
@@ -1080,6 +1051,10 @@ int build_tables(hub_t h, int natoms, const double* pos, const int* kb_nchan, co
         HUB_CUDA_TRY(h, cudaStreamSynchronize(h->stream));     // values are ready
         if ((rc = build_bricks(h, t, site_pts))) return rc;
     }
+    if (!t.dense && t.nsites > 0) {
+        HUB_CUDA_TRY(h, cudaStreamSynchronize(h->stream));     // values are ready
+        if ((rc = build_oz_tables(h, t, site_pts))) return rc;
+    }
     const size_t mbytes = (size_t)std::max(t.nhub, 1) * 25 * sizeof(double) * (h->cplx ? 2 : 1);
     for (int s = 0; s < 2; ++s) {
         HUB_CUDA_TRY(h, cudaMalloc((void**)&t.d_M[s], mbytes));
@@ -1183,6 +1158,7 @@ static int gather_t(hub_t h, const void* X, int ncol, int ld, int spin, bool wan
 
 int launch_gather(hub_t h, const void* X, int ncol, int ld, int spin, bool want_W) {
     if (ncol == 0 || h->proj.nsites == 0) return HUB_OK;
+    if (gather_digits(h, ncol)) return launch_gather_oz(h, X, ncol, ld, spin, want_W);
     if (h->gather_dense && use_dense(h, X, ld)) return gather_dense(h, X, ncol, ld, spin, want_W);
     if (h->esize == 8) return h->cplx ? gather_t<double, true>(h, X, ncol, ld, spin, want_W)
                                       : gather_t<double, false>(h, X, ncol, ld, spin, want_W);
@@ -1205,8 +1181,10 @@ static int scatter_t(hub_t h, void* Y, int ncol, int ld, double alpha, const dou
     return HUB_OK;
 }
 
-int launch_scatter(hub_t h, void* Y, int ncol, int ld, double alpha, const double* alpha_dev) {
+int launch_scatter(hub_t h, void* Y, int ncol, int ld, double alpha, const double* alpha_dev, bool w_from_gather) {
     if (ncol == 0 || h->proj.nsites == 0) return HUB_OK;
+    if (scatter_digits(h, ncol))
+        return launch_scatter_oz(h, Y, ncol, ld, alpha, alpha_dev, w_from_gather && gather_digits(h, ncol));
     if (use_dense(h, Y, ld)) {
         if (h->gather_dense == 3 && h->proj.tc) return launch_scatter_tc(h, Y, ncol, ld, alpha, alpha_dev);
         return scatter_dense(h, Y, ncol, ld, alpha, alpha_dev);

@@ -6,7 +6,7 @@
 //   Yout = alpha * (-1/2 Lap_h Y + V .* Y - shift * Y) + beta * Yprev        (Sec. II.B)
 //
 // Number format.  Every column has one power-of-two scale: with E the biased exponent of its
-// largest |x| (k_fx_colmax), X = x * 2^(1081 - E) rounded to an integer, |X| <= 2^59, so an
+// largest |x| (colmax.cu), X = x * 2^(1081 - E) rounded to an integer, |X| <= 2^59, so an
 // element keeps all 53 bits down to 2^-6 of the column's maximum and is never off by more
 // than 2^-60 of it (one FP64 rounding of the sum, which holds terms of ~300 x, is larger).
 // X is kept as two signed limbs, X = xh 2^30 + xl: pair sums of limbs need no carry.
@@ -38,7 +38,6 @@ namespace {
 constexpr int FXH = 6;             // halo
 constexpr int FXP = 44;            // row pitch of a plane in shared memory: tiles of at most 32 points
 constexpr int FXS = 8;             // ring planes
-constexpr int FXPARTS = 8;         // partial maxima per column
 constexpr int kFxEmin = 123, kFxEmax = 1923;
 
 struct FxArgs {
@@ -48,7 +47,7 @@ struct FxArgs {
     const double* V;
     const int2* Vq;               // (V 2^(sf - 25)) as limbs of 30 bits
     const int* vinfo;             // largest high word of |V|; not covered (0 or 1); sf
-    const unsigned* cmax;         // [ncol * FXPARTS] largest high words of |x|
+    const unsigned* cmax;         // column maxima (colmax.cu)
     int n1, n2, n3, ld;
     int tx, ty, tilesx, tiles;    // tile shape and count
     int zchunk, nzc;
@@ -120,10 +119,7 @@ k_stencil_fx(const __grid_constant__ FxArgs a) {
     const double alpha = a.coef ? a.coef[0] : a.alpha, beta = a.coef ? a.coef[1] : a.beta;
     const double shift = a.coef ? a.coef[2] : a.shift;
 
-    unsigned mx = 0;
-#pragma unroll
-    for (int i = 0; i < FXPARTS; ++i) mx = max(mx, a.cmax[(size_t)col * FXPARTS + i]);
-    const int emax = (int)(mx >> 20);
+    const int emax = (int)(column_max(a.cmax, col) >> 20);
     const int sf = a.vinfo[2];
     const bool fits = fabs(shift) < scalbn(1.0, 83 - sf);       // NaN: false
     if (emax < kFxEmin || emax > kFxEmax || !fits || a.vinfo[1]) {    // the same for the whole CTA
@@ -246,32 +242,6 @@ k_stencil_fx(const __grid_constant__ FxArgs a) {
     }
 }
 
-// largest high word of |x| of every column, in FXPARTS slices (plain stores: no clearing)
-__global__ void __launch_bounds__(512)
-k_fx_colmax(const double* __restrict__ X, long ld, long Nd, unsigned* __restrict__ cmax) {
-    const double* col = X + (size_t)blockIdx.y * ld;
-    const long per = (Nd + FXPARTS - 1) / FXPARTS;
-    const long g0 = (long)blockIdx.x * per, g1 = min(g0 + per, Nd);
-    unsigned m = 0;
-    long g = g0 + threadIdx.x;
-    for (; g + 7 * 512 < g1; g += 8 * 512) {
-        unsigned v[8];
-#pragma unroll
-        for (int i = 0; i < 8; ++i) v[i] = (unsigned)__double2hiint(col[g + i * 512]) & 0x7fffffffu;
-#pragma unroll
-        for (int i = 0; i < 8; ++i) m = max(m, v[i]);
-    }
-    for (; g < g1; g += 512) m = max(m, (unsigned)__double2hiint(col[g]) & 0x7fffffffu);
-    __shared__ unsigned s[16];
-    m = __reduce_max_sync(0xffffffffu, m);
-    if ((threadIdx.x & 31) == 0) s[threadIdx.x >> 5] = m;
-    __syncthreads();
-    if (threadIdx.x < 32) {
-        m = __reduce_max_sync(0xffffffffu, threadIdx.x < 16 ? s[threadIdx.x] : 0u);
-        if (threadIdx.x == 0) cmax[(size_t)blockIdx.y * FXPARTS + blockIdx.x] = m;
-    }
-}
-
 __global__ void k_fx_vmax(const double* __restrict__ V, int* __restrict__ info, long n) {
     unsigned m = 0;
     for (long t = (long)blockIdx.x * blockDim.x + threadIdx.x; t < n; t += (long)gridDim.x * blockDim.x)
@@ -348,15 +318,7 @@ template <int NT, int CTAS, int FXPER>
 static int run_fx(hub_t h, const StencilArgs& s) {
     FxArgs a{};
     int rc;
-    if ((rc = ensure(h, (void**)&h->d_cmax, &h->cmax_bytes,
-                     std::max(h->cmax_bytes, (size_t)s.ncol * FXPARTS * sizeof(unsigned))))) return rc;
-    {
-        ProfScope ps(h, HUB_K_STENCIL);
-        for (int c0 = 0; c0 < s.ncol; c0 += 65535)
-            k_fx_colmax<<<dim3(FXPARTS, std::min(65535, s.ncol - c0)), 512, 0, h->stream>>>(
-                (const double*)s.Y + (size_t)c0 * s.ld, s.ld, h->Nd, h->d_cmax + (size_t)c0 * FXPARTS);
-    }
-    HUB_CUDA_TRY(h, cudaGetLastError());
+    if (!s.cmax_ready && (rc = launch_colmax(h, s.Y, s.ncol, s.ld))) return rc;
     a.Y = (const double*)s.Y;
     a.Yprev = (const double*)s.Yprev;
     a.Yout = (double*)s.Yout;
