@@ -153,6 +153,7 @@ struct hub_ctx {
     int prec = HUB_F64;
     int esize = 8;                // bytes per real component of the working type
     int bf16_terms = 3;           // mixed handles: 1 = one 16-bit product, 3 = hi/lo split products
+    int fx_plan[3] = {-1, 0, 0};  // FP64 stencil: key (columns, variant), rows per tile, planes per chunk
     int stencil_variant = 0;      // tile shape chosen by the autotuner (stencil_variants)
     int gather_dense = 0;         // real float: gather in the brick form (else point-major)
     int gemm_split = 2;           // tensor-core split-K: CTAs per SM of the Gram products

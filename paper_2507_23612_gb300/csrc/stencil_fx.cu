@@ -22,10 +22,12 @@
 // that would leave F under 51 bits and shifts beyond 2^(83 - sf) Ha (the largest kinetic
 // energy of the grid, at least) are computed by fx_slow in plain FP64.
 //
-// Kernel: one CTA owns a TX x TY tile of the x-y plane of one column and marches along z.  A
-// ring of 8 planes (with a halo of 6 in x and y) in shared memory holds the limbs; plane z + 7
-// is converted and stored while plane z is computed, and plane z + 8 is in flight in
-// registers, so there is one barrier per plane.  The 13 z-neighbours live in registers.
+// Kernel: one CTA owns a tile of the x-y plane of one column and marches along z.  A ring of 8
+// planes (with a halo of 6 in x and y) in shared memory holds the limbs; plane z + 7 is
+// converted and stored while plane z is computed, and plane z + 8 is in flight in registers, so
+// there is one barrier per plane.  The 13 z-neighbours live in registers.  Bound: the integer
+// pipes (50 multiply-adds at half rate and ~300 other instructions per point); 17.15 -> 4.12 ms
+// on 88 x 88 x 84 x 348 (DRAM floor 0.80 ms), plus 0.27 ms for the column maxima.
 #include <algorithm>
 #include <cmath>
 
@@ -64,17 +66,16 @@ __device__ __forceinline__ int wrap(int i, int n) {      // i is at most a few n
     return i;
 }
 
-// x as limbs, emax the biased exponent of the column's maximum (>= 123, so that a denormal x
-// shifts to zero whatever its hidden bit)
-__device__ __forceinline__ int2 to_limbs(double v, int emax) {
+// x as limbs, cut towards zero; e20 the biased exponent of the column's maximum << 20 (at least
+// 123, so that a denormal x shifts to zero whatever its hidden bit)
+__device__ __forceinline__ int2 to_limbs(double v, int e20) {
     const unsigned hi = (unsigned)__double2hiint(v), lo = (unsigned)__double2loint(v);
-    const int e = (int)(hi >> 20) & 0x7ff;
-    const int sh = min(emax - e, 63);
-    unsigned long long t = ((unsigned long long)((hi & 0xfffffu) | 0x100000u) << 32) | lo;
-    t = (((t << 7) >> sh) + 1) >> 1;
-    int xh = (int)(t >> 30), xl = (int)((unsigned)t & 0x3fffffffu);
-    if ((int)hi < 0) { xh = -xh; xl = -xl; }
-    return make_int2(xh, xl);
+    const int s = min((e20 - (int)(hi & 0x7ff00000u)) >> 20, 61) + 2;
+    // the significand times 2^8, 61 bits: X = t >> s
+    const unsigned th = __funnelshift_l(lo, (hi & 0xfffffu) | 0x100000u, 8), tl = lo << 8;
+    const unsigned xl = (unsigned)((((unsigned long long)th << 32) | tl) >> s) & 0x3fffffffu;
+    const unsigned xh = __funnelshift_rc(th, 0u, s - 2);
+    return (int)hi < 0 ? make_int2(-(int)xh, -(int)xl) : make_int2((int)xh, (int)xl);
 }
 
 // the plain FP64 form of one tile and chunk, straight from global memory
@@ -98,11 +99,11 @@ __device__ __noinline__ void fx_slow(const FxArgs& a, const double* __restrict__
     }
 }
 
-// (hi, lo) sums of limb products: acc += w * s
 __device__ __forceinline__ void mad(long long& acc, int s, int w) { acc += (long long)s * w; }
 
-// PER: halo'd points per thread
-template <bool YP, int NTMAX, int CTAS, int FXPER>
+// ROWS = 2: two rows per thread; the 14 rows that the y-sums of both need are loaded once, the
+// halo is 12 rows for twice the tile's, and the loop's own instructions serve two points.
+template <bool YP, int ROWS, int NTMAX, int CTAS, int PER>
 __global__ void __launch_bounds__(NTMAX, CTAS)
 k_stencil_fx(const __grid_constant__ FxArgs a) {
     extern __shared__ __align__(16) int2 ring[];
@@ -112,14 +113,14 @@ k_stencil_fx(const __grid_constant__ FxArgs a) {
     const int gx0 = (tile % a.tilesx) * a.tx, gy0 = (tile / a.tilesx) * a.ty;
     const int z0 = zc * a.zchunk, z1 = min(z0 + a.zchunk, a.n3);
     const int n1 = a.n1, n2 = a.n2, n3 = a.n3;
-    const long plane = (long)n1 * n2;
+    const long plane = (long)n1 * n2, cell = plane * n3;
     const double* __restrict__ Y = a.Y + (size_t)col * a.ld;
     const double* Yp = YP ? a.Yprev + (size_t)col * a.ld : nullptr;
     double* Yo = a.Yout + (size_t)col * a.ld;
     const double alpha = a.coef ? a.coef[0] : a.alpha, beta = a.coef ? a.coef[1] : a.beta;
     const double shift = a.coef ? a.coef[2] : a.shift;
 
-    const int emax = (int)(column_max(a.cmax, col) >> 20);
+    const int emax = (int)(column_max(a.cmax, col) >> 20), e20 = emax << 20;
     const int sf = a.vinfo[2];
     const bool fits = fabs(shift) < scalbn(1.0, 83 - sf);       // NaN: false
     if (emax < kFxEmin || emax > kFxEmax || !fits || a.vinfo[1]) {    // the same for the whole CTA
@@ -128,6 +129,7 @@ k_stencil_fx(const __grid_constant__ FxArgs a) {
     }
     const double scale = scalbn(alpha, 81 - sf + emax - 1081);
     const long long shq = __double2ll_rn(scalbn(shift, sf - 25));
+    const int shh = (int)(shq >> 30), shl = (int)(shq & 0x3fffffff);
     int fh[3], fl[3];                             // F 2^sf as limbs of 30 bits
 #pragma unroll
     for (int ax = 0; ax < 3; ++ax) {
@@ -135,19 +137,18 @@ k_stencil_fx(const __grid_constant__ FxArgs a) {
         fh[ax] = (int)(fq >> 30);
         fl[ax] = (int)(fq & 0x3fffffff);
     }
-    const int shh = (int)(shq >> 30), shl = (int)(shq & 0x3fffffff);
     // Sums start at half a unit of the bits shifted out, M1 also at the mean of the dropped
     // ul * fl: a bias of one unit would be the same at every point, and the filter, which keeps
     // the smooth part of its input and damps the rest, would keep all of it
     const long long m1 = (1 << 29) + (((long long)fl[0] + fl[1] + fl[2]) >> 1);
 
-    // this thread's halo'd points of a plane
-    const int sx = a.tx + 2 * FXH, sy = a.ty + 2 * FXH, stage = sy * FXP;
-    int s_idx[FXPER], s_off[FXPER];
+    // this thread's halo'd points of a plane (beyond the last one: a point that nobody reads)
+    const int sx = a.tx + 2 * FXH, sy = a.ty + 2 * FXH, stage = sy * FXP + 2;
+    int s_idx[PER], s_off[PER];
 #pragma unroll
-    for (int k = 0; k < FXPER; ++k) {
+    for (int k = 0; k < PER; ++k) {
         const int i = tid + k * nt;
-        s_idx[k] = -1;
+        s_idx[k] = sy * FXP;
         s_off[k] = 0;
         if (i < sx * sy) {
             const int iy = i / sx, ix = i - iy * sx;
@@ -155,89 +156,154 @@ k_stencil_fx(const __grid_constant__ FxArgs a) {
             s_off[k] = wrap(gy0 - FXH + iy, n2) * n1 + wrap(gx0 - FXH + ix, n1);
         }
     }
+    // rows ROWS * ty .. of the tile
     const int ty = tid / a.tx, tx = tid - ty * a.tx;
-    const bool active = ty < a.ty && gx0 + tx < n1 && gy0 + ty < n2;
-    // inactive threads read a point of their own plane region (never stored)
-    const int ctr = active ? (ty + FXH) * FXP + tx + FXH : FXH * FXP + FXH;
-    const int own = active ? (gy0 + ty) * n1 + gx0 + tx : gy0 * n1 + gx0;
+    bool act[ROWS];
+    int own[ROWS];
+#pragma unroll
+    for (int r = 0; r < ROWS; ++r) {
+        const int y = ROWS * ty + r;
+        act[r] = y < a.ty && gx0 + tx < n1 && gy0 + y < n2;
+        own[r] = act[r] ? (gy0 + y) * n1 + gx0 + tx : gy0 * n1 + gx0;
+    }
+    const int ctr = act[0] ? (ROWS * ty + FXH) * FXP + tx + FXH : FXH * FXP + FXH;
     const int last = z1 + FXH - 1;                // highest plane needed
 
-    auto load = [&](int p, double (&v)[FXPER]) {
-        const double* src = Y + (long)wrap(p, n3) * plane;
+    auto load = [&](long zo, double (&v)[PER]) {
 #pragma unroll
-        for (int k = 0; k < FXPER; ++k) v[k] = s_idx[k] >= 0 ? src[s_off[k]] : 0.0;
+        for (int k = 0; k < PER; ++k) v[k] = Y[zo + s_off[k]];
     };
-    auto store = [&](int p, const double (&v)[FXPER]) {
-        int2* dst = ring + (p & (FXS - 1)) * stage;
+    auto store = [&](int j, const double (&v)[PER]) {
+        int2* dst = ring + (j & (FXS - 1)) * stage;
 #pragma unroll
-        for (int k = 0; k < FXPER; ++k)
-            if (s_idx[k] >= 0) dst[s_idx[k]] = to_limbs(v[k], emax);
+        for (int k = 0; k < PER; ++k) dst[s_idx[k]] = to_limbs(v[k], e20);
     };
 
     // planes z0 .. z0 + 6 into the ring (stage index: plane - z0), z-queue z0 - 6 .. z0 + 5
-    double pf[FXPER];
+    double pf[PER];
+    long zl = (long)z0 * plane;                   // plane to load next
     for (int j = 0; j <= FXH; ++j) {
-        load(z0 + j, pf);
+        load(zl, pf);
         store(j, pf);
+        zl += plane;
+        if (zl == cell) zl = 0;
     }
-    int2 q[2 * FXH + 1];
-    {
-        double v[FXH];
+    int2 q[ROWS][2 * FXH + 1];                    // [i]: plane z - 7 + i before the shift
 #pragma unroll
-        for (int j = 0; j < FXH; ++j) v[j] = Y[(long)wrap(z0 - FXH + j, n3) * plane + own];
+    for (int j = 0; j < FXH; ++j) {
+        const long zo = (long)wrap(z0 - FXH + j, n3) * plane;
 #pragma unroll
-        for (int j = 0; j < FXH; ++j) q[1 + j] = to_limbs(v[j], emax);
+        for (int r = 0; r < ROWS; ++r) q[r][1 + j] = to_limbs(Y[zo + own[r]], e20);
     }
-    load(z0 + FXH + 1 <= last ? z0 + FXH + 1 : last, pf);
-    int2 vq = a.Vq[(long)z0 * plane + own];
-    double yp = YP ? Yp[(long)z0 * plane + own] : 0.0;
+    load(zl, pf);                                 // plane z0 + 7 (needed or not: inside the block)
+    long zo = (long)z0 * plane;
+    int2 vq[ROWS];
+    double yp[ROWS];
+#pragma unroll
+    for (int r = 0; r < ROWS; ++r) {
+        vq[r] = a.Vq[zo + own[r]];
+        yp[r] = YP ? Yp[zo + own[r]] : 0.0;
+    }
     __syncthreads();
 #pragma unroll
-    for (int j = 0; j < FXH; ++j) q[FXH + 1 + j] = ring[j * stage + ctr];
+    for (int j = 0; j < FXH; ++j)
+#pragma unroll
+        for (int r = 0; r < ROWS; ++r) q[r][FXH + 1 + j] = ring[j * stage + ctr + r * FXP];
 
-    // The loop body is one plane; the shift of the queue is 24 register moves
 #pragma unroll 1
     for (int j = 0; j < z1 - z0; ++j) {
-        const int z = z0 + j;
+        const int2* f = ring + ((j + FXH) & (FXS - 1)) * stage + ctr;
 #pragma unroll
-        for (int i = 0; i < 2 * FXH; ++i) q[i] = q[i + 1];
-        q[2 * FXH] = ring[((j + FXH) & (FXS - 1)) * stage + ctr];
-        if (z + FXH + 1 <= last) store(j + FXH + 1, pf);          // the ring slot of plane z - 1
-        if (z + FXH + 2 <= last) load(z + FXH + 2, pf);
-        const int2 vc = make_int2(vq.x - shh, vq.y - shl);
-        const double ypc = yp;
-        if (z + 1 < z1) {
-            vq = a.Vq[(long)(z + 1) * plane + own];
-            if (YP) yp = Yp[(long)(z + 1) * plane + own];
+        for (int r = 0; r < ROWS; ++r) {
+#pragma unroll
+            for (int i = 0; i < 2 * FXH; ++i) q[r][i] = q[r][i + 1];
+            q[r][2 * FXH] = f[r * FXP];
         }
-        const int2 c = q[FXH];
-        const long long ch = (long long)c.x * a.k[0], cl = (long long)c.y * a.k[0] + (1 << 19);
-        long long H = 0, M1 = m1, M2 = 1 << 30;
-        const int2* ps = ring + (j & (FXS - 1)) * stage + ctr;
+        store(j + FXH + 1, pf);                   // the ring slot of plane z - 1
+        if (z0 + j + FXH + 2 <= last) {
+            zl += plane;
+            if (zl == cell) zl = 0;
+            load(zl, pf);
+        }
+        int2 vc[ROWS];
+        double ypc[ROWS];
+        const long zn = zo + plane;
 #pragma unroll
-        for (int ax = 0; ax < 3; ++ax) {
-            long long A = ch, B = cl;
+        for (int r = 0; r < ROWS; ++r) {
+            vc[r] = make_int2(vq[r].x - shh, vq[r].y - shl);
+            ypc[r] = yp[r];
+            if (j + 1 < z1 - z0) {
+                vq[r] = a.Vq[zn + own[r]];
+                if (YP) yp[r] = Yp[zn + own[r]];
+            }
+        }
+        long long ch[ROWS], cl[ROWS], H[ROWS], M1[ROWS], M2[ROWS], A[ROWS], B[ROWS];
+#pragma unroll
+        for (int r = 0; r < ROWS; ++r) {
+            ch[r] = (long long)q[r][FXH].x * a.k[0];
+            cl[r] = (long long)q[r][FXH].y * a.k[0] + (1 << 19);
+            H[r] = 0;
+            M1[r] = m1;
+            M2[r] = 1 << 30;
+        }
+        auto start = [&]() {
+#pragma unroll
+            for (int r = 0; r < ROWS; ++r) { A[r] = ch[r]; B[r] = cl[r]; }
+        };
+        auto pair = [&](int r, int2 u, int2 w, int k) {
+            mad(A[r], u.x + w.x, k);
+            mad(B[r], u.y + w.y, k);
+        };
+        auto end = [&](int ax) {
+#pragma unroll
+            for (int r = 0; r < ROWS; ++r) {
+                const long long U = (A[r] << 10) + (B[r] >> 20);
+                const int uh = (int)(U >> 31), ul = (int)((unsigned)U & 0x7fffffffu);
+                mad(H[r], uh, fh[ax]);
+                mad(M1[r], uh, fl[ax]);
+                mad(M2[r], ul, fh[ax]);
+            }
+        };
+        const int2* ps = ring + (j & (FXS - 1)) * stage + ctr;
+        start();
+#pragma unroll
+        for (int p = 1; p <= FXH; ++p)
+#pragma unroll
+            for (int r = 0; r < ROWS; ++r) pair(r, q[r][FXH + p], q[r][FXH - p], a.k[p]);
+        end(2);
+        start();
+#pragma unroll
+        for (int p = 1; p <= FXH; ++p)
+#pragma unroll
+            for (int r = 0; r < ROWS; ++r) pair(r, ps[r * FXP + p], ps[r * FXP - p], a.k[p]);
+        end(0);
+        start();
+        if constexpr (ROWS == 2) {
+            int2 up = q[1][FXH], dn = q[0][FXH];  // rows p and 1 - p
 #pragma unroll
             for (int p = 1; p <= FXH; ++p) {
-                int2 u, v;
-                if (ax == 2) { u = q[FXH + p]; v = q[FXH - p]; }
-                else { u = ps[ax == 0 ? p : p * FXP]; v = ps[ax == 0 ? -p : -p * FXP]; }
-                mad(A, u.x + v.x, a.k[p]);
-                mad(B, u.y + v.y, a.k[p]);
+                const int2 un = ps[(p + 1) * FXP], dm = ps[-p * FXP];
+                pair(0, up, dm, a.k[p]);          // rows p and -p
+                pair(1, un, dn, a.k[p]);          // rows 1 + p and 1 - p
+                up = un;
+                dn = dm;
             }
-            const long long U = (A << 10) + (B >> 20);
-            const int uh = (int)(U >> 31), ul = (int)((unsigned)U & 0x7fffffffu);
-            mad(H, uh, fh[ax]);
-            mad(M1, uh, fl[ax]);
-            mad(M2, ul, fh[ax]);
+        } else {
+#pragma unroll
+            for (int p = 1; p <= FXH; ++p) pair(0, ps[p * FXP], ps[-p * FXP], a.k[p]);
         }
-        long long M3 = 1 << 25;
-        mad(M3, c.x, vc.y);
-        mad(M3, c.y, vc.x);
-        const long long Z = H + (M1 >> 30) + (M2 >> 31) + (((long long)c.x * vc.x) << 4) + (M3 >> 26);
-        double r = (double)Z * scale;
-        if (YP) r = fma(beta, ypc, r);
-        if (active) Yo[(long)z * plane + own] = r;
+        end(1);
+#pragma unroll
+        for (int r = 0; r < ROWS; ++r) {
+            const int2 c = q[r][FXH];
+            long long M3 = 1 << 25;
+            mad(M3, c.x, vc[r].y);
+            mad(M3, c.y, vc[r].x);
+            const long long Z = H[r] + (M1[r] >> 30) + (M2[r] >> 31) + (((long long)c.x * vc[r].x) << 4) + (M3 >> 26);
+            const double t = (double)Z * scale;
+            if (act[r]) Yo[zo + own[r]] = YP ? fma(beta, ypc[r], t) : t;
+        }
+        zo = zn;
         __syncthreads();
     }
 }
@@ -314,7 +380,7 @@ int launch_fx_veff(hub_t h, const void* V) {
     return HUB_OK;
 }
 
-template <int NT, int CTAS, int FXPER>
+template <int ROWS, int NT, int CTAS, int PER>
 static int run_fx(hub_t h, const StencilArgs& s) {
     FxArgs a{};
     int rc;
@@ -342,23 +408,39 @@ static int run_fx(hub_t h, const StencilArgs& s) {
     a.beta = s.beta;
     a.shift = s.shift;
     a.coef = s.coef;
-    // tiles of equal width close to 32 (rows are contiguous; the halo costs 12 points a row),
-    // rows so that a CTA has at most NT threads and FXPER points of the halo'd plane each
+    // Tiles of equal width close to 32 (rows are contiguous; the halo costs 12 points a row).  Rows
+    // per tile (even: two per thread) and chunks along z by the instructions of a CTA (25 per
+    // converted point, 540 per thread and plane; a chunk converts 7 planes and 12 points more)
+    // times the CTAs that a slot runs one after another; a wave that is not full counts whole.
     const int ntx = (s.n1 + 31) / 32;
     a.tx = (s.n1 + ntx - 1) / ntx;
-    const int rows = std::min(std::min(NT / a.tx, FXPER * NT / (a.tx + 2 * FXH) - 2 * FXH), 60);   // 60: 200 KB
-    const int nty = (s.n2 + rows - 1) / rows;
-    a.ty = (s.n2 + nty - 1) / nty;
     a.tilesx = ntx;
-    a.tiles = ntx * nty;
-    const int slots = (a.tx + 2 * FXH) * (a.ty + 2 * FXH);
-    const int nt = (std::max(a.tx * a.ty, (slots + FXPER - 1) / FXPER) + 31) / 32 * 32;
-    // chunks along z: about two waves of CTAs, each chunk re-reading 12 planes
-    const long per = (long)a.tiles * s.ncol, want = 4L * CTAS * h->num_sms;
-    int nzc = per < want ? (int)((want + per - 1) / per) : 1;
-    a.zchunk = std::max(std::min(s.n3, 8), (s.n3 + nzc - 1) / nzc);
+    const int rows = std::min(std::min(ROWS * (NT / a.tx), PER * NT / (a.tx + 2 * FXH) - 2 * FXH), 60) / ROWS * ROWS;   // 60: 200 KB
+    const int key = s.ncol * 8 + h->stencil_variant;
+    if (h->fx_plan[0] != key) {
+        double best = 1e300;
+        for (int ty = rows; ty >= ROWS; ty -= ROWS) {
+            if (ty < rows && ty >= s.n2 + ROWS) continue;
+            const int nt = (std::max(a.tx * ty / ROWS, ((a.tx + 2 * FXH) * (ty + 2 * FXH) + PER - 1) / PER) + 31) / 32 * 32;
+            const long tiles = (long)ntx * ((s.n2 + ty - 1) / ty) * s.ncol;
+            for (int nzc = 1; nzc <= s.n3; ++nzc) {
+                const int zc = (s.n3 + nzc - 1) / nzc;
+                const double waves = (double)(tiles * ((s.n3 + zc - 1) / zc)) / (CTAS * h->num_sms);
+                const double cost = nt * (zc * (25.0 * PER + 100.0 + 220.0 * ROWS) + 25.0 * (7 * PER + 12 * ROWS) + 1000.0);
+                const double t = cost * (waves < 1.0 ? 0.5 + 0.5 * waves : waves < 8.0 ? std::ceil(waves) : waves + 0.5);
+                if (t < best) { best = t; h->fx_plan[1] = ty; h->fx_plan[2] = zc; }
+                if (zc <= 4) break;
+            }
+        }
+        h->fx_plan[0] = key;
+    }
+    a.ty = h->fx_plan[1];
+    a.zchunk = h->fx_plan[2];
     a.nzc = (s.n3 + a.zchunk - 1) / a.zchunk;
-    const size_t smem = (size_t)FXS * (a.ty + 2 * FXH) * FXP * sizeof(int2);
+    a.tiles = ntx * ((s.n2 + a.ty - 1) / a.ty);
+    const int slots = (a.tx + 2 * FXH) * (a.ty + 2 * FXH);
+    const int nt = (std::max(a.tx * a.ty / ROWS, (slots + PER - 1) / PER) + 31) / 32 * 32;
+    const size_t smem = (size_t)FXS * ((a.ty + 2 * FXH) * FXP + 2) * sizeof(int2);
     const long grid = (long)a.tiles * a.nzc * s.ncol;
     if (grid > 0x7fffffffL) return fail(h, HUB_EINVAL, "stencil: too many tiles");
     ProfScope ps(h, HUB_K_STENCIL);
@@ -367,19 +449,19 @@ static int run_fx(hub_t h, const StencilArgs& s) {
         kernel<<<(unsigned)grid, nt, smem, h->stream>>>(a);
         return HUB_OK;
     };
-    if ((rc = s.Yprev ? run(k_stencil_fx<true, NT, CTAS, FXPER>) : run(k_stencil_fx<false, NT, CTAS, FXPER>))) return rc;
+    if ((rc = s.Yprev ? run(k_stencil_fx<true, ROWS, NT, CTAS, PER>) : run(k_stencil_fx<false, ROWS, NT, CTAS, PER>))) return rc;
     HUB_CUDA_TRY(h, cudaGetLastError());
     return HUB_OK;
 }
 
-// CTA shapes (hub_set_tuning; 0 is the default).  Three CTAs of 256 threads (80 registers) hide
-// the barrier of one another's planes: 4.5 ms on 88 x 88 x 84 x 348, against 4.8 (two of 384),
-// 5.0 (two of 256 with 96 registers) and 6.4 (one of 512).
+// CTA shapes (hub_set_tuning; 0 is the default), on 88 x 88 x 84 x 348: 4.12, 4.25 and 4.40 ms.
+// Four CTAs of 192 threads hide the barriers of one another's planes; two rows per thread need
+// fewer instructions (382 against ~450 per point) but leave 16 warps per SM.
 int launch_stencil_fx(hub_t h, const StencilArgs& s) {
     switch (h->stencil_variant) {
-        case 1: return run_fx<384, 2, 3>(h, s);
-        case 2: return run_fx<256, 2, 4>(h, s);
-        default: return run_fx<256, 3, 4>(h, s);
+        case 1: return run_fx<1, 256, 3, 4>(h, s);
+        case 2: return run_fx<2, 256, 2, 5>(h, s);
+        default: return run_fx<1, 192, 4, 4>(h, s);
     }
 }
 
