@@ -43,15 +43,12 @@ k_colmax(const R* __restrict__ X, long ld, long n, unsigned* __restrict__ cmax) 
 
 }  // namespace
 
-int launch_colmax(hub_t h, const void* X, int ncol, int ld) {
-    int rc;
-    if ((rc = ensure(h, (void**)&h->d_cmax, &h->cmax_bytes,
-                     std::max(h->cmax_bytes, (size_t)ncol * kColParts * sizeof(unsigned))))) return rc;
+int launch_colmax_at(hub_t h, const void* X, int ncol, int ld, unsigned* cmax) {
     const int cw = h->cplx ? 2 : 1;
     ProfScope ps(h, HUB_K_COPY);
     for (int c0 = 0; c0 < ncol; c0 += 65535) {
         const dim3 grid(kColParts, (unsigned)std::min(65535, ncol - c0));
-        unsigned* out = h->d_cmax + (size_t)c0 * kColParts;
+        unsigned* out = cmax + (size_t)c0 * kColParts;
         if (h->esize == 8)
             k_colmax<double><<<grid, 512, 0, h->stream>>>((const double*)X + (size_t)c0 * ld * cw, (long)ld * cw, h->Nd * cw, out);
         else
@@ -59,6 +56,13 @@ int launch_colmax(hub_t h, const void* X, int ncol, int ld) {
     }
     HUB_CUDA_TRY(h, cudaGetLastError());
     return HUB_OK;
+}
+
+int launch_colmax(hub_t h, const void* X, int ncol, int ld) {
+    int rc;
+    if ((rc = ensure(h, (void**)&h->d_cmax, &h->cmax_bytes,
+                     std::max(h->cmax_bytes, (size_t)ncol * kColParts * sizeof(unsigned))))) return rc;
+    return launch_colmax_at(h, X, ncol, ld, h->d_cmax);
 }
 
 }  // namespace hub

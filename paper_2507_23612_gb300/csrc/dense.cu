@@ -20,9 +20,13 @@ constexpr int NB = 32;   // Cholesky block
 // factor the jb x jb diagonal block at (j0, j0) in place (one CTA, NB x NB in shared memory);
 // the diagonal of a Hermitian matrix is real, so is L's
 template <typename T>
-__global__ void k_potf2(T* A, int lda, int j0, int jb, int* flags) {
+__global__ void k_potf2(T* A, int lda, int j0, int jb, int* flags, double* __restrict__ diag, int n) {
     __shared__ T s[NB][NB + 1];
     const int t = threadIdx.x;
+    // the diagonal as it was: a pivot within the rounding of its own update (8 x 2^-53 of the
+    // diagonal element) cannot be told from zero
+    if (j0 == 0)
+        for (int i = t; i < n; i += blockDim.x) diag[i] = re_of(A[(size_t)i * lda + i]);
     for (int e = t; e < jb * jb; e += blockDim.x) {
         const int i = e / jb, j = e % jb;
         s[i][j] = A[(size_t)(j0 + i) * lda + j0 + j];
@@ -31,7 +35,7 @@ __global__ void k_potf2(T* A, int lda, int j0, int jb, int* flags) {
     for (int k = 0; k < jb; ++k) {
         if (t == 0) {
             const double d = re_of(s[k][k]);
-            if (!(d > 0.0) || !isfinite(d)) {
+            if (!(d > 8.8817841970012523e-16 * diag[j0 + k]) || !isfinite(d)) {
                 flags[FLAG_NOTSPD] = 1;
                 s[k][k] = from_real<T>(1.0);
             } else {
@@ -394,10 +398,10 @@ int gemm_t(hub_t h, bool ta, bool tb, int m, int n, int k, double alpha, const T
 }
 
 template <typename T>
-int cholesky_t(hub_t h, T* A, int n) {
+int cholesky_t(hub_t h, T* A, int n, double* diag) {
     for (int j0 = 0; j0 < n; j0 += NB) {
         const int jb = std::min(NB, n - j0);
-        { ProfScope ps(h, HUB_K_CHOLESKY); k_potf2<T><<<1, 256, 0, h->stream>>>(A, n, j0, jb, h->d_flags); }
+        { ProfScope ps(h, HUB_K_CHOLESKY); k_potf2<T><<<1, 256, 0, h->stream>>>(A, n, j0, jb, h->d_flags, diag, n); }
         HUB_CUDA_TRY(h, cudaGetLastError());
         const int rest = n - j0 - jb;
         if (rest <= 0) continue;
@@ -480,8 +484,8 @@ int dense_gemm(hub_t h, bool ta, bool tb, int m, int n, int k, double alpha, con
     return gemm_t<double>(h, ta, tb, m, n, k, alpha, A, lda, B, ldb, beta, C, ldc);
 }
 
-int dense_cholesky(hub_t h, double* A, int n) {
-    return h->cplx ? cholesky_t<double2>(h, (double2*)A, n) : cholesky_t<double>(h, A, n);
+int dense_cholesky(hub_t h, double* A, int n, double* diag) {
+    return h->cplx ? cholesky_t<double2>(h, (double2*)A, n, diag) : cholesky_t<double>(h, A, n, diag);
 }
 
 int dense_tri_inverse(hub_t h, const double* L, double* Linv, int n) {

@@ -389,6 +389,21 @@ int gram_t(hub_t h, const void* A, int lda, const void* B, int ldb, int m, int n
 
 }  // namespace
 
+// Real blocks as digit products on the tensor cores (gemm_oz.cu; complex blocks stay here).  The
+// digit sums hold 2^25 grid points.  Doubles always: the Gram product is level with the FP64 pipe at
+// 14^3 x 6 (54 us) and ahead from there on (88x88x84 x 348, symmetric: 83.0 -> 3.6 ms; the rotation
+// 140.4 -> 4.0).  Floats: the conversions have to be earned.  The Gram product is ahead from some
+// thousand points on (14^3 x 24: 23 against 29 us; 24^3 x 24: 63 against 33; 88x88x84 x 348: 4.4
+// against 1.9 ms), the rotation only over many columns (with its conversions, 88x88x84 x 96: 0.49
+// against 0.75 ms, x 130: 1.06 against 1.0, x 348: 5.1 against 2.2; 28x30x56 x 130: 0.09 against
+// 0.10, x 200: 0.16 against 0.13).
+static bool gram_digits(hub_t h) {
+    return !h->cplx && h->Nd <= (1L << 25) && (h->esize == 8 || h->Nd >= 8192);
+}
+static bool rotate_digits(hub_t h, int k, int n) {
+    return !h->cplx && h->Nd <= (1L << 25) && (h->esize == 8 || (k > 128 && (double)k * n * h->Nd >= 1.5e9));
+}
+
 int launch_gram(hub_t h, const void* A, int lda, const void* B, int ldb, int m, int n,
                 double alpha, bool sym, double* G) {
     if (m == 0 || n == 0) return HUB_OK;
@@ -396,6 +411,7 @@ int launch_gram(hub_t h, const void* A, int lda, const void* B, int ldb, int m, 
         if (h->esize == 8) return gram_t<double2>(h, A, lda, B, ldb, m, n, alpha, sym, G);
         return gram_t<float2>(h, A, lda, B, ldb, m, n, alpha, sym, G);
     }
+    if (gram_digits(h)) return launch_gram_oz(h, A, lda, B, ldb, m, n, alpha, sym, G);
     if (h->esize == 8) return gram_t<double>(h, A, lda, B, ldb, m, n, alpha, sym, G);
     if (lda % 4 == 0 && ldb % 4 == 0 && (uintptr_t)A % 16 == 0 && (uintptr_t)B % 16 == 0)
         return gram_f32x8(h, (const float*)A, lda, (const float*)B, ldb, m, n, alpha, sym, G);
@@ -404,6 +420,7 @@ int launch_gram(hub_t h, const void* A, int lda, const void* B, int ldb, int m, 
 
 int launch_rotate(hub_t h, const void* X, int ldx, const double* Q, int k, int n, void* Y, int ldy) {
     if (n == 0) return HUB_OK;
+    if (rotate_digits(h, k, n)) return launch_rotate_oz(h, X, ldx, Q, k, n, Y, ldy);
     dim3 grid((unsigned)((h->Nd + BM - 1) / BM), (n + BN - 1) / BN);
     ProfScope ps(h, HUB_K_ROTATE);
     const double2* Qz = (const double2*)Q;

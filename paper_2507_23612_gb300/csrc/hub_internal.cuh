@@ -270,6 +270,7 @@ int stencil_variants(hub_t h);
 // each column (biased exponent on top)
 constexpr int kColParts = 8;
 int launch_colmax(hub_t h, const void* X, int ncol, int ld);
+int launch_colmax_at(hub_t h, const void* X, int ncol, int ld, unsigned* cmax);   // into cmax
 #ifdef __CUDACC__
 __device__ __forceinline__ unsigned column_max(const unsigned* cmax, int col) {
     unsigned m = 0;
@@ -342,6 +343,10 @@ int launch_gram(hub_t h, const void* A, int lda, const void* B, int ldb, int m, 
 // Y[K x n] = X[K x k] Q[k x n]; Q double column-major [k x n] (ldq = k)
 int launch_rotate(hub_t h, const void* X, int ldx, const double* Q, int k, int n, void* Y,
                   int ldy);
+// gemm_oz.cu: the same for real blocks as exact digit products on the tensor cores
+int launch_gram_oz(hub_t h, const void* A, int lda, const void* B, int ldb, int m, int n,
+                   double alpha, bool sym, double* G);
+int launch_rotate_oz(hub_t h, const void* X, int ldx, const double* Q, int k, int n, void* Y, int ldy);
 // mixed-precision variants (tcgen05 path; 16-bit operand type from h->prec)
 // true when the Rayleigh-Ritz block products of this handle run on the tensor cores: a mixed
 // handle (BF16 or FP16 operands), real blocks, and a product form with 1 or 3 terms
@@ -354,7 +359,7 @@ int launch_rotate_bf16(hub_t h, const void* X, int ldx, const double* Q, int k, 
                        void* Y, int ldy);
 
 // dense.cu (double, n x n, row-major)
-int dense_cholesky(hub_t h, double* A, int n);                 // lower L in place
+int dense_cholesky(hub_t h, double* A, int n, double* diag);   // lower L in place; diag: n doubles of workspace
 int dense_tri_inverse(hub_t h, const double* L, double* Linv, int n);
 // C = alpha op(A) op(B) + beta C ; row-major n x n style small matrices
 int dense_gemm(hub_t h, bool ta, bool tb, int m, int n, int k, double alpha, const double* A,

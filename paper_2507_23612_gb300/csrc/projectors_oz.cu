@@ -95,24 +95,6 @@ struct SCfg {
 __device__ __forceinline__ uint32_t desc_lo(const void* p, uint32_t lbo) { return ((saddr(p) & 0x3FFFF) >> 4) | ((lbo >> 4) << 16); }
 constexpr uint32_t kDescHi = 8u | (1u << 14);
 
-// eight accumulator columns of S levels (STEP columns apart)
-__device__ __forceinline__ void tmem_ld8(uint32_t addr, uint32_t* r) {
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
-                 : "r"(addr));
-}
-__device__ __forceinline__ void keep8(uint32_t* r) {
-    asm volatile("" : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]));
-}
-template <int S, int STEP>
-__device__ __forceinline__ void tmem_levels(uint32_t addr, uint32_t (&v)[S * 8]) {
-#pragma unroll
-    for (int l = 0; l < S; ++l) tmem_ld8(addr + (uint32_t)(l * STEP), v + 8 * l);
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-    for (int l = 0; l < S; ++l) keep8(v + 8 * l);      // no use of the values moves above the wait
-}
-
 struct OzGather {
     const void* X;
     const int4* grp;          // brick, slots, 16-byte offset, first slot

@@ -147,4 +147,22 @@ __device__ __forceinline__ void mma_tf32(uint32_t tmem_d, uint64_t ad, uint64_t 
                  ::"r"(tmem_d), "l"(ad), "l"(bd), "r"(idesc), "r"(acc) : "memory");
 }
 
+// eight accumulator columns of S levels (STEP columns apart)
+__device__ __forceinline__ void tmem_ld8(uint32_t addr, uint32_t* r) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+                 : "r"(addr));
+}
+__device__ __forceinline__ void keep8(uint32_t* r) {
+    asm volatile("" : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]));
+}
+template <int S, int STEP>
+__device__ __forceinline__ void tmem_levels(uint32_t addr, uint32_t (&v)[S * 8]) {
+#pragma unroll
+    for (int l = 0; l < S; ++l) tmem_ld8(addr + (uint32_t)(l * STEP), v + 8 * l);
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+    for (int l = 0; l < S; ++l) keep8(v + 8 * l);      // no use of the values moves above the wait
+}
+
 }  // namespace hub
