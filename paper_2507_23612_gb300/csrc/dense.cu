@@ -152,216 +152,349 @@ __global__ void k_symmetrize(T* A, int n) {
 }
 
 // ---------------------------------------------------------------------------- Jacobi
+constexpr int kJacThreads = 256;
 constexpr long kSpinLimit = 1L << 22;
 
-// bounded grid barrier for a cooperative launch; returns false once any wait ran out
-__device__ bool grid_barrier(unsigned int* bar, unsigned int nblocks, int* flags) {
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        volatile unsigned int* vgen = bar + 1;
-        const unsigned int gen = *vgen;
-        __threadfence();
-        const unsigned int arrived = atomicAdd(bar, 1u);
-        if (arrived == nblocks - 1) {
-            atomicExch(bar, 0u);
-            __threadfence();
-            atomicAdd(bar + 1, 1u);
-        } else {
-            long it = 0;
-            while (*vgen == gen) {
-                if (++it > kSpinLimit) { atomicExch(flags + FLAG_TIMEOUT, 1); break; }
-                __nanosleep(64);
-            }
+__device__ __forceinline__ unsigned ld_acquire(const unsigned* p) {
+    unsigned v;
+    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+// one thread waits until the counter has reached target; bounded, false once a wait ran out
+__device__ __forceinline__ bool wait_count(const unsigned* bar, unsigned target, int* flags) {
+    for (long it = 0; (int)(ld_acquire(bar) - target) < 0; ++it) {
+        if (it > kSpinLimit || ((it & 1023) == 1023 && *((volatile int*)(flags + FLAG_TIMEOUT)) != 0)) {
+            atomicExch(flags + FLAG_TIMEOUT, 1);
+            return false;
         }
-        __threadfence();
     }
-    __syncthreads();
-    return *((volatile int*)(flags + FLAG_TIMEOUT)) == 0;
+    return true;
 }
 
 __device__ __forceinline__ void pair_of(int step, int k, int N, int& p, int& q) {
-    // round-robin ("circle") schedule: player N-1 fixed, players 0..N-2 rotate
+    // round-robin ("circle") schedule: player N-1 fixed, players 0..N-2 rotate; step < N - 1
     if (k == 0) { p = N - 1; q = step; }
     else {
-        p = (step + k) % (N - 1);
-        q = (step - k + (N - 1)) % (N - 1);
+        p = step + k;
+        if (p >= N - 1) p -= N - 1;
+        q = step - k;
+        if (q < 0) q += N - 1;
     }
     if (p > q) { const int t = p; p = q; q = t; }
 }
 
-// Parallel cyclic Jacobi with the round-robin pair schedule.  Each step applies n/2
-// disjoint rotations.  Every CTA computes all rotation angles of a step itself from the
-// current matrix (identical inputs and operations, so all copies agree), and the step
-// writes the rotated matrix into the other of two buffers: nothing the step reads is
-// written during it, so one grid barrier per step suffices.  V is rotated in place (only
-// the step's own rotations touch a given V element).
+// Elements of other CTAs: from L2
+__device__ __forceinline__ double ld_far(const double* p) { return __ldcg(p); }
+__device__ __forceinline__ double2 ld_far(const double2* p) { return __ldcg(p); }
+
+__device__ __forceinline__ int exponent_of(double v) { return (__double2hiint(v) >> 20) & 0x7ff; }
+
+// c and sg = s exp(i arg a_pq) of the rotation that zeroes a_pq: s = t c, t the smaller root of
+// t^2 + 2 theta t = 1 with theta = (a_qq - a_pp) / (2 |a_pq|).  t (and the phase) in float, c and s
+// from it in double: the rotation is unitary to rounding, and the pair's coupling falls by 2^-22
+// instead of to rounding, which the next sweep makes up for.  (The divisions and square roots of a
+// double angle are some 50 dependent instructions of the FP64 pipe, of about 64 clocks each.)
+template <typename T>
+__device__ __forceinline__ void jacobi_angle(double app, double aqq, T apq, double& c, T& sg) {
+    constexpr bool CPLX = sizeof(T) == 16;
+    const double d = aqq - app;
+    // all by the power of two that brings the largest of them near 1
+    int e = exponent_of(d);
+    if constexpr (CPLX) e = max(e, max(exponent_of(apq.x), exponent_of(apq.y)) + 1);
+    else e = max(e, exponent_of(apq) + 1);
+    const double sc = __hiloint2double(max(1, min(2046, 2046 - e)) << 20, 0);
+    const float df = (float)(d * sc);
+    float mf, ph = 1.0f, ph2 = 0.0f;
+    if constexpr (CPLX) {
+        const float x = (float)(apq.x * sc), y = (float)(apq.y * sc);
+        const float big = fmaxf(fabsf(x), fabsf(y)), up = big < 1e-15f ? 1e18f : 1.0f;      // keeps the square in range
+        const float xs = x * up, ys = y * up, r = rsqrtf(fmaf(xs, xs, ys * ys));
+        ph = xs * r;
+        ph2 = ys * r;
+        mf = 2.0f * (fabsf(x) * fabsf(ph) + fabsf(y) * fabsf(ph2));
+    } else {
+        mf = 2.0f * fabsf((float)(apq * sc));
+    }
+    const float tf = copysignf(__fdividef(mf, fabsf(df) + sqrtf(fmaf(df, df, mf * mf))), df);
+    const double t = (double)tf, y = (double)rsqrtf(fmaf(tf, tf, 1.0f));   // 2^-22
+    const double u = fma(t, t, 1.0);
+    const double h = fma(-(u * y), y, 1.0);
+    c = fma(y * h, fma(0.375, h, 0.5), y);                                 // y (1 + h/2 + 3 h^2/8): 2^-66
+    const double s = t * c;
+    if constexpr (CPLX) {
+        const double px = (double)ph, py = (double)ph2;
+        const double k = 1.0 - fma(px, px, py * py);
+        const double w = s * fma(k, fma(0.375, k, 0.5), 1.0);
+        sg = make_double2(px * w, py * w);
+    } else {
+        sg = apq >= 0.0 ? s : -s;
+    }
+}
+__device__ __forceinline__ double largest_part(double v) { return fabs(v); }
+__device__ __forceinline__ double largest_part(double2 v) { return fmax(fabs(v.x), fabs(v.y)); }
+
+template <typename T>
+struct JacobiArgs {
+    T* A[2];                    // matrices (result: the diagonal)
+    T* Ab[2];                   // second buffers
+    T* V[2];                    // eigenvectors as columns
+    double* ang[2];             // [2][RS * H]: the angles of the last step and this one
+    unsigned long long* red[2]; // 4 slots each
+    unsigned* bar;              // one counter per matrix, zeroed
+    int* flags;
+    int* sweeps;
+    int nmat, n, N, max_sweeps, g, ng, v_shared;
+    double tol;
+};
+
+// Parallel cyclic Jacobi with the round-robin pair schedule.  Each step applies n/2 disjoint
+// rotations and writes the rotated matrix into the other of two buffers: nothing the step reads is
+// written during it, so one grid-wide barrier per step suffices.  3500 steps of the 348-orbital
+// block follow one another, so the length of a step is what counts: barrier, loads from L2, angles,
+// update, stores.
+//   * A CTA owns the blocks of one pair of groups of g pairs (upper triangle, the adjoint written
+//     too), so that it needs 2 g angles and not all n/2, one per thread, from elements loaded
+//     together with those of its blocks.  All copies of an angle have the same inputs and operations.
+//   * The rotation of V is one step late and overlaps the barrier: a CTA keeps some rows of V in
+//     shared memory (in global memory if they don't fit) and applies the angles of the step before,
+//     which the CTAs of the diagonal groups leave in memory, between its arrival and the release.
+//     One warp only waits.
+// 348 orbitals: 29.9 -> 13.5 ms (58: 3.3 -> 1.7 ms; complex 348: 53.2 -> 22.6 ms) against every CTA
+// computing every angle in double and V between the loads and the barrier.  Of a step's 8300 clocks
+// 2600 go into loads and angles, 1700 into the update, 1000 into the stores and 1700 into the wait.
 // The rotation of a pair (p, q) is J = [[c, sg], [-conj(sg), c]] with c real and
 // sg = s exp(i arg a_pq): the phase makes the pivot real, then the real Jacobi angle of
 // (a_pp, |a_pq|, a_qq) zeroes it; for real matrices sg = +-s and J is the plain rotation.
-// With nmat = 2 the grid solves two independent matrices of the same size at once: each
-// half of the CTAs owns one matrix, its buffers, its barrier counters and its reduction
-// slots, and only the error flags are shared (a timeout in one half ends both).
+// With nmat = 2 the grid solves two independent matrices of the same size at once: each half of
+// the CTAs owns one matrix, its buffers, its barrier counter and its reduction slots, and only the
+// error flags are shared (a timeout in one half ends both).
 template <typename T>
-__global__ void k_jacobi(T* A0, T* Ab0, T* V0, T* A1, T* Ab1, T* V1, int nmat,
-                         int n, int N, int max_sweeps, double tol, unsigned int* bar, int* flags,
-                         unsigned long long* red0, unsigned long long* red1, int* sweeps_out) {
+__global__ void __launch_bounds__(kJacThreads, 1) k_jacobi(const __grid_constant__ JacobiArgs<T> a) {
     constexpr bool CPLX = sizeof(T) == 2 * sizeof(double);
     constexpr int RS = CPLX ? 3 : 2;              // doubles per pair: c, sg (re[, im])
-    extern __shared__ double rot[];               // [RS * N / 2]
-    auto sg_of = [&](int k) -> T {
-        if constexpr (CPLX) return make_double2(rot[RS * k + 1], rot[RS * k + 2]);
-        else return rot[RS * k + 1];
+    constexpr int VT = kJacThreads - 32;          // threads that rotate V
+    extern __shared__ double2 jac_smem[];
+    __shared__ int ok_sh;
+    const int n = a.n, N = a.N, H = N / 2, g = a.g, tid = threadIdx.x;
+    const int grp = (a.nmat == 2 && blockIdx.x >= gridDim.x / 2) ? 1 : 0;
+    const int nb = a.nmat == 2 ? gridDim.x / 2 : gridDim.x, cta = blockIdx.x - grp * nb;
+    double* rot = (double*)jac_smem;              // angles of this CTA's groups
+    double* late = rot + (2 * RS * g + 1) / 2 * 2;                 // all angles of the step before
+    T* vrows = a.v_shared ? (T*)(late + (RS * H + 1) / 2 * 2) : nullptr;
+    T* V = a.V[grp];
+    double* ang = a.ang[grp];
+    unsigned* bar = a.bar + grp;
+    unsigned arrived = 0;
+    // groups of this CTA: row I of the upper triangle of ng x ng
+    int I = 0, J = cta;
+    while (J >= a.ng - I) { J -= a.ng - I; ++I; }
+    J += I;
+    const int rows = cta < n ? (n - cta + nb - 1) / nb : 0;        // rows cta, cta + nb, ... of V
+    auto vrow = [&](int r) -> T* { return vrows ? vrows + (size_t)r * n : V + (size_t)(cta + r * nb) * n; };
+    for (int r = 0; r < rows; ++r)
+        for (int j = tid; j < n; j += kJacThreads) vrow(r)[j] = from_real<T>(j == cta + r * nb ? 1.0 : 0.0);
+    auto get = [](const double* w, double& c, T& sg) {
+        c = w[0];
+        if constexpr (CPLX) sg = make_double2(w[1], w[2]);
+        else sg = w[1];
     };
-    const int grp = (nmat == 2 && blockIdx.x >= gridDim.x / 2) ? 1 : 0;
-    const unsigned int nb = nmat == 2 ? gridDim.x / 2 : gridDim.x;
-    T* A = grp ? A1 : A0;
-    T* Ab = grp ? Ab1 : Ab0;
-    T* V = grp ? V1 : V0;
-    unsigned long long* red = grp ? red1 : red0;
-    bar += 2 * grp;
-    sweeps_out += grp;
-    const long tid = (long)(blockIdx.x - grp * nb) * blockDim.x + threadIdx.x;
-    const long nthr = (long)nb * blockDim.x;
-    const int H = N / 2;
-    T* cur = A;
-    T* nxt = Ab;
+    auto rotate_v = [&](int step, int t0, int nt) {
+        int r = t0 / H, k = t0 - r * H;
+        const int dr = nt / H, dk = nt - dr * H;
+        while (r < rows) {
+            double c;
+            T sg;
+            get(late + RS * k, c, sg);
+            int p, q;
+            pair_of(step, k, N, p, q);
+            if (q < n && largest_part(sg) != 0.0) {
+                T* v = vrow(r);
+                const T vp = v[p], vq = v[q];
+                v[p] = csub(mulr(c, vp), cmul(cconj(sg), vq));
+                v[q] = cfma(sg, vp, mulr(c, vq));
+            }
+            r += dr;
+            k += dk;
+            if (k >= H) { k -= H; ++r; }
+        }
+    };
+    // arrival (after every thread's stores) and wait of a grid-wide barrier
+    auto arrive = [&] {
+        __threadfence();
+        atomicAdd(bar, 1u);
+    };
+    auto barrier = [&]() -> bool {
+        __syncthreads();
+        arrived += nb;
+        if (tid == 0) {
+            arrive();
+            ok_sh = wait_count(bar, arrived, a.flags);
+        }
+        __syncthreads();
+        return ok_sh != 0;
+    };
+    T* cur = a.A[grp];
+    T* nxt = a.Ab[grp];
+    unsigned long long* red = a.red[grp];
     const T zero = zero_of(T());
-    int sweep = 0;
-    for (; sweep < max_sweeps; ++sweep) {
+    const int e0 = tid < g * g ? tid / g * 65536 + tid % g : g * 65536;       // this thread's first block of the CTA's
+    int sweep = 0, before = -1, par = 0;          // the step before (none), half of ang to write
+    for (; sweep < a.max_sweeps; ++sweep) {
         // convergence: max |a_ij| (i != j) against max |a_ii|
         unsigned long long* acc = red + 2 * (sweep & 1);
         double off = 0.0, dia = 0.0;
-        for (long e = tid; e < (long)n * n; e += nthr) {
-            const int i = (int)(e / n), j = (int)(e % n);
-            const double v = cabs_of(cur[e]);
-            if (i == j) dia = fmax(dia, v); else off = fmax(off, v);
-        }
+        for (int i = cta; i < n; i += nb)
+            for (int j = tid; j < n; j += kJacThreads) {
+                const double v = cabs_of(ld_far(cur + (size_t)i * n + j));
+                if (i == j) dia = fmax(dia, v); else off = fmax(off, v);
+            }
         for (int o = 16; o > 0; o >>= 1) {
             off = fmax(off, __shfl_down_sync(0xffffffffu, off, o));
             dia = fmax(dia, __shfl_down_sync(0xffffffffu, dia, o));
         }
-        if ((threadIdx.x & 31) == 0) {
+        if ((tid & 31) == 0) {
             atomicMax(acc, (unsigned long long)__double_as_longlong(off));
             atomicMax(acc + 1, (unsigned long long)__double_as_longlong(dia));
         }
-        if (!grid_barrier(bar, nb, flags)) return;
-        const double goff = __longlong_as_double((long long)*((volatile unsigned long long*)acc));
-        const double gdia = __longlong_as_double((long long)*((volatile unsigned long long*)(acc + 1)));
-        if (tid == 0) {                          // the group's first thread
+        if (!barrier()) return;
+        const double goff = __longlong_as_double((long long)__ldcg(acc));
+        const double gdia = __longlong_as_double((long long)__ldcg(acc + 1));
+        if (cta == 0 && tid == 0) {
             unsigned long long* other = red + 2 * ((sweep + 1) & 1);
             other[0] = 0ull;
             other[1] = 0ull;
         }
-        if (goff <= tol * fmax(gdia, 1e-300)) break;
-        if (sweep == max_sweeps - 1) {
-            if (tid == 0) flags[FLAG_NOCONV] = 1;
+        if (goff <= a.tol * fmax(gdia, 1e-300)) break;
+        if (sweep == a.max_sweeps - 1) {
+            if (cta == 0 && tid == 0) a.flags[FLAG_NOCONV] = 1;
             break;
         }
         // pairs whose coupling is below this are left alone (threshold Jacobi)
-        const double skip = 1e-3 * tol * fmax(gdia, 1e-300);
+        const double skip = (CPLX ? 0.7e-3 : 1e-3) * a.tol * fmax(gdia, 1e-300);
         for (int step = 0; step < N - 1; ++step) {
-            // phase 1 (per CTA): the n/2 disjoint rotations of this step
-            for (int k = threadIdx.x; k < H; k += blockDim.x) {
+            // the angles of the step before come in while this step's are computed
+            if (before >= 0) {
+                const double2* src = (const double2*)(ang + (size_t)(par ^ 1) * ((RS * H + 1) / 2 * 2));
+                for (int i = tid; i < (RS * H + 1) / 2; i += kJacThreads)
+                    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared((double2*)late + i)),
+                                 "l"(src + i) : "memory");
+                asm volatile("cp.async.commit_group;" ::: "memory");
+            }
+            int p1, q1, p2, q2;
+            T b00, b01, b10, b11;
+            auto ld = [&](int i, int j) { return (i < n && j < n) ? ld_far(cur + (size_t)i * n + j) : zero; };
+            auto load_block = [&](int i, int j) -> bool {
+                const int P = I * g + i, Q = J * g + j;
+                if (P >= Q || i >= g || Q >= H) return false;
+                pair_of(step, P, N, p1, q1);
+                pair_of(step, Q, N, p2, q2);
+                b00 = ld(p1, p2); b01 = ld(p1, q2); b10 = ld(q1, p2); b11 = ld(q1, q2);
+                return true;
+            };
+            bool have = load_block(e0 / 65536, e0 % 65536);
+            // angles: one thread per pair; in a diagonal group also the pair's own block, which
+            // gets the corrections of the diagonal and what is left of the coupling
+            for (int i = tid; i < (I == J ? g : 2 * g); i += kJacThreads) {
+                const int k = i < g ? I * g + i : J * g + i - g;
+                if (k >= H) continue;
                 int p, q;
                 pair_of(step, k, N, p, q);
-                double c = 1.0, sr = 0.0, si = 0.0;
+                double c = 1.0;
+                T sg = zero;
                 if (q < n) {
-                    const T apq = cur[(size_t)p * n + q];
-                    const double mag = cabs_of(apq);
-                    if (mag > skip) {
-                        const double app = re_of(cur[(size_t)p * n + p]), aqq = re_of(cur[(size_t)q * n + q]);
-                        const double theta = (aqq - app) / (2.0 * mag);
-                        double t;
-                        if (fabs(theta) > 1e150) t = 0.5 / theta;
-                        else t = (theta >= 0.0 ? 1.0 : -1.0) / (fabs(theta) + sqrt(theta * theta + 1.0));
-                        c = 1.0 / sqrt(t * t + 1.0);
-                        const double s = t * c;
-                        if constexpr (CPLX) { sr = s * (apq.x / mag); si = s * (apq.y / mag); }
-                        else sr = apq >= 0.0 ? s : -s;
-                    }
+                    const T apq = ld(p, q);
+                    const double app = re_of(ld(p, p)), aqq = re_of(ld(q, q));
+                    if (largest_part(apq) > skip) jacobi_angle(app, aqq, apq, c, sg);
                 }
-                rot[RS * k] = c;
-                rot[RS * k + 1] = sr;
-                if constexpr (CPLX) rot[RS * k + 2] = si;
+                double* w = rot + RS * i;
+                w[0] = c;
+                if constexpr (CPLX) { w[1] = sg.x; w[2] = sg.y; }
+                else w[1] = sg;
+                if (I == J) {
+                    double* out = ang + (size_t)par * ((RS * H + 1) / 2 * 2) + (size_t)RS * k;
+                    for (int d = 0; d < RS; ++d) __stcg(out + d, w[d]);
+                }
             }
             __syncthreads();
-            // phase 2: every 2x2 block (P, Q) of the next matrix <- J_P^H B J_Q (blocks of two
-            // identity rotations are copied), and V <- V J in place
-            // the matrix stays Hermitian: only the blocks P <= Q are computed, and each
-            // writes its adjoint too
-            const long nblk = (long)H * (H + 1) / 2;
-            for (long e = tid; e < nblk + (long)n * H; e += nthr) {
-                if (e < nblk) {
-                    // row P of the upper triangle holds H - P blocks; S(P) = P (2H - P + 1) / 2
-                    // (estimate in float arithmetic: the FP64 pipe is the scarce one; the two
-                    // loops below correct the estimate)
-                    const float h2 = 2.0f * H + 1.0f;
-                    int P = (int)((h2 - sqrtf(fmaxf(h2 * h2 - 8.0f * (float)e, 0.0f))) * 0.5f);
-                    P = max(0, min(P, H - 1));
-                    auto S = [&](long r) { return r * (2L * H - r + 1) / 2; };
-                    while (P > 0 && S(P) > e) --P;
-                    while (P < H - 1 && S(P + 1) <= e) ++P;
-                    const int Q = P + (int)(e - S(P));
-                    const T g1 = sg_of(P), g2 = sg_of(Q);
-                    const double c1 = rot[RS * P], c2 = rot[RS * Q];
-                    const bool r1 = cabs_of(g1) != 0.0, r2 = cabs_of(g2) != 0.0;
-                    int p1, q1, p2, q2;
-                    pair_of(step, P, N, p1, q1);
-                    pair_of(step, Q, N, p2, q2);
-                    auto ld = [&](int i, int j) { return (i < n && j < n) ? cur[(size_t)i * n + j] : zero; };
-                    const T b00 = ld(p1, p2), b01 = ld(p1, q2), b10 = ld(q1, p2), b11 = ld(q1, q2);
-                    T n00 = b00, n01 = b01, n10 = b10, n11 = b11;
-                    if (r1 || r2) {
-                        const T r00 = csub(mulr(c1, b00), cmul(g1, b10));
-                        const T r01 = csub(mulr(c1, b01), cmul(g1, b11));
-                        const T r10 = cfma(cconj(g1), b00, mulr(c1, b10));
-                        const T r11 = cfma(cconj(g1), b01, mulr(c1, b11));
-                        n00 = csub(mulr(c2, r00), cmul(cconj(g2), r01));
-                        n01 = cfma(g2, r00, mulr(c2, r01));
-                        n10 = csub(mulr(c2, r10), cmul(cconj(g2), r11));
-                        n11 = cfma(g2, r10, mulr(c2, r11));
-                        if (P == Q && q1 < n) {
-                            // the rotated pair: exact zero off-diagonal, diagonal by the t-update
-                            // (t |a_pq| = Re(conj(sg) a_pq) / c)
-                            const double ta = re_of(cmul(cconj(g1), b01)) / c1;
-                            n00 = from_real<T>(re_of(b00) - ta);
-                            n11 = from_real<T>(re_of(b11) + ta);
-                            n01 = zero;
-                            n10 = zero;
-                        }
-                    }
-                    if (p1 < n && p2 < n) { nxt[(size_t)p1 * n + p2] = n00; nxt[(size_t)p2 * n + p1] = cconj(n00); }
-                    if (p1 < n && q2 < n) { nxt[(size_t)p1 * n + q2] = n01; nxt[(size_t)q2 * n + p1] = cconj(n01); }
-                    if (q1 < n && p2 < n) { nxt[(size_t)q1 * n + p2] = n10; nxt[(size_t)p2 * n + q1] = cconj(n10); }
-                    if (q1 < n && q2 < n) { nxt[(size_t)q1 * n + q2] = n11; nxt[(size_t)q2 * n + q1] = cconj(n11); }
-                } else {
-                    const long f = e - nblk;
-                    const int r = (int)(f / H), P = (int)(f % H);
-                    const T g = sg_of(P);
-                    if (cabs_of(g) == 0.0) continue;
-                    int p, q;
-                    pair_of(step, P, N, p, q);
-                    if (q >= n) continue;
-                    const double c = rot[RS * P];
-                    const T vp = V[(size_t)r * n + p], vq = V[(size_t)r * n + q];
-                    V[(size_t)r * n + p] = csub(mulr(c, vp), cmul(cconj(g), vq));
-                    V[(size_t)r * n + q] = cfma(g, vp, mulr(c, vq));
-                }
+            // every 2x2 block (P, Q) of the next matrix <- J_P^H B J_Q; the matrix stays Hermitian:
+            // only the blocks P <= Q are computed, and each writes its adjoint too
+            auto st = [&](int i, int j, T v) {
+                if (i >= n || j >= n) return;
+                nxt[(size_t)i * n + j] = v;
+                nxt[(size_t)j * n + i] = cconj(v);
+            };
+            for (int e = tid; e < g * g; e += kJacThreads) {
+                int i = e0 / 65536, j = e0 % 65536;
+                if (e != tid) { i = e / g; j = e - i * g; have = load_block(i, j); }
+                if (!have) continue;
+                double c1, c2;
+                T g1, g2;
+                get(rot + RS * i, c1, g1);
+                get(rot + RS * (j + (I == J ? 0 : g)), c2, g2);
+                const T r00 = csub(mulr(c1, b00), cmul(g1, b10));
+                const T r01 = csub(mulr(c1, b01), cmul(g1, b11));
+                const T r10 = cfma(cconj(g1), b00, mulr(c1, b10));
+                const T r11 = cfma(cconj(g1), b01, mulr(c1, b11));
+                st(p1, p2, csub(mulr(c2, r00), cmul(cconj(g2), r01)));
+                st(p1, q2, cfma(g2, r00, mulr(c2, r01)));
+                st(q1, p2, csub(mulr(c2, r10), cmul(cconj(g2), r11)));
+                st(q1, q2, cfma(g2, r10, mulr(c2, r11)));
             }
-            if (!grid_barrier(bar, nb, flags)) return;
+            if (I == J)
+                for (int i = kJacThreads - 1 - tid; i < g; i += kJacThreads) {     // the last warps first
+                    const int k = I * g + i;
+                    if (k >= H) continue;
+                    int p, q;
+                    pair_of(step, k, N, p, q);
+                    double c;
+                    T sg;
+                    get(rot + RS * i, c, sg);
+                    const T apq = ld(p, q);
+                    const double app = re_of(ld(p, p));
+                    if (q >= n) {
+                        nxt[(size_t)p * n + p] = from_real<T>(app);
+                        continue;
+                    }
+                    const double aqq = re_of(ld(q, q));
+                    const double d = aqq - app, s2 = re_of(cmul(cconj(sg), sg)), w = re_of(cmul(cconj(sg), apq));
+                    const double u = fma(s2, d, -2.0 * c * w);
+                    nxt[(size_t)p * n + p] = from_real<T>(app + u);
+                    nxt[(size_t)q * n + q] = from_real<T>(aqq - u);
+                    st(p, q, csub(csub(mulr(c * c, apq), cmul(cmul(sg, sg), cconj(apq))), mulr(c * d, sg)));
+                }
+            asm volatile("cp.async.wait_all;" ::: "memory");
+            __syncthreads();
+            arrived += nb;
+            if (tid >= VT) {
+                if (tid == VT) {
+                    arrive();
+                    ok_sh = wait_count(bar, arrived, a.flags);
+                }
+            } else if (before >= 0) {
+                rotate_v(before, tid, VT);
+            }
+            __syncthreads();
+            if (!ok_sh) return;
+            before = step;
+            par ^= 1;
             T* t = cur; cur = nxt; nxt = t;
         }
     }
-    if (cur != A)
-        for (long e = tid; e < (long)n * n; e += nthr) A[e] = cur[e];
-    if (tid == 0) *sweeps_out = sweep;
-}
-
-template <typename T>
-__global__ void k_eye(T* V, int n) {
-    const long t = (long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= (long)n * n) return;
-    V[t] = from_real<T>(((t / n) == (t % n)) ? 1.0 : 0.0);
+    // the last step's rotations of V
+    if (before >= 0) {
+        const double* src = ang + (size_t)(par ^ 1) * ((RS * H + 1) / 2 * 2);
+        for (int i = tid; i < RS * H; i += kJacThreads) late[i] = __ldcg(src + i);
+        __syncthreads();
+        rotate_v(before, tid, kJacThreads);
+        __syncthreads();
+    }
+    if (vrows)
+        for (int r = 0; r < rows; ++r)
+            for (int j = tid; j < n; j += kJacThreads) V[(size_t)(cta + r * nb) * n + j] = vrows[(size_t)r * n + j];
+    if (cur != a.A[grp])
+        for (int i = cta; i < n; i += nb)
+            for (int j = tid; j < n; j += kJacThreads) a.A[grp][(size_t)i * n + j] = ld_far(cur + (size_t)i * n + j);
+    if (cta == 0 && tid == 0) a.sweeps[grp] = sweep;
 }
 
 // ascending order: rank by (value, index); V columns follow
@@ -417,58 +550,57 @@ int cholesky_t(hub_t h, T* A, int n, double* diag) {
 
 template <typename T>
 int jacobi_t(hub_t h, int nmat, T* const* A, T* const* V, double* const* eig, int n) {
-    const int N = n + (n & 1);
+    const int N = n + (n & 1), H = N / 2;
     const size_t nn = (size_t)n * n;
-    constexpr int CW = sizeof(T) / sizeof(double);
-    const size_t per = 2 * CW * nn + 8;                         // doubles of workspace per matrix
+    constexpr int CW = sizeof(T) / sizeof(double), RS = CW + 1;
+    const size_t nang = (size_t)(RS * H + 1) / 2 * 2;
+    const size_t per = 2 * CW * nn + 2 * nang + 4;         // doubles of workspace per matrix
     int rc;
     if ((rc = ensure(h, &h->d_work2, &h->work2_bytes, std::max(nmat * per * sizeof(double), h->work2_bytes))))
         return rc;
-    T* Vt[2];
-    T* Ab[2];
-    unsigned long long* red[2];
+    JacobiArgs<T> a{};
     for (int g = 0; g < 2; ++g) {
         const int m = g < nmat ? g : 0;
-        double* base = (double*)h->d_work2 + m * per;
-        Vt[g] = (T*)base;
-        Ab[g] = Vt[g] + nn;                                     // second matrix buffer
-        red[g] = (unsigned long long*)(base + 2 * CW * nn);     // 4 slots
+        a.A[g] = A[m];
+        a.ang[g] = (double*)h->d_work2 + m * per;               // 16-byte aligned
+        a.red[g] = (unsigned long long*)(a.ang[g] + 2 * nang);
+        a.V[g] = (T*)(a.ang[g] + 2 * nang + 4);
+        a.Ab[g] = a.V[g] + nn;                                  // second matrix buffer
+        if (g < nmat) HUB_CUDA_TRY(h, cudaMemsetAsync(a.red[g], 0, 4 * sizeof(unsigned long long), h->stream));
     }
-    int* sweeps = h->d_flags + 6;                               // slots 6 and 7
-    for (int g = 0; g < nmat; ++g) {
-        {
-            ProfScope ps(h, HUB_K_EIG_MISC);
-            k_eye<T><<<(unsigned)((nn + 255) / 256), 256, 0, h->stream>>>(Vt[g], n);
-        }
-        HUB_CUDA_TRY(h, cudaGetLastError());
-        HUB_CUDA_TRY(h, cudaMemsetAsync(red[g], 0, 4 * sizeof(unsigned long long), h->stream));
-    }
+    a.sweeps = h->d_flags + 6;                                  // slots 6 and 7
+    a.bar = h->d_bar;
+    a.flags = h->d_flags;
+    a.nmat = nmat;
+    a.n = n;
+    a.N = N;
+    a.max_sweeps = 60;
+    a.tol = 1e-13;
     HUB_CUDA_TRY(h, cudaMemsetAsync(h->d_bar, 0, 4 * sizeof(unsigned int), h->stream));
-    HUB_CUDA_TRY(h, cudaMemsetAsync(sweeps, 0, 2 * sizeof(int), h->stream));
-    int per_sm = 0;
-    const size_t rot_bytes = (size_t)(N / 2) * (CW + 1) * sizeof(double);
-    if (rot_bytes > 48 * 1024) return fail(h, HUB_EINVAL, "subspace too large for the Jacobi solver");
-    HUB_CUDA_TRY(h, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_jacobi<T>, 256, rot_bytes));
-    int blocks = std::max(1, std::min(per_sm, 1)) * h->num_sms / nmat;   // per matrix
-    const long work = (long)(N / 2) * (N / 2 + 1) / 2 + (long)n * (N / 2);
-    blocks = (int)std::min<long>(blocks, std::max<long>(1, (work + 255) / 256));
-    blocks = std::max(1, blocks) * nmat;
-    int max_sweeps = 60;
-    double tol = 1e-13;
-    unsigned int* bar = h->d_bar;
-    int* flags = h->d_flags;
-    T* A0 = A[0];
-    T* A1 = nmat > 1 ? A[1] : A[0];
-    void* args[] = {&A0, &Ab[0], &Vt[0], &A1, &Ab[1], &Vt[1], &nmat, &n, (void*)&N, &max_sweeps, &tol, &bar,
-                    &flags, &red[0], &red[1], &sweeps};
+    HUB_CUDA_TRY(h, cudaMemsetAsync(a.sweeps, 0, 2 * sizeof(int), h->stream));
+    if ((size_t)H * RS * sizeof(double) > 48 * 1024) return fail(h, HUB_EINVAL, "subspace too large for the Jacobi solver");
+    // groups of g pairs, one CTA per pair of groups: as many groups as the SMs of one matrix hold,
+    // of at least 6 pairs (fewer CTAs wait for one another: 58 orbitals take 15)
+    const int room = std::max(1, h->num_sms / nmat);
+    int ng = 1;
+    while ((ng + 1) * (ng + 2) / 2 <= room && (H + ng) / (ng + 1) >= 6) ++ng;
+    a.g = (H + ng - 1) / ng;
+    a.ng = (H + a.g - 1) / a.g;
+    const int blocks = a.ng * (a.ng + 1) / 2;
+    const size_t base = ((size_t)(2 * RS * a.g + 1) / 2 * 2 + nang) * sizeof(double);
+    const size_t vbytes = (size_t)((n + blocks - 1) / blocks) * n * sizeof(T);
+    a.v_shared = base + vbytes <= 200 * 1024;
+    const size_t smem = base + (a.v_shared ? vbytes : 0);
+    HUB_CUDA_TRY(h, cudaFuncSetAttribute(k_jacobi<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    void* args[] = {&a};
     {
         ProfScope ps(h, HUB_K_JACOBI);
-        HUB_CUDA_TRY(h, cudaLaunchCooperativeKernel((void*)k_jacobi<T>, dim3(blocks), dim3(256), args, rot_bytes,
+        HUB_CUDA_TRY(h, cudaLaunchCooperativeKernel((void*)k_jacobi<T>, dim3(blocks * nmat), dim3(kJacThreads), args, smem,
                                                     h->stream));
     }
     for (int g = 0; g < nmat; ++g) {
         ProfScope ps(h, HUB_K_EIG_MISC);
-        k_sort_eig<T><<<(n + 127) / 128, 128, 0, h->stream>>>(A[g], Vt[g], n, eig[g], V[g]);
+        k_sort_eig<T><<<(n + 127) / 128, 128, 0, h->stream>>>(A[g], a.V[g], n, eig[g], V[g]);
     }
     HUB_CUDA_TRY(h, cudaGetLastError());
     return HUB_OK;
@@ -509,7 +641,7 @@ int dense_symmetrize(hub_t h, double* A, int n) {
 }
 
 // A (n x n Hermitian, destroyed) -> eig ascending (device [n]) and V (device n x n row-major,
-// column j = eigenvector j).  Uses 2 n x n matrices + 8 doubles of scratch per matrix.
+// column j = eigenvector j).  Uses 2 n x n matrices and two steps' angles of scratch per matrix.
 int dense_jacobi_eigh_multi(hub_t h, int nmat, double* const* A, double* const* V, double* const* eig, int n) {
     if (n == 0) return HUB_OK;
     if (nmat < 1 || nmat > 2) return fail(h, HUB_EINVAL, "one or two matrices per Jacobi launch");
