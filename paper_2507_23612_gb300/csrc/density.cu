@@ -19,6 +19,7 @@
 
 #include "hub_internal.cuh"
 #include "cplx.cuh"
+#include "grid_sum.cuh"
 
 namespace hub {
 
@@ -46,10 +47,8 @@ __device__ __forceinline__ void block_partial(double v, double* part) {
     }
 }
 
-// out[slot] = scale * sum(part[0..n)); one CTA, fixed order.  With copy_from >= 0 also
-// out[copy_to] = out[copy_from] first (the CG's rr <- rr_new hand-over).
-__global__ void k_reduce(const double* __restrict__ part, int n, double scale, double* __restrict__ out,
-                         int slot, int copy_from, int copy_to) {
+// out[slot] = scale * sum(part[0..n)); one CTA, fixed order
+__global__ void k_reduce(const double* __restrict__ part, int n, double scale, double* __restrict__ out, int slot) {
     __shared__ double red[kThreads];
     double s = 0.0;
     for (int i = threadIdx.x; i < n; i += kThreads) s += part[i];
@@ -60,7 +59,6 @@ __global__ void k_reduce(const double* __restrict__ part, int n, double scale, d
         __syncthreads();
     }
     if (threadIdx.x == 0) {
-        if (copy_from >= 0) out[copy_to] = out[copy_from];
         out[slot] = scale * red[0];
     }
 }
@@ -90,12 +88,11 @@ struct LapArgs {
     int n0, n1, n2, n3;
 };
 
-// y = shift x - Lap_h x (periodic); with part != nullptr also block partials of x . y
+// y = -Lap_h x (periodic)
 __global__ void __launch_bounds__(kThreads)
-k_neg_lap(const double* __restrict__ x, double* __restrict__ y, LapArgs a, double shift, double* __restrict__ part) {
+k_neg_lap(const double* __restrict__ x, double* __restrict__ y, LapArgs a) {
     const long Nd = (long)a.n1 * a.n2 * a.n3;
     const long g = (long)blockIdx.x * kThreads + threadIdx.x;
-    double dot = 0.0;
     if (g < Nd) {
         const int i = (int)(g % a.n1);
         const long t = g / a.n1;
@@ -119,59 +116,108 @@ k_neg_lap(const double* __restrict__ x, double* __restrict__ y, LapArgs a, doubl
             lap = fma(a.w[1][p - 1], col[(long)jp * sy] + col[(long)jm * sy], lap);
             lap = fma(a.w[2][p - 1], pil[(long)kp * sz] + pil[(long)km * sz], lap);
         }
-        const double out = shift * x0 - lap;
-        y[g] = out;
-        dot = x0 * out;
+        y[g] = -lap;
     }
-    if (part) block_partial(dot, part);
 }
 
 // ---------------------------------------------------------------------------- CG steps
-// scalar slots: 0 rr, 1 pq, 2 rr_new, 3 bb, 4 scratch
-enum { S_RR = 0, S_PQ = 1, S_RRN = 2, S_BB = 3, S_TMP = 4 };
+// scalar slots: 0 rr, 1 pq, 2 rr_new, 3 bb, 4 scratch, 5 CTAs done (a counter), 6 alpha = rr / pq,
+// 7 beta = rr_new / rr (divided once, by the thread that has the sum: a division per thread was a
+// third of the steps' time)
+enum { S_RR = 0, S_PQ = 1, S_RRN = 2, S_BB = 3, S_TMP = 4, S_CNT = 5, S_ALPHA = 6, S_BETA = 7 };
 
-// r = b - q, p = r; partials of r . r and of b . b (part, part + nblk)
+// elements of a CTA of the vector steps: 4 per thread, loaded before any is stored
+constexpr int kCgPer = 4;
+
+// largest leading word of |v| over the threads, for the scale of the fixed-point stencil
+__device__ __forceinline__ unsigned lead(double v) { return (unsigned)__double2hiint(v) & 0x7fffffffu; }
+__device__ __forceinline__ void raise_max(unsigned m, unsigned* cmax) {
+    m = __reduce_max_sync(0xffffffffu, m);
+    if ((threadIdx.x & 31) == 0) atomicMax(cmax + blockIdx.x % kColParts, m);
+}
+
+__global__ void __launch_bounds__(kThreads)
+k_vec_max(const double* __restrict__ x, long n, unsigned* __restrict__ cmax) {
+    const long g = (long)blockIdx.x * kThreads + threadIdx.x;
+    raise_max(g < n ? lead(x[g]) : 0, cmax);
+}
+
+// r = b - q, p = r; partials of r . r and of b . b (part, part + nblk); cmax: of p
 __global__ void __launch_bounds__(kThreads)
 k_cg_start(const double* __restrict__ b, const double* __restrict__ q, double* __restrict__ r, double* __restrict__ p,
-           long n, double* __restrict__ part, int nblk) {
+           long n, double* __restrict__ part, int nblk, unsigned* __restrict__ cmax) {
     const long g = (long)blockIdx.x * kThreads + threadIdx.x;
     double rr = 0.0, bb = 0.0;
+    unsigned m = 0;
     if (g < n) {
         const double v = b[g] - q[g];
         r[g] = v;
         p[g] = v;
         rr = v * v;
         bb = b[g] * b[g];
+        m = lead(v);
     }
+    raise_max(m, cmax);
     block_partial(rr, part);
     __syncthreads();
     block_partial(bb, part + nblk);
 }
 
-// alpha = rr / pq; x += alpha p; r -= alpha q; partials of r . r
+// x += alpha p; r -= alpha q; rr_new = r . r, beta; clears the maxima for k_cg_direction
 __global__ void __launch_bounds__(kThreads)
 k_cg_update(double* __restrict__ x, double* __restrict__ r, const double* __restrict__ p, const double* __restrict__ q,
-            long n, const double* __restrict__ s, double* __restrict__ part) {
-    const double pq = s[S_PQ];
-    const double alpha = pq > 0.0 ? s[S_RR] / pq : 0.0;
-    const long g = (long)blockIdx.x * kThreads + threadIdx.x;
-    double rr = 0.0;
-    if (g < n) {
-        x[g] = fma(alpha, p[g], x[g]);
-        const double v = fma(-alpha, q[g], r[g]);
-        r[g] = v;
-        rr = v * v;
+            long n, double* __restrict__ s, double* __restrict__ part, unsigned* __restrict__ cmax) {
+    const long g0 = (long)blockIdx.x * (kCgPer * kThreads) + threadIdx.x;
+    double xv[kCgPer], rv[kCgPer], pv[kCgPer], qv[kCgPer];
+#pragma unroll
+    for (int i = 0; i < kCgPer; ++i) {
+        const long g = g0 + i * kThreads;
+        const bool in = g < n;
+        xv[i] = in ? x[g] : 0.0;
+        rv[i] = in ? r[g] : 0.0;
+        pv[i] = in ? p[g] : 0.0;
+        qv[i] = in ? q[g] : 0.0;
     }
-    block_partial(rr, part);
+    const double alpha = s[S_ALPHA];
+    double rr = 0.0, total;
+#pragma unroll
+    for (int i = 0; i < kCgPer; ++i) {
+        const long g = g0 + i * kThreads;
+        if (g >= n) continue;
+        x[g] = fma(alpha, pv[i], xv[i]);
+        const double v = fma(-alpha, qv[i], rv[i]);
+        r[g] = v;
+        rr = fma(v, v, rr);
+    }
+    if (grid_sum(rr, part, (unsigned*)(s + S_CNT), total)) {
+        s[S_RRN] = total;
+        s[S_BETA] = s[S_RR] > 0.0 ? total / s[S_RR] : 0.0;
+        for (int i = 0; i < kColParts; ++i) cmax[i] = 0;
+    }
 }
 
-// beta = rr_new / rr; p = r + beta p
+// p = r + beta p; cmax: of p
 __global__ void __launch_bounds__(kThreads)
-k_cg_direction(const double* __restrict__ r, double* __restrict__ p, long n, const double* __restrict__ s) {
-    const double rr = s[S_RR];
-    const double beta = rr > 0.0 ? s[S_RRN] / rr : 0.0;
-    const long g = (long)blockIdx.x * kThreads + threadIdx.x;
-    if (g < n) p[g] = fma(beta, p[g], r[g]);
+k_cg_direction(const double* __restrict__ r, double* __restrict__ p, long n, const double* __restrict__ s,
+               unsigned* __restrict__ cmax) {
+    const long g0 = (long)blockIdx.x * (kCgPer * kThreads) + threadIdx.x;
+    double rv[kCgPer], pv[kCgPer];
+#pragma unroll
+    for (int i = 0; i < kCgPer; ++i) {
+        const long g = g0 + i * kThreads;
+        rv[i] = g < n ? r[g] : 0.0;
+        pv[i] = g < n ? p[g] : 0.0;
+    }
+    const double beta = s[S_BETA];
+    unsigned m = 0;
+#pragma unroll
+    for (int i = 0; i < kCgPer; ++i) {
+        const long g = g0 + i * kThreads;
+        const double v = fma(beta, pv[i], rv[i]);
+        if (g < n) p[g] = v;
+        m = max(m, lead(v));
+    }
+    raise_max(m, cmax);
 }
 
 // y = c0 * (x - s[slot] / n) (c0 = 4 pi: the Poisson right-hand side; slot holds sum x)
@@ -243,16 +289,18 @@ unsigned blocks_for(long n) { return (unsigned)((n + kThreads - 1) / kThreads); 
 }  // namespace
 
 // ---------------------------------------------------------------------------- host side
-// workspace: [nblk*2 partials][8 scalars][r][p][q][b] doubles
+// workspace: [partials: 2 nblk, one per 32 points of a row][8 scalars][r][p][q][b] doubles, and a
+// zero potential in the form of the fixed-point stencil
 static int dens_ws(hub_t h, double** part, double** s, double** r, double** p, double** q, double** b) {
     const long n = h->Nd;
     const long nblk = blocks_for(n);
-    const size_t need = (size_t)(2 * nblk + 8 + 4 * n) * sizeof(double);
+    const size_t npart = std::max<size_t>(2 * nblk, (size_t)((h->n1 + 31) / 32) * h->n2 * h->n3);
+    const size_t need = (npart + 8 + 5 * n) * sizeof(double) + fx_veff_bytes(n);
     int rc = ensure(h, &h->d_dens, &h->dens_bytes, need);
     if (rc) return rc;
     double* base = (double*)h->d_dens;
     *part = base;
-    *s = base + 2 * nblk;
+    *s = base + npart;
     *r = *s + 8;
     *p = *r + n;
     *q = *p + n;
@@ -277,13 +325,92 @@ static LapArgs lap_args(hub_t h) {
 }
 
 // s[slot] = scale * sum of the partials of the last partial kernel
-static int reduce_to(hub_t h, const double* part, int nblk, double scale, double* s, int slot,
-                     int copy_from = -1, int copy_to = -1) {
-    k_reduce<<<1, kThreads, 0, h->stream>>>(part, nblk, scale, s, slot, copy_from, copy_to);
+static int reduce_to(hub_t h, const double* part, int nblk, double scale, double* s, int slot) {
+    k_reduce<<<1, kThreads, 0, h->stream>>>(part, nblk, scale, s, slot);
     h->launches++;
     HUB_CUDA_TRY(h, cudaGetLastError());
     return HUB_OK;
 }
+
+// The CG on one right-hand side; zero: a potential of zeros with its fixed-point form
+struct CgState {
+    double shift;
+    double *part, *s, *r, *p, *q, *x;
+    const double* zero;
+};
+
+// q = (-Lap_h + shift) v as twice the kinetic stencil in fixed point (stencil_fx.cu) with the scale in
+// h->d_cmax, and v . q.  The plain form is bound by the FP64 pipe (37 operations per point; 75 us on
+// 88x88x84 against 31, whose few CTAs convert most points several times).
+static int cg_apply(hub_t h, const CgState& c, const double* v) {
+    const LapArgs la = lap_args(h);
+    StencilArgs a{};
+    a.Y = v;
+    a.Yout = c.q;
+    a.V = c.zero;
+    a.n1 = h->n1; a.n2 = h->n2; a.n3 = h->n3;
+    a.ld = (int)h->Nd;
+    a.ncol = 1;
+    a.n0 = h->n0;
+    for (int ax = 0; ax < 3; ++ax)
+        for (int p = 0; p < h->n0; ++p) a.wbase[ax][p] = -0.5 * la.w[ax][p];
+    a.alpha = 2.0;
+    a.shift = -0.5 * c.shift;
+    a.cmax_ready = true;
+    return launch_stencil_fx_dot(h, a, StencilDot{c.s + S_RR, c.part, (unsigned*)(c.s + S_CNT)});
+}
+
+// k iterations: stencil with p . q, x and r with r . r, p with its largest magnitude
+static int cg_steps(hub_t h, const CgState& c, int k) {
+    const long n = h->Nd;
+    const unsigned nb = (unsigned)((n + kCgPer * kThreads - 1) / (kCgPer * kThreads));
+    int rc;
+    for (int i = 0; i < k; ++i) {
+        if ((rc = cg_apply(h, c, c.p))) return rc;
+        k_cg_update<<<nb, kThreads, 0, h->stream>>>(c.x, c.r, c.p, c.q, n, c.s, c.part, h->d_cmax);
+        k_cg_direction<<<nb, kThreads, 0, h->stream>>>(c.r, c.p, n, c.s, h->d_cmax);
+        h->launches += 2;
+    }
+    HUB_CUDA_TRY(h, cudaGetLastError());
+    return HUB_OK;
+}
+
+// kCgCheck iterations as a graph of this solve (its buffers are this solve's): below some 10^5 points
+// the host's launches are what an iteration waits for (28x30x56: 30.0 us per iteration with five plain
+// launches, 23.3 so; 88x88x84, where the device is the slower: 110 and 49 us)
+struct CgGraph {
+    cudaStream_t side = nullptr;
+    cudaGraphExec_t exec = nullptr;
+    long long launches = 0;
+    ~CgGraph() {
+        if (exec) cudaGraphExecDestroy(exec);
+        if (side) cudaStreamDestroy(side);
+    }
+    int capture(hub_t h, const CgState& c) {
+        HUB_CUDA_TRY(h, cudaStreamCreateWithFlags(&side, cudaStreamNonBlocking));
+        HUB_CUDA_TRY(h, cudaStreamBeginCapture(side, cudaStreamCaptureModeThreadLocal));
+        const cudaStream_t saved = h->stream;
+        const long long l0 = h->launches;
+        h->stream = side;
+        h->capturing = 1;
+        const int rc = cg_steps(h, c, kCgCheck);
+        h->capturing = 0;
+        h->stream = saved;
+        launches = h->launches - l0;
+        h->launches = l0;
+        cudaGraph_t graph = nullptr;
+        const cudaError_t e = cudaStreamEndCapture(side, &graph);
+        if (rc || e != cudaSuccess) {
+            if (graph) cudaGraphDestroy(graph);
+            if (rc) return rc;
+            HUB_CUDA_TRY(h, e);
+        }
+        const cudaError_t ei = cudaGraphInstantiate(&exec, graph, 0);
+        cudaGraphDestroy(graph);
+        HUB_CUDA_TRY(h, ei);
+        return HUB_OK;
+    }
+};
 
 // (-Lap_h + shift) x = b by CG from the x given; |r| <= tol |b| or max_iter iterations.
 // b lives in the workspace slot `bw` (untouched).  Returns HUB_ENOCONV past max_iter.
@@ -293,10 +420,20 @@ static int cg_solve(hub_t h, double shift, const double* bw, double* x, double t
     if (rc) return rc;
     const long n = h->Nd;
     const unsigned nb = blocks_for(n);
-    const LapArgs la = lap_args(h);
-    ProfScope ps(h, HUB_K_DENSITY);                    // counts the first launch
-    k_neg_lap<<<nb, kThreads, 0, h->stream>>>(x, q, la, shift, nullptr);
-    k_cg_start<<<nb, kThreads, 0, h->stream>>>(bw, q, r, p, n, part, (int)nb);
+    double* zero = b + n;
+    if ((rc = ensure(h, (void**)&h->d_cmax, &h->cmax_bytes, std::max(h->cmax_bytes, kColParts * sizeof(unsigned))))) return rc;
+    HUB_CUDA_TRY(h, cudaMemsetAsync(s, 0, 8 * sizeof(double), h->stream));
+    HUB_CUDA_TRY(h, cudaMemsetAsync(zero, 0, n * sizeof(double), h->stream));
+    HUB_CUDA_TRY(h, cudaMemsetAsync(h->d_cmax, 0, kColParts * sizeof(unsigned), h->stream));
+    if ((rc = launch_fx_veff(h, zero))) return rc;
+    {
+        ProfScope ps(h, HUB_K_DENSITY);
+        k_vec_max<<<nb, kThreads, 0, h->stream>>>(x, n, h->d_cmax);
+    }
+    const CgState c{shift, part, s, r, p, q, x, zero};
+    if ((rc = cg_apply(h, c, x))) return rc;
+    HUB_CUDA_TRY(h, cudaMemsetAsync(h->d_cmax, 0, kColParts * sizeof(unsigned), h->stream));
+    k_cg_start<<<nb, kThreads, 0, h->stream>>>(bw, q, r, p, n, part, (int)nb, h->d_cmax);
     h->launches += 1;
     HUB_CUDA_TRY(h, cudaGetLastError());
     if ((rc = reduce_to(h, part, nb, 1.0, s, S_RRN))) return rc;
@@ -312,19 +449,16 @@ static int cg_solve(hub_t h, double shift, const double* bw, double* x, double t
         return HUB_OK;
     }
     double rr = chk[S_RRN];
+    CgGraph graph;
     while (rr > tol * tol * bb && it < max_iter) {
         const int chunk = std::min(kCgCheck, max_iter - it);
-        for (int c = 0; c < chunk; ++c) {
-            k_neg_lap<<<nb, kThreads, 0, h->stream>>>(p, q, la, shift, part);
-            h->launches++;
-            if ((rc = reduce_to(h, part, nb, 1.0, s, S_PQ, S_RRN, S_RR))) return rc;
-            k_cg_update<<<nb, kThreads, 0, h->stream>>>(x, r, p, q, n, s, part);
-            h->launches++;
-            if ((rc = reduce_to(h, part, nb, 1.0, s, S_RRN))) return rc;
-            k_cg_direction<<<nb, kThreads, 0, h->stream>>>(r, p, n, s);
-            h->launches++;
+        if (chunk == kCgCheck && it > 0) {
+            if (!graph.exec && (rc = graph.capture(h, c))) return rc;
+            HUB_CUDA_TRY(h, cudaGraphLaunch(graph.exec, h->stream));
+            h->launches += graph.launches;
+        } else if ((rc = cg_steps(h, c, chunk))) {
+            return rc;
         }
-        HUB_CUDA_TRY(h, cudaGetLastError());
         it += chunk;
         HUB_CUDA_TRY(h, cudaMemcpyAsync(&rr, s + S_RRN, sizeof(double), cudaMemcpyDeviceToHost, h->stream));
         HUB_CUDA_TRY(h, cudaStreamSynchronize(h->stream));
@@ -504,7 +638,7 @@ int hub_kerker(hub_t h, const double* r_dev, double* z_dev, double kappa, double
     const unsigned nb = blocks_for(h->Nd);
     {
         ProfScope ps(h, HUB_K_DENSITY);
-        k_neg_lap<<<nb, kThreads, 0, h->stream>>>(r_dev, b, lap_args(h), 0.0, nullptr);   // b = -Lap r
+        k_neg_lap<<<nb, kThreads, 0, h->stream>>>(r_dev, b, lap_args(h));   // b = -Lap r
         HUB_CUDA_TRY(h, cudaGetLastError());
     }
     HUB_CUDA_TRY(h, cudaMemsetAsync(z_dev, 0, h->Nd * sizeof(double), h->stream));

@@ -282,6 +282,15 @@ __device__ __forceinline__ unsigned column_max(const unsigned* cmax, int col) {
 // stencil_fx.cu: the real FP64 stencil in fixed point.  A potential of Nd doubles is followed
 // by its fixed-point form (fx_veff_bytes bytes), written by launch_fx_veff
 int launch_stencil_fx(hub_t h, const StencilArgs& a);
+// ... of one column without Yprev, on a handle of any type, with d_cmax set: dot[0] = dot[2], dot[1] = sum
+// of Y * Yout, dot[6] = dot[0] / dot[1] (0 unless dot[1] > 0); part: one double per CTA (at most one per
+// 32 points of a row), counter: zero
+struct StencilDot {
+    double* dot;
+    double* part;
+    unsigned* counter;
+};
+int launch_stencil_fx_dot(hub_t h, const StencilArgs& a, const StencilDot& d);
 size_t fx_veff_bytes(int64_t Nd);
 int launch_fx_veff(hub_t h, const void* V);
 inline size_t veff_bytes(const hub_ctx* h) {

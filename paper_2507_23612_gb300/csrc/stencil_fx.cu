@@ -32,6 +32,7 @@
 #include <cmath>
 
 #include "hub_internal.cuh"
+#include "grid_sum.cuh"
 
 namespace hub {
 
@@ -58,6 +59,9 @@ struct FxArgs {
     double alpha, beta, shift;
     const double* coef;           // device {alpha, beta, shift} or nullptr
     double w[3][FXH], cen;        // FP64 weights (alpha = 1) of the slow form
+    double* dot;                  // StencilDot
+    double* part;
+    unsigned* counter;
 };
 
 __device__ __forceinline__ int wrap(int i, int n) {      // i is at most a few n away
@@ -78,11 +82,13 @@ __device__ __forceinline__ int2 to_limbs(double v, int e20) {
     return (int)hi < 0 ? make_int2(-(int)xh, -(int)xl) : make_int2((int)xh, (int)xl);
 }
 
-// the plain FP64 form of one tile and chunk, straight from global memory
-__device__ __noinline__ void fx_slow(const FxArgs& a, const double* __restrict__ Y, const double* Yp, double* Yo, int gx0,
+// the plain FP64 form of one tile and chunk, straight from global memory; returns this thread's sum
+// of Y * Yout
+__device__ __noinline__ double fx_slow(const FxArgs& a, const double* __restrict__ Y, const double* Yp, double* Yo, int gx0,
                                      int gy0, int z0, int z1, double alpha, double beta, double shift) {
     const long plane = (long)a.n1 * a.n2;
     const int per = a.tx * a.ty;
+    double dot = 0.0;
     for (int i = threadIdx.x; i < per * (z1 - z0); i += blockDim.x) {
         const int z = z0 + i / per, x = gx0 + i % per % a.tx, y = gy0 + i % per / a.tx;
         if (x >= a.n1 || y >= a.n2) continue;
@@ -96,16 +102,31 @@ __device__ __noinline__ void fx_slow(const FxArgs& a, const double* __restrict__
         }
         acc *= alpha;
         Yo[g] = Yp ? fma(beta, Yp[g], acc) : acc;
+        dot = fma(Y[g], acc, dot);
     }
+    return dot;
 }
 
 __device__ __forceinline__ void mad(long long& acc, int s, int w) { acc += (long long)s * w; }
 
+// the product for a conjugate-gradient step: dot[1] = sum, dot[0] = dot[2], dot[6] = dot[0] / dot[1] or 0
+__device__ __forceinline__ void finish_dot(const FxArgs& a, double v) {
+    double total;
+    if (grid_sum(v, a.part, a.counter, total)) {
+        const double rr = a.dot[2];
+        a.dot[0] = rr;
+        a.dot[1] = total;
+        a.dot[6] = total > 0.0 ? rr / total : 0.0;
+    }
+}
+
 // ROWS = 2: two rows per thread; the 14 rows that the y-sums of both need are loaded once, the
 // halo is 12 rows for twice the tile's, and the loop's own instructions serve two points.
-template <bool YP, int ROWS, int NTMAX, int CTAS, int PER>
+// MODE: 0 plain, 1 with Yprev, 2 with the sum of Y * Yout (one column).
+template <int MODE, int ROWS, int NTMAX, int CTAS, int PER>
 __global__ void __launch_bounds__(NTMAX, CTAS)
 k_stencil_fx(const __grid_constant__ FxArgs a) {
+    constexpr bool YP = MODE == 1, DOT = MODE == 2;
     extern __shared__ __align__(16) int2 ring[];
     const int tid = threadIdx.x, nt = blockDim.x;
     const int tile = (int)(blockIdx.x % a.tiles);
@@ -124,7 +145,8 @@ k_stencil_fx(const __grid_constant__ FxArgs a) {
     const int sf = a.vinfo[2];
     const bool fits = fabs(shift) < scalbn(1.0, 83 - sf);       // NaN: false
     if (emax < kFxEmin || emax > kFxEmax || !fits || a.vinfo[1]) {    // the same for the whole CTA
-        fx_slow(a, Y, Yp, Yo, gx0, gy0, z0, z1, alpha, beta, shift);
+        const double sum = fx_slow(a, Y, Yp, Yo, gx0, gy0, z0, z1, alpha, beta, shift);
+        if constexpr (DOT) finish_dot(a, sum);
         return;
     }
     const double scale = scalbn(alpha, 81 - sf + emax - 1081);
@@ -202,8 +224,9 @@ k_stencil_fx(const __grid_constant__ FxArgs a) {
 #pragma unroll
     for (int r = 0; r < ROWS; ++r) {
         vq[r] = a.Vq[zo + own[r]];
-        yp[r] = YP ? Yp[zo + own[r]] : 0.0;
+        yp[r] = YP ? Yp[zo + own[r]] : DOT ? Y[zo + own[r]] : 0.0;
     }
+    double dot = 0.0;
     __syncthreads();
 #pragma unroll
     for (int j = 0; j < FXH; ++j)
@@ -235,6 +258,7 @@ k_stencil_fx(const __grid_constant__ FxArgs a) {
             if (j + 1 < z1 - z0) {
                 vq[r] = a.Vq[zn + own[r]];
                 if (YP) yp[r] = Yp[zn + own[r]];
+                if (DOT) yp[r] = Y[zn + own[r]];
             }
         }
         long long ch[ROWS], cl[ROWS], H[ROWS], M1[ROWS], M2[ROWS], A[ROWS], B[ROWS];
@@ -302,10 +326,12 @@ k_stencil_fx(const __grid_constant__ FxArgs a) {
             const long long Z = H[r] + (M1[r] >> 30) + (M2[r] >> 31) + (((long long)c.x * vc[r].x) << 4) + (M3 >> 26);
             const double t = (double)Z * scale;
             if (act[r]) Yo[zo + own[r]] = YP ? fma(beta, ypc[r], t) : t;
+            if (DOT && act[r]) dot = fma(ypc[r], t, dot);
         }
         zo = zn;
         __syncthreads();
     }
+    if constexpr (DOT) finish_dot(a, dot);
 }
 
 __global__ void k_fx_vmax(const double* __restrict__ V, int* __restrict__ info, long n) {
@@ -381,7 +407,7 @@ int launch_fx_veff(hub_t h, const void* V) {
 }
 
 template <int ROWS, int NT, int CTAS, int PER>
-static int run_fx(hub_t h, const StencilArgs& s) {
+static int run_fx(hub_t h, const StencilArgs& s, int variant, const StencilDot* dot = nullptr) {
     FxArgs a{};
     int rc;
     if (!s.cmax_ready && (rc = launch_colmax(h, s.Y, s.ncol, s.ld))) return rc;
@@ -416,7 +442,7 @@ static int run_fx(hub_t h, const StencilArgs& s) {
     a.tx = (s.n1 + ntx - 1) / ntx;
     a.tilesx = ntx;
     const int rows = std::min(std::min(ROWS * (NT / a.tx), PER * NT / (a.tx + 2 * FXH) - 2 * FXH), 60) / ROWS * ROWS;   // 60: 200 KB
-    const int key = s.ncol * 8 + h->stencil_variant;
+    const int key = s.ncol * 8 + variant;
     if (h->fx_plan[0] != key) {
         double best = 1e300;
         for (int ty = rows; ty >= ROWS; ty -= ROWS) {
@@ -449,7 +475,17 @@ static int run_fx(hub_t h, const StencilArgs& s) {
         kernel<<<(unsigned)grid, nt, smem, h->stream>>>(a);
         return HUB_OK;
     };
-    if ((rc = s.Yprev ? run(k_stencil_fx<true, ROWS, NT, CTAS, PER>) : run(k_stencil_fx<false, ROWS, NT, CTAS, PER>))) return rc;
+    if constexpr (ROWS == 1 && CTAS == 4) {
+        if (dot) {
+            a.dot = dot->dot;
+            a.part = dot->part;
+            a.counter = dot->counter;
+            if ((rc = run(k_stencil_fx<2, ROWS, NT, CTAS, PER>))) return rc;
+            HUB_CUDA_TRY(h, cudaGetLastError());
+            return HUB_OK;
+        }
+    }
+    if ((rc = s.Yprev ? run(k_stencil_fx<1, ROWS, NT, CTAS, PER>) : run(k_stencil_fx<0, ROWS, NT, CTAS, PER>))) return rc;
     HUB_CUDA_TRY(h, cudaGetLastError());
     return HUB_OK;
 }
@@ -459,10 +495,12 @@ static int run_fx(hub_t h, const StencilArgs& s) {
 // fewer instructions (382 against ~450 per point) but leave 16 warps per SM.
 int launch_stencil_fx(hub_t h, const StencilArgs& s) {
     switch (h->stencil_variant) {
-        case 1: return run_fx<1, 256, 3, 4>(h, s);
-        case 2: return run_fx<2, 256, 2, 5>(h, s);
-        default: return run_fx<1, 192, 4, 4>(h, s);
+        case 1: return run_fx<1, 256, 3, 4>(h, s, 1);
+        case 2: return run_fx<2, 256, 2, 5>(h, s, 2);
+        default: return run_fx<1, 192, 4, 4>(h, s, 0);
     }
 }
+
+int launch_stencil_fx_dot(hub_t h, const StencilArgs& s, const StencilDot& d) { return run_fx<1, 192, 4, 4>(h, s, 0, &d); }
 
 }  // namespace hub
