@@ -403,6 +403,13 @@ static bool gram_digits(hub_t h) {
 static bool rotate_digits(hub_t h, int k, int n) {
     return !h->cplx && h->Nd <= (1L << 25) && (h->esize == 8 || (k > 128 && (double)k * n * h->Nd >= 1.5e9));
 }
+// The digits take up to 2 GB of workspace, claimed before the first launch: on a full device the
+// product is left to the CUDA cores, which need little.
+static bool no_memory(int rc) {
+    if (rc != HUB_ENOMEM) return false;
+    cudaGetLastError();               // the failed allocation's, which later launches would report
+    return true;
+}
 
 int launch_gram(hub_t h, const void* A, int lda, const void* B, int ldb, int m, int n,
                 double alpha, bool sym, double* G) {
@@ -411,7 +418,10 @@ int launch_gram(hub_t h, const void* A, int lda, const void* B, int ldb, int m, 
         if (h->esize == 8) return gram_t<double2>(h, A, lda, B, ldb, m, n, alpha, sym, G);
         return gram_t<float2>(h, A, lda, B, ldb, m, n, alpha, sym, G);
     }
-    if (gram_digits(h)) return launch_gram_oz(h, A, lda, B, ldb, m, n, alpha, sym, G);
+    if (gram_digits(h)) {
+        const int rc = launch_gram_oz(h, A, lda, B, ldb, m, n, alpha, sym, G);
+        if (!no_memory(rc)) return rc;
+    }
     if (h->esize == 8) return gram_t<double>(h, A, lda, B, ldb, m, n, alpha, sym, G);
     if (lda % 4 == 0 && ldb % 4 == 0 && (uintptr_t)A % 16 == 0 && (uintptr_t)B % 16 == 0)
         return gram_f32x8(h, (const float*)A, lda, (const float*)B, ldb, m, n, alpha, sym, G);
@@ -420,7 +430,10 @@ int launch_gram(hub_t h, const void* A, int lda, const void* B, int ldb, int m, 
 
 int launch_rotate(hub_t h, const void* X, int ldx, const double* Q, int k, int n, void* Y, int ldy) {
     if (n == 0) return HUB_OK;
-    if (rotate_digits(h, k, n)) return launch_rotate_oz(h, X, ldx, Q, k, n, Y, ldy);
+    if (rotate_digits(h, k, n)) {
+        const int rc = launch_rotate_oz(h, X, ldx, Q, k, n, Y, ldy);
+        if (!no_memory(rc)) return rc;
+    }
     dim3 grid((unsigned)((h->Nd + BM - 1) / BM), (n + BN - 1) / BN);
     ProfScope ps(h, HUB_K_ROTATE);
     const double2* Qz = (const double2*)Q;

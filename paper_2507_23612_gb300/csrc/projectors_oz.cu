@@ -960,14 +960,19 @@ int build_oz(hub_t h, Table& t, const std::vector<std::vector<int>>& site_pts) {
         boff += (size_t)SC::PASSES * (K / 16) * SC::AU;
         if (K > OZ_MAXK || goff >= (1ull << 31) || boff >= (1ull << 31) || prow * CW >= (1L << 31)) return HUB_OK;
     }
+    // on a device without room for both layouts the point-major form does all products
+    if (cudaMalloc((void**)&t.d_ozg_val, goff * 16) != cudaSuccess || cudaMalloc((void**)&t.d_ozb_val, boff * 16) != cudaSuccess) {
+        cudaGetLastError();
+        cudaFree(t.d_ozg_val);
+        t.d_ozg_val = nullptr;
+        return HUB_OK;
+    }
     int rc;
     int *d_row_pair = nullptr, *d_gfn = nullptr, *d_bfn = nullptr;
     int4* d_pairs = nullptr;
     if ((rc = put(h, &t.d_ozg, grp)) || (rc = put(h, &t.d_ozg_row, gslot)) || (rc = put(h, &t.d_ozb, brk)) ||
         (rc = put(h, &t.d_ozb_row, bslot)) || (rc = put(h, &t.d_oz_roff, roff)) || (rc = put(h, &t.d_oz_rent, rent))) return rc;
     HUB_CUDA_TRY(h, cudaMalloc((void**)&t.d_oz_exp, std::max(t.nproj, 1) * sizeof(int)));
-    HUB_CUDA_TRY(h, cudaMalloc((void**)&t.d_ozg_val, goff * 16));
-    HUB_CUDA_TRY(h, cudaMalloc((void**)&t.d_ozb_val, boff * 16));
     HUB_CUDA_TRY(h, cudaMemsetAsync(t.d_ozg_val, 0, goff * 16, h->stream));
     HUB_CUDA_TRY(h, cudaMemsetAsync(t.d_ozb_val, 0, boff * 16, h->stream));
     if (!(rc = put(h, &d_row_pair, row_pair)) && !(rc = put(h, &d_pairs, pairs)) && !(rc = put(h, &d_gfn, gfn)) &&
