@@ -15,8 +15,8 @@
 // lo*hi) with FP32 accumulation in TMEM, about 22 significant bits (the float path's own
 // accuracy) and no rounding bias.  The two small correction
 // products accumulate apart from hi*hi (the tensor core aligns the addends of a sum to the
-// largest, so corrections added to the large accumulator lose their low bits) and the two
-// accumulators are added when the result is read out.
+// largest, so corrections added to the large accumulator lose their low bits), hi*hi in three
+// (GT_ACCS), and the accumulators are added when the result is read out.
 //
 // Operands are K-major in the 128-byte-swizzled layout of tcgen05 (rows of 128 bytes = 32
 // brick points, 8-row groups of 1024 bytes, the 16-byte chunk c of row r stored at chunk
@@ -53,7 +53,11 @@ constexpr int GT_XB = GT_M * GT_K * 4;        // 16 KB: one X slice
 constexpr int GT_BB = GT_NP * GT_K * 4;       // 8 KB: one value slice at most
 constexpr int GT_STAGE = 2 * GT_XB + 2 * GT_BB;   // X hi, X lo, values hi, values lo
 constexpr int GT_THREADS = 320;           // producer, MMA, 4 converter and 4 epilogue warps
-constexpr uint32_t GT_TMEM_COLS = 4 * GT_NP;  // two units in flight x (hi*hi, corrections)
+// An accumulator cuts every addition off, which after the 32 additions of a unit left the inner
+// products 1e-6 of their value too small: three accumulators take hi*hi of slices 0-2, 3-5 and 6-7.
+constexpr int GT_ACCS = 4;                    // accumulators of a unit: three of hi*hi, the corrections
+constexpr uint32_t GT_TMEM_COLS = 2 * GT_ACCS * GT_NP;  // two units in flight
+static_assert(GT_TMEM_COLS <= 512, "TMEM");
 constexpr int GT_D = 4;                       // raw X slices in flight per converter thread
 constexpr size_t GT_SMEM = (size_t)GT_S * GT_STAGE + (size_t)GT_D * GT_XB + 1024;
 constexpr uint32_t kTf32Hi = 0xFFFFE000u;     // sign, exponent and the 10 TF32 significand bits
@@ -174,8 +178,8 @@ k_gather_tc(GtcArgs a) {
                 if (uu >= 2 && !mbar_wait(&tempty_bar[buf], ((uu >> 1) - 1) & 1, &abort_flag)) break;
                 tc_fence_after();
                 const uint32_t idesc = instr_desc_tf32(GT_M, G.z);
-                const uint32_t dcol = tmem + (uint32_t)(2 * buf * GT_NP);      // hi * hi
-                const uint32_t ccol = dcol + (uint32_t)GT_NP;                  // hi * lo + lo * hi
+                const uint32_t dcol = tmem + (uint32_t)(GT_ACCS * buf * GT_NP);      // hi * hi
+                const uint32_t ccol = dcol + (uint32_t)((GT_ACCS - 1) * GT_NP);      // hi * lo + lo * hi
                 bool stop = false;
                 for (int q = 0; q < GT_SLICES; ++q, ++i) {
                     const int s = i % GT_S;
@@ -189,7 +193,7 @@ k_gather_tc(GtcArgs a) {
                     for (int kk = 0; kk < GT_K / 8; ++kk) {
                         const uint64_t ko = (uint64_t)(kk * 32) >> 4;     // 8 TF32 = 32 bytes along a row
                         const uint32_t acc = (q > 0 || kk > 0) ? 1u : 0u;
-                        mma_tf32(dcol, ah + ko, bh + ko, idesc, acc);
+                        mma_tf32(dcol + (uint32_t)(q / 3 * GT_NP), ah + ko, bh + ko, idesc, (q % 3 > 0 || kk > 0) ? 1u : 0u);
                         mma_tf32(ccol, ah + ko, bl + ko, idesc, acc);
                         mma_tf32(ccol, al + ko, bh + ko, idesc, 1u);
                     }
@@ -255,9 +259,10 @@ k_gather_tc(GtcArgs a) {
             const int4 G = a.grp[e];
             const int col = ct * GT_M + row;
             for (int c0 = 0; c0 < G.z; c0 += 16) {
-                float v[16], w[16];
-                tmem_ld16(tmem + lane_base + (uint32_t)(2 * buf * GT_NP + c0), v);
-                tmem_ld16(tmem + lane_base + (uint32_t)(2 * buf * GT_NP + GT_NP + c0), w);
+                float v[GT_ACCS][16];
+#pragma unroll
+                for (int k = 0; k < GT_ACCS; ++k)
+                    tmem_ld16(tmem + lane_base + (uint32_t)((GT_ACCS * buf + k) * GT_NP + c0), v[k]);
                 const int4* gr = reinterpret_cast<const int4*>(a.grow + G.w + c0);   // 16 slots
                 int r[16];
 #pragma unroll
@@ -268,7 +273,7 @@ k_gather_tc(GtcArgs a) {
                 if (col < a.ncol) {
 #pragma unroll
                     for (int f = 0; f < 16; ++f)
-                        if (r[f] >= 0) a.part[(size_t)r[f] * a.ncol + col] = v[f] + w[f];
+                        if (r[f] >= 0) a.part[(size_t)r[f] * a.ncol + col] = (v[0][f] + v[1][f]) + (v[2][f] + v[3][f]);
                 }
             }
             tc_fence_before();
