@@ -230,7 +230,7 @@ k_mm_oz(const __grid_constant__ MzArgs a) {
 #pragma unroll
                 for (int c0 = 0; c0 < 32; c0 += 8) {
                     uint32_t v[C::L * 8];
-                    tmem_levels<C::L, MZ_N>(tmem + lane_base + (uint32_t)(half * 32 + c0), v);
+                    tmem_levels<C::L, MZ_N, 8>(tmem + lane_base + (uint32_t)(half * 32 + c0), v);
 #pragma unroll
                     for (int f = 0; f < 8; ++f) {
                         long long lo;

@@ -4,7 +4,7 @@
 //
 // GB300's FP64 pipe does 2 multiply-adds per clock and SM, so the FP64 products of the
 // point-major form ran at its limit (gather 9.09 ms, scatter 8.99 ms on 88 x 88 x 84 x 348; now
-// 1.28 and 1.50 ms).  Both are small dense products per brick of 8 x 8 x 4 points, and here they run on the FP16
+// 1.28 and 1.37 ms).  Both are small dense products per brick of 8 x 8 x 4 points, and here they run on the FP16
 // tensor cores with operands split into 7 (double) or 4 (float) 8-bit digits (digits.cuh):
 // every digit product and sum is exact, so the result carries the rounding of the operands to
 // 54 (30) bits below the largest magnitude of their column or function and one rounding of the
@@ -28,7 +28,9 @@
 // units.  Warp 0 issues the value copies, warp 1 the MMAs into one of two accumulators, two sets of
 // 8 warps, on alternate slices of 16 k, copy raw X by cp.async (each warp its own 16 orbitals),
 // convert and store the digits, and 4 warps add the levels of finished units.  Scatter kernel: units (brick, 256 reals, NT
-// orbitals); warps 2-3 build the digits of W, warps 4-11 update Y.  Every mbarrier wait is
+// orbitals); 2 (double) or 4 warps build the digits of W and 16 update Y: with 8, in one set, a unit's
+// loads of Y waited for the stores of the one before (1.50 -> 1.37 ms); complex float needs the four
+// builders as well (88 x 88 x 56 x 230: 0.94 -> 0.67 ms; with two 0.97).  Every mbarrier wait is
 // bounded: after its limit the CTA raises FLAG_TIMEOUT, stops issuing, drains what it issued,
 // frees its TMEM and returns.
 //
@@ -51,7 +53,7 @@ constexpr int OZ_M = 128;                     // orbitals (gather) or reals (sca
 constexpr int OZ_CH = 2;                      // 8-real chunks per gather slice (one MMA of K = 16)
 constexpr int OZ_MAXK = 512;                  // slots per brick at most
 constexpr int OZ_SETS = 2;                     // sets of 8 converter warps, on alternate slices
-constexpr int OZ_GTHREADS = 32 * (2 + 8 * OZ_SETS + 4), OZ_STHREADS = 384;
+constexpr int OZ_GTHREADS = 32 * (2 + 8 * OZ_SETS + 4);
 constexpr int kWOff = 4096;                   // d_wmax: biased exponent + kWOff, 0 for a zero column
 constexpr int kWBad = 1 << 20;                // d_wmax of a column with non-finite values
 
@@ -84,6 +86,8 @@ struct SCfg {
     static constexpr int BB = 2 * S * NT * 16;
     static constexpr int NS = S == 7 ? 3 : 5;                     // chunks of values in flight or resident
     static constexpr int NB = 8;                                  // chunks of W digits
+    static constexpr int BW = S == 7 ? 2 : 4;                     // warps that build the digits of W
+    static constexpr int THREADS = 32 * (2 + BW + 16);
     static constexpr int ACC = S * NT;
     static constexpr size_t SMEM = (size_t)NS * AB + NB * BB + 1024;
     static_assert(4 * ACC <= 512 && ACC <= 256, "two units of two tiles in TMEM");
@@ -573,7 +577,7 @@ __device__ __noinline__ double oz_plain(const OzScatter& a, long g, int comp, in
 }
 
 template <typename R, int CW>
-__global__ void __launch_bounds__(OZ_STHREADS, 1)
+__global__ void __launch_bounds__(SCfg<R, CW>::THREADS, 1)
 k_scatter_oz(OzScatter a) {
     using C = SCfg<R, CW>;
     constexpr int S = C::S, NT = C::NT;
@@ -679,8 +683,8 @@ k_scatter_oz(OzScatter a) {
             ia += keep ? nk : nk * a.ctiles;
         }
         if (el) mma_commit(&done_bar);
-    } else if (warp < 4) {
-        // digits of W^T, chunks of 16 slots: warp b builds the chunks b, b + 2, ... (NB is even: a
+    } else if (warp < 2 + C::BW) {
+        // digits of W^T, chunks of 16 slots: warp b builds the chunks b, b + C::BW, ... (which divides NB: a
         // warp waits for every phase of its own stages in turn); lane task (orbital, 8 slots),
         // NT / 16 tasks per lane
         const int b = warp - 2;
@@ -690,7 +694,7 @@ k_scatter_oz(OzScatter a) {
             const int4 B = a.brick[pair_of(q) / C::PASSES];
             const int nk = B.y / 16;
             for (int l = 0; l < nk * a.ctiles; ++l, ++i) {
-                if ((i & 1) != b) continue;
+                if (i % C::BW != b) continue;
                 const int s = i % C::NB, c = l % nk, c0 = (l / nk) * NT;
                 typename Digits<R>::I v[NT / 16][8];
 #pragma unroll
@@ -732,9 +736,12 @@ k_scatter_oz(OzScatter a) {
             }
         }
     } else {
-        // Y update: warps 4-7 the first 128 reals of a unit, 8-11 the second; TMEM lane = real.
-        // The unit's Y values and column exponents are loaded before its product is awaited.
-        const int t = (warp - 4) >> 2, quad = warp & 3;
+        // Y update: two sets of 8 warps on alternate units, so that one's loads of Y are in flight
+        // while the other adds and stores; warps 0-3 of a set the first 128 reals of a unit, 4-7
+        // the second; TMEM lane = real.  The unit's Y values and column exponents are loaded before
+        // its product is awaited.
+        const int set = (warp - 2 - C::BW) >> 3, t = ((warp - 2 - C::BW) >> 2) & 1, quad = warp & 3;
+        constexpr int F = S == 7 ? 4 : 8;          // columns at a time: the registers allow no more
         const uint32_t lane_base = (uint32_t)(32 * quad) << 16;
         const double alpha = a.alpha_dev ? a.alpha_dev[0] : a.alpha;
         int uu = 0;
@@ -748,7 +755,8 @@ k_scatter_oz(OzScatter a) {
             const bool in = x < a.n1 && y < a.n2 && z < a.n3;
             const long g = in ? x + (long)a.n1 * (y + (long)a.n2 * z) : 0;
             for (int ct = 0; ct < a.ctiles; ++ct, ++uu) {
-                const int buf = uu & 1, c0 = ct * NT, nc = in ? min(NT, a.ncol - c0) : 0;
+                if ((uu & 1) != set) continue;
+                const int buf = set, c0 = ct * NT, nc = in ? min(NT, a.ncol - c0) : 0;
                 R* Y = (R*)a.Y + g * CW + comp + (size_t)c0 * a.ld;
                 R yv[NT];
 #pragma unroll
@@ -761,14 +769,14 @@ k_scatter_oz(OzScatter a) {
                 if (__any_sync(0xffffffffu, !ok)) { stop = true; break; }
                 tc_fence_after();
 #pragma unroll
-                for (int o0 = 0; o0 < NT; o0 += 8) {
-                    uint32_t v[S * 8];
-                    tmem_levels<S, NT>(tmem + lane_base + (uint32_t)(buf * 2 * C::ACC + t * C::ACC + o0), v);
+                for (int o0 = 0; o0 < NT; o0 += F) {
+                    uint32_t v[S * F];
+                    tmem_levels<S, NT, F>(tmem + lane_base + (uint32_t)(buf * 2 * C::ACC + t * C::ACC + o0), v);
 #pragma unroll
-                    for (int f = 0; f < 8; ++f) {
+                    for (int f = 0; f < F; ++f) {
                         const int Ef = __shfl_sync(0xffffffffu, E, o0 + f);
                         long long lo;
-                        const long long hi = level_sum<R, 8>(v + f, &lo);
+                        const long long hi = level_sum<R, F>(v + f, &lo);
                         if constexpr (S == 7) {
                             // (hi 2^24 + lo) 256^6 with the low 10 bits rounded off; at least 2^-800 or zero
                             const double r = (double)((hi << 14) + ((lo + 512) >> 10));
@@ -1091,7 +1099,7 @@ int scatter_oz(hub_t h, void* Y, int ncol, int ld, double alpha, const double* a
     const int npair = t.oz_nbricks * C::PASSES;
     HUB_CUDA_TRY(h, cudaFuncSetAttribute(k_scatter_oz<R, CW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM));
     ProfScope ps(h, HUB_K_SCATTER);
-    k_scatter_oz<R, CW><<<std::max(1, std::min(npair, h->num_sms)), OZ_STHREADS, C::SMEM, h->stream>>>(a);
+    k_scatter_oz<R, CW><<<std::max(1, std::min(npair, h->num_sms)), C::THREADS, C::SMEM, h->stream>>>(a);
     HUB_CUDA_TRY(h, cudaGetLastError());
     return HUB_OK;
 }

@@ -156,13 +156,25 @@ __device__ __forceinline__ void tmem_ld8(uint32_t addr, uint32_t* r) {
 __device__ __forceinline__ void keep8(uint32_t* r) {
     asm volatile("" : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]));
 }
-template <int S, int STEP>
-__device__ __forceinline__ void tmem_levels(uint32_t addr, uint32_t (&v)[S * 8]) {
+__device__ __forceinline__ void tmem_ld4(uint32_t addr, uint32_t* r) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr));
+}
+__device__ __forceinline__ void keep4(uint32_t* r) { asm volatile("" : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3])); }
+// F (8 or 4) columns of each level
+template <int S, int STEP, int F>
+__device__ __forceinline__ void tmem_levels(uint32_t addr, uint32_t (&v)[S * F]) {
 #pragma unroll
-    for (int l = 0; l < S; ++l) tmem_ld8(addr + (uint32_t)(l * STEP), v + 8 * l);
+    for (int l = 0; l < S; ++l) {
+        if constexpr (F == 8) tmem_ld8(addr + (uint32_t)(l * STEP), v + 8 * l);
+        else tmem_ld4(addr + (uint32_t)(l * STEP), v + 4 * l);
+    }
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
-    for (int l = 0; l < S; ++l) keep8(v + 8 * l);      // no use of the values moves above the wait
+    for (int l = 0; l < S; ++l) {                      // no use of the values moves above the wait
+        if constexpr (F == 8) keep8(v + 8 * l);
+        else keep4(v + 4 * l);
+    }
 }
 
 }  // namespace hub
