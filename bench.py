@@ -219,13 +219,10 @@ def cpu_oracle_sample(workload: str, seconds: float, cols: int = 2, procs: int =
 # kernel whose source has changed since reports traffic null until it is captured again.
 # Captured on the rutile 2x2x3 workload (348 orbitals, one launch = 226.4 M point-orbitals)
 # with `ncu --metrics dram__bytes_read.sum,dram__bytes_write.sum,gpu__time_duration.sum
-# --clock-control none -k regex:"k_stencil|k_gather|k_scatter" -s 300 -c 3` (FP64) and `-c 6`
-# (`--prec f32`) around `python bench.py [--prec f32] --steps 1 --warmup 1 --no-scf-tts
-# --no-e2e --no-cpu-baseline`; the float gather and scatter are the tensor-core brick forms.
+# --clock-control none -k regex:"k_stencil|k_gather|k_scatter" -s 300 -c 6` around `python bench.py
+# --prec f32 --steps 1 --warmup 1 --no-scf-tts --no-e2e --no-cpu-baseline`; the float gather and
+# scatter are the tensor-core brick forms.
 TRAFFIC_CAPTURES = {
-    ("f64", "stencil"): (25.36, "stencil.cu", "7095f36bbcbc94c0"),
-    ("f64", "gather"): (95.82, "projectors.cu", "4b61aaf339edd58a"),
-    ("f64", "scatter"): (50.96, "projectors.cu", "4b61aaf339edd58a"),
     ("f32", "stencil"): (12.52, "stencil.cu", "7095f36bbcbc94c0"),
     ("f32", "gather"): (5.71, "projectors_tc.cu", "c1f826507f2e5e4b"),
     ("f32", "scatter"): (10.42, "projectors_tc.cu", "c1f826507f2e5e4b"),
@@ -262,7 +259,10 @@ def kernel_roofline(name, t_n, wl, prec, function_points):
                point-orbital (read Y and Yprev, write Yout) against HBM
       gather   FP64: 2 flop per function-point and column against the FP64 pipe; float: one
                read of the block (4 B per point-orbital) against HBM
-      scatter  FP64: as the gather; float: read and write of the block (8 B per point-orbital)"""
+      scatter  FP64: as the gather; float: read and write of the block (8 B per point-orbital)
+    The FP64 kernels compute the same sums in integers (stencil) and on the FP16 tensor cores
+    (gather, scatter), so their fraction of the FP64 pipe can exceed 1; hbm_frac beside it is the
+    same launch against HBM (24, 8 and 16 B per point-orbital)."""
     t_ms, n = t_n
     per_launch_s = t_ms / n / 1e3
     pts_orb = wl.Nd * wl.ncol
@@ -275,6 +275,8 @@ def kernel_roofline(name, t_n, wl, prec, function_points):
                "traffic": traffic * pts_orb if traffic else None, "traffic_unit": "DRAM bytes per launch",
                "kernel": name, "ms_per_launch": t_ms / n,
                "peak_source": "FP64 pipe: 152 SM x 2 FMA/clk x 2.07 GHz (nominal; bench.py --probe-alu measured 1.253)"}
+        gbs = {"stencil": 24.0, "gather": 8.0, "scatter": 16.0}[name] * pts_orb / per_launch_s / 1e9
+        out["hbm_achieved_gbs"], out["hbm_frac"] = gbs, gbs / hbm_peak()[0]
         if name == "stencil":
             out["flop_per_point_orbital"] = STENCIL_FLOP
             out["frac_fma_as_two_flops"] = STENCIL_FLOP_FMA2 * pts_orb / per_launch_s / 1e12 / peak
