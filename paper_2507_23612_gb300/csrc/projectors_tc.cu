@@ -259,10 +259,10 @@ k_gather_tc(GtcArgs a) {
             const int4 G = a.grp[e];
             const int col = ct * GT_M + row;
             for (int c0 = 0; c0 < G.z; c0 += 16) {
-                float v[GT_ACCS][16];
+                uint32_t v[GT_ACCS][16];                     // one wait: a small cell's units are read out in the open
 #pragma unroll
                 for (int k = 0; k < GT_ACCS; ++k)
-                    tmem_ld16(tmem + lane_base + (uint32_t)((GT_ACCS * buf + k) * GT_NP + c0), v[k]);
+                    tmem_ld16_async(tmem + lane_base + (uint32_t)((GT_ACCS * buf + k) * GT_NP + c0), v[k]);
                 const int4* gr = reinterpret_cast<const int4*>(a.grow + G.w + c0);   // 16 slots
                 int r[16];
 #pragma unroll
@@ -270,10 +270,14 @@ k_gather_tc(GtcArgs a) {
                     const int4 q4 = gr[k];
                     r[4 * k] = q4.x; r[4 * k + 1] = q4.y; r[4 * k + 2] = q4.z; r[4 * k + 3] = q4.w;
                 }
+                asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+                for (int k = 0; k < GT_ACCS; ++k) keep16(v[k]);
+                auto f32 = [&](int k, int f) { return __uint_as_float(v[k][f]); };
                 if (col < a.ncol) {
 #pragma unroll
                     for (int f = 0; f < 16; ++f)
-                        if (r[f] >= 0) a.part[(size_t)r[f] * a.ncol + col] = (v[0][f] + v[1][f]) + (v[2][f] + v[3][f]);
+                        if (r[f] >= 0) a.part[(size_t)r[f] * a.ncol + col] = (f32(0, f) + f32(1, f)) + (f32(2, f) + f32(3, f));
                 }
             }
             tc_fence_before();
