@@ -190,10 +190,12 @@ __device__ __forceinline__ double2 ld_far(const double2* p) { return __ldcg(p); 
 __device__ __forceinline__ int exponent_of(double v) { return (__double2hiint(v) >> 20) & 0x7ff; }
 
 // c and sg = s exp(i arg a_pq) of the rotation that zeroes a_pq: s = t c, t the smaller root of
-// t^2 + 2 theta t = 1 with theta = (a_qq - a_pp) / (2 |a_pq|).  t (and the phase) in float, c and s
-// from it in double: the rotation is unitary to rounding, and the pair's coupling falls by 2^-22
-// instead of to rounding, which the next sweep makes up for.  (The divisions and square roots of a
-// double angle are some 50 dependent instructions of the FP64 pipe, of about 64 clocks each.)
+// |a_pq| t^2 + (a_qq - a_pp) t = |a_pq|.  t, 1 / sqrt(1 + t^2) and the phase are estimated in float
+// (2^-22) and corrected once in double (t to 2^-43, the others to rounding), so that the coupling
+// falls below the convergence threshold and one step ends a 2 x 2 problem.  (The divisions and
+// square roots of a double angle are some 50 dependent instructions of the FP64 pipe, of about 64
+// clocks each; these are 11.
+// Left at the float estimates, a step costs 0.15 us less and the coupling falls to 2^-22.)
 template <typename T>
 __device__ __forceinline__ void jacobi_angle(double app, double aqq, T apq, double& c, T& sg) {
     constexpr bool CPLX = sizeof(T) == 16;
@@ -203,35 +205,44 @@ __device__ __forceinline__ void jacobi_angle(double app, double aqq, T apq, doub
     if constexpr (CPLX) e = max(e, max(exponent_of(apq.x), exponent_of(apq.y)) + 1);
     else e = max(e, exponent_of(apq) + 1);
     const double sc = __hiloint2double(max(1, min(2046, 2046 - e)) << 20, 0);
-    const float df = (float)(d * sc);
-    float mf, ph = 1.0f, ph2 = 0.0f;
+    const double D = fabs(d * sc);
+    double a, px = 1.0, py = 0.0;              // |a_pq| and its phase
+    float af;
     if constexpr (CPLX) {
-        const float x = (float)(apq.x * sc), y = (float)(apq.y * sc);
+        const double xd = apq.x * sc, yd = apq.y * sc;
+        const float x = (float)xd, y = (float)yd;
         const float big = fmaxf(fabsf(x), fabsf(y)), up = big < 1e-15f ? 1e18f : 1.0f;      // keeps the square in range
-        const float xs = x * up, ys = y * up, r = rsqrtf(fmaf(xs, xs, ys * ys));
-        ph = xs * r;
-        ph2 = ys * r;
-        mf = 2.0f * (fabsf(x) * fabsf(ph) + fabsf(y) * fabsf(ph2));
+        const float xs = x * up, ys = y * up, rf = rsqrtf(fmaf(xs, xs, ys * ys));
+        af = fabsf(x) * fabsf(xs * rf) + fabsf(y) * fabsf(ys * rf);
+        const double r = (double)rf * (double)up, m = fma(xd, xd, yd * yd);
+        const double h = fma(-(m * r), r, 1.0);
+        const double r1 = fma(r * h, fma(0.375, h, 0.5), r);                // r (1 + h/2 + 3 h^2/8)
+        px = xd * r1;
+        py = yd * r1;
+        a = m * r1;
     } else {
-        mf = 2.0f * fabsf((float)(apq * sc));
+        a = fabs(apq * sc);
+        af = (float)a;
     }
-    const float tf = copysignf(__fdividef(mf, fabsf(df) + sqrtf(fmaf(df, df, mf * mf))), df);
-    const double t = (double)tf, y = (double)rsqrtf(fmaf(tf, tf, 1.0f));   // 2^-22
-    const double u = fma(t, t, 1.0);
-    const double h = fma(-(u * y), y, 1.0);
-    c = fma(y * h, fma(0.375, h, 0.5), y);                                 // y (1 + h/2 + 3 h^2/8): 2^-66
-    const double s = t * c;
-    if constexpr (CPLX) {
-        const double px = (double)ph, py = (double)ph2;
-        const double k = 1.0 - fma(px, px, py * py);
-        const double w = s * fma(k, fma(0.375, k, 0.5), 1.0);
-        sg = make_double2(px * w, py * w);
-    } else {
-        sg = apq >= 0.0 ? s : -s;
-    }
+    const float df = (float)D, mf = 2.0f * af;
+    const float tf = __fdividef(mf, df + sqrtf(fmaf(df, df, mf * mf)));
+    const double t0 = (double)tf, y = (double)rsqrtf(fmaf(tf, tf, 1.0f)), y2 = y * y;
+    const double g = (double)__fdividef(1.0f, fmaf(mf, tf, df));          // one over the derivative
+    const double t = fma(-fma(fma(a, t0, D), t0, -a), g, t0);
+    const double u = fma(t, t, 1.0), ty = t * y;
+    const double h = fma(-u, y2, 1.0), k = fma(0.375, h, 0.5);
+    c = fma(y * h, k, y);                                                  // y (1 + h/2 + 3 h^2/8)
+    const double s = fma(ty * h, k, ty);
+    // the signs of a_qq - a_pp and a_pq by their bits: comparisons are FP64 instructions too
+    int sign = __double2hiint(d);
+    if constexpr (!CPLX) sign ^= __double2hiint(apq);
+    const double ss = __hiloint2double(__double2hiint(s) ^ (sign & (int)0x80000000), __double2loint(s));
+    if constexpr (CPLX) sg = make_double2(px * ss, py * ss);
+    else sg = ss;
 }
-__device__ __forceinline__ double largest_part(double v) { return fabs(v); }
-__device__ __forceinline__ double largest_part(double2 v) { return fmax(fabs(v.x), fabs(v.y)); }
+// the leading word of |v| (of the larger part): compared as integers, off the FP64 pipe
+__device__ __forceinline__ int lead(double v) { return __double2hiint(v) & 0x7fffffff; }
+__device__ __forceinline__ int lead(double2 v) { return max(lead(v.x), lead(v.y)); }
 
 template <typename T>
 struct JacobiArgs {
@@ -259,7 +270,7 @@ struct JacobiArgs {
 //     shared memory (in global memory if they don't fit) and applies the angles of the step before,
 //     which the CTAs of the diagonal groups leave in memory, between its arrival and the release.
 //     One warp only waits.
-// 348 orbitals: 29.9 -> 13.5 ms (58: 3.3 -> 1.7 ms; complex 348: 53.2 -> 22.6 ms) against every CTA
+// 348 orbitals: 29.9 -> 14.0 ms (58: 3.3 -> 1.7 ms; complex 348: 53.2 -> 22.6 ms) against every CTA
 // computing every angle in double and V between the loads and the barrier.  Of a step's 8300 clocks
 // 2600 go into loads and angles, 1700 into the update, 1000 into the stores and 1700 into the wait.
 // The rotation of a pair (p, q) is J = [[c, sg], [-conj(sg), c]] with c real and
@@ -307,7 +318,7 @@ __global__ void __launch_bounds__(kJacThreads, 1) k_jacobi(const __grid_constant
             get(late + RS * k, c, sg);
             int p, q;
             pair_of(step, k, N, p, q);
-            if (q < n && largest_part(sg) != 0.0) {
+            if (q < n && lead(sg) != 0) {
                 T* v = vrow(r);
                 const T vp = v[p], vq = v[q];
                 v[p] = csub(mulr(c, vp), cmul(cconj(sg), vq));
@@ -370,7 +381,7 @@ __global__ void __launch_bounds__(kJacThreads, 1) k_jacobi(const __grid_constant
             break;
         }
         // pairs whose coupling is below this are left alone (threshold Jacobi)
-        const double skip = (CPLX ? 0.7e-3 : 1e-3) * a.tol * fmax(gdia, 1e-300);
+        const int skip = lead((CPLX ? 0.7e-3 : 1e-3) * a.tol * fmax(gdia, 1e-300));
         for (int step = 0; step < N - 1; ++step) {
             // the angles of the step before come in while this step's are computed
             if (before >= 0) {
@@ -404,7 +415,7 @@ __global__ void __launch_bounds__(kJacThreads, 1) k_jacobi(const __grid_constant
                 if (q < n) {
                     const T apq = ld(p, q);
                     const double app = re_of(ld(p, p)), aqq = re_of(ld(q, q));
-                    if (largest_part(apq) > skip) jacobi_angle(app, aqq, apq, c, sg);
+                    if (lead(apq) > skip && lead(apq) <= 0x7ff00000) jacobi_angle(app, aqq, apq, c, sg);   // not NaN
                 }
                 double* w = rot + RS * i;
                 w[0] = c;
