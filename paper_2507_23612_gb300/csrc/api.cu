@@ -344,7 +344,8 @@ namespace hub {
 // block like X.  Complex (Bloch) blocks: S = dV X^H X = L L^H, Hs = dV X^H HX, H^ = L^-1 Hs
 // L^-H (Hermitian), H^ = V diag(eig) V^H, X <- X L^-H V.
 static size_t rr_mat(hub_t h, int n) { return (size_t)n * n * (h->cplx ? 2 : 1); }
-static size_t rr_ws_doubles(hub_t h, int n) { return 6 * rr_mat(h, n) + n; }
+// (an even count: the second spin's matrices follow, and complex ones are read 16 bytes at a time)
+static size_t rr_ws_doubles(hub_t h, int n) { return 6 * rr_mat(h, n) + (n + 1) / 2 * 2; }
 
 static int rr_prepare(hub_t h, int spin, void* X, int n, int ld, void* HX, double* ws) {
     const size_t nn = rr_mat(h, n);
@@ -368,7 +369,7 @@ static int rr_prepare(hub_t h, int spin, void* X, int n, int ld, void* HX, doubl
         if ((rc = launch_gram(h, X, ld, X, ld, n, n, h->dV, true, S))) return rc;
         if ((rc = launch_gram(h, X, ld, HX, ld, n, n, h->dV, true, Hs))) return rc;
     }
-    if ((rc = dense_cholesky(h, S, n, ws + 6 * nn))) return rc;      // scratch: the eigenvalues come later
+    if ((rc = dense_cholesky(h, S, n, ws + 6 * nn))) return rc;     // scratch: the eigenvalues come later
     if ((rc = check_flags(h))) return rc;
     if ((rc = dense_tri_inverse(h, S, Linv, n))) return rc;
     if ((rc = dense_gemm(h, false, false, n, n, n, 1.0, Linv, n, Hs, n, 0.0, T, n))) return rc;
