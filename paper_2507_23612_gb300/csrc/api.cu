@@ -369,7 +369,7 @@ static int rr_prepare(hub_t h, int spin, void* X, int n, int ld, void* HX, doubl
         if ((rc = launch_gram(h, X, ld, X, ld, n, n, h->dV, true, S))) return rc;
         if ((rc = launch_gram(h, X, ld, HX, ld, n, n, h->dV, true, Hs))) return rc;
     }
-    if ((rc = dense_cholesky(h, S, n, ws + 6 * nn))) return rc;     // scratch: the eigenvalues come later
+    if ((rc = dense_cholesky(h, S, n, T))) return rc;     // T, Vs and Q: written later
     if ((rc = check_flags(h))) return rc;
     if ((rc = dense_tri_inverse(h, S, Linv, n))) return rc;
     if ((rc = dense_gemm(h, false, false, n, n, n, 1.0, Linv, n, Hs, n, 0.0, T, n))) return rc;

@@ -17,66 +17,120 @@ namespace {
 
 constexpr int NB = 32;   // Cholesky block
 
+// Cholesky S = L L^H by elimination with multipliers, a_ij <- a_ij - l_ik conj(w_jk) with the
+// column w_k as it stands and l_ik = w_ik / w_kk; L = w_k / sqrt(w_kk).  Every kernel applies the
+// steps k in the same order with the same operation, so that the rows of two equal columns of X
+// stay equal bit for bit, their multiplier is 1 and the second pivot is zero or below: a block with
+// a column twice is refused, and every positive pivot is accepted.  (With products of elements of
+// L that pivot is the rounding of a square root, of either sign.)
+__device__ __forceinline__ double eliminate(double a, double l, double w) { return fma(-l, w, a); }
+__device__ __forceinline__ double2 eliminate(double2 a, double2 l, double2 w) {
+    return make_double2(fma(-l.y, w.y, fma(-l.x, w.x, a.x)), fma(l.x, w.y, fma(-l.y, w.x, a.y)));
+}
+// workspace of a panel: pivots, the diagonal block as it stands, then the rows below: l, w
+template <typename T>
+struct CholWs {
+    double* d;      // [NB]
+    T* w;           // [NB][NB]
+    T *lr, *wr;     // [n - NB][NB]
+};
+
 // factor the jb x jb diagonal block at (j0, j0) in place (one CTA, NB x NB in shared memory);
 // the diagonal of a Hermitian matrix is real, so is L's
 template <typename T>
-__global__ void k_potf2(T* A, int lda, int j0, int jb, int* flags, double* __restrict__ diag, int n) {
+__global__ void k_potf2(T* A, int lda, int j0, int jb, int* flags, CholWs<T> ws, int below) {
     __shared__ T s[NB][NB + 1];
+    __shared__ T l[NB];
+    __shared__ double piv[NB];
     const int t = threadIdx.x;
-    // the diagonal as it was: a pivot within the rounding of its own update (8 x 2^-53 of the
-    // diagonal element) cannot be told from zero
-    if (j0 == 0)
-        for (int i = t; i < n; i += blockDim.x) diag[i] = re_of(A[(size_t)i * lda + i]);
     for (int e = t; e < jb * jb; e += blockDim.x) {
         const int i = e / jb, j = e % jb;
         s[i][j] = A[(size_t)(j0 + i) * lda + j0 + j];
     }
     __syncthreads();
     for (int k = 0; k < jb; ++k) {
+        double d = re_of(s[k][k]);
+        const bool ok = d > 0.0 && isfinite(d);
+        if (!ok) d = 1.0;
         if (t == 0) {
-            const double d = re_of(s[k][k]);
-            if (!(d > 8.8817841970012523e-16 * diag[j0 + k]) || !isfinite(d)) {
-                flags[FLAG_NOTSPD] = 1;
-                s[k][k] = from_real<T>(1.0);
-            } else {
-                s[k][k] = from_real<T>(sqrt(d));
-            }
+            if (!ok) flags[FLAG_NOTSPD] = 1;
+            piv[k] = d;
         }
-        __syncthreads();
-        const double dkk = re_of(s[k][k]);
-        for (int i = k + 1 + t; i < jb; i += blockDim.x) s[i][k] = divr(s[i][k], dkk);
+        for (int i = k + 1 + t; i < jb; i += blockDim.x) l[i] = divr(s[i][k], d);
         __syncthreads();
         for (int e = t; e < jb * jb; e += blockDim.x) {
             const int i = e / jb, j = e % jb;
-            if (i > k && j > k && j <= i) s[i][j] = csub(s[i][j], cmul(s[i][k], cconj(s[j][k])));
+            if (i > k && j > k && j <= i) s[i][j] = eliminate(s[i][j], l[i], s[j][k]);
         }
         __syncthreads();
     }
     for (int e = t; e < jb * jb; e += blockDim.x) {
         const int i = e / jb, j = e % jb;
-        A[(size_t)(j0 + i) * lda + j0 + j] = (j <= i) ? s[i][j] : zero_of(T());
+        const double r = sqrt(piv[j]);
+        A[(size_t)(j0 + i) * lda + j0 + j] = j < i ? divr(s[i][j], r) : j == i ? from_real<T>(r) : zero_of(T());
+        if (below) {
+            ws.w[i * NB + j] = s[i][j];
+            if (i == 0) ws.d[j] = piv[j];
+        }
     }
 }
 
-// rows below the diagonal block: L21 = A21 L11^-H (each thread solves one row)
+// the lower triangle of a Hermitian matrix from the upper one: the Gram product computes both within
+// a tile and mirrors the others, which differ in the rounding of their imaginary parts
+__global__ void k_mirror(double2* A, int n) {
+    const long t = (long)blockIdx.x * blockDim.x + threadIdx.x;
+    const int i = (int)(t / n), j = (int)(t % n);
+    if (i < n && j < i) A[(size_t)i * n + j] = cconj(A[(size_t)j * n + i]);
+}
+
+// rows below the diagonal block: one thread per row
 template <typename T>
-__global__ void k_trsm_rows(T* A, int lda, int j0, int jb, int n) {
-    __shared__ T L[NB][NB + 1];
-    for (int e = threadIdx.x; e < jb * jb; e += blockDim.x) {
-        const int i = e / jb, j = e % jb;
-        L[i][j] = A[(size_t)(j0 + i) * lda + j0 + j];
+__global__ void k_panel(T* A, int lda, int j0, int n, CholWs<T> ws) {
+    __shared__ T w[NB][NB + 1];
+    __shared__ double d[NB], root[NB];
+    for (int e = threadIdx.x; e < NB * NB; e += blockDim.x) w[e / NB][e % NB] = ws.w[e];
+    for (int e = threadIdx.x; e < NB; e += blockDim.x) { d[e] = ws.d[e]; root[e] = sqrt(ws.d[e]); }
+    __syncthreads();
+    const int r = blockIdx.x * blockDim.x + threadIdx.x;
+    if (j0 + NB + r >= n) return;
+    T l[NB];
+    T* row = A + (size_t)(j0 + NB + r) * lda + j0;
+    for (int c = 0; c < NB; ++c) {
+        T v = row[c];
+        for (int k = 0; k < c; ++k) v = eliminate(v, l[k], w[c][k]);
+        l[c] = divr(v, d[c]);
+        ws.wr[(size_t)r * NB + c] = v;
+        ws.lr[(size_t)r * NB + c] = l[c];
+        row[c] = divr(v, root[c]);
+    }
+}
+
+// the lower triangle behind the panel, 32 x 32 tiles
+template <typename T>
+__global__ void k_trail(T* A, int lda, int j1, int n, CholWs<T> ws) {
+    __shared__ T l[NB][NB + 1], w[NB][NB + 1];
+    if (blockIdx.x > blockIdx.y) return;
+    const int tx = threadIdx.x % NB, ty = threadIdx.x / NB, m = n - j1;      // NB x 8 threads
+    const int i0 = blockIdx.y * NB, c0 = blockIdx.x * NB;
+    for (int r = ty; r < NB; r += 8) {
+        l[r][tx] = i0 + r < m ? ws.lr[(size_t)(i0 + r) * NB + tx] : zero_of(T());
+        w[r][tx] = c0 + r < m ? ws.wr[(size_t)(c0 + r) * NB + tx] : zero_of(T());
     }
     __syncthreads();
-    const int r = j0 + jb + blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= n) return;
-    T x[NB];
-    T* row = A + (size_t)r * lda + j0;
-    for (int c = 0; c < jb; ++c) {
-        T v = row[c];
-        for (int cc = 0; cc < c; ++cc) v = csub(v, cmul(x[cc], cconj(L[c][cc])));
-        x[c] = divr(v, re_of(L[c][c]));
+    if (c0 + tx >= m) return;
+    T acc[NB / 8];
+#pragma unroll
+    for (int q = 0; q < NB / 8; ++q)
+        acc[q] = i0 + ty + 8 * q >= m ? zero_of(T()) : A[(size_t)(j1 + i0 + ty + 8 * q) * lda + j1 + c0 + tx];
+#pragma unroll 8
+    for (int k = 0; k < NB; ++k) {
+        const T wk = w[tx][k];
+#pragma unroll
+        for (int q = 0; q < NB / 8; ++q) acc[q] = eliminate(acc[q], l[ty + 8 * q][k], wk);
     }
-    for (int c = 0; c < jb; ++c) row[c] = x[c];
+#pragma unroll
+    for (int q = 0; q < NB / 8; ++q)
+        if (i0 + ty + 8 * q < m) A[(size_t)(j1 + i0 + ty + 8 * q) * lda + j1 + c0 + tx] = acc[q];
 }
 
 // C = alpha op(A) op(B) + beta C, row-major, 32 x 32 tiles; op = identity or the adjoint
@@ -542,19 +596,29 @@ int gemm_t(hub_t h, bool ta, bool tb, int m, int n, int k, double alpha, const T
 }
 
 template <typename T>
-int cholesky_t(hub_t h, T* A, int n, double* diag) {
+int cholesky_t(hub_t h, T* A, int n, double* work) {
+    CholWs<T> ws{};
+    if (n > NB) {
+        ws.d = work;                                     // NB doubles: 16-byte multiples follow
+        ws.w = (T*)(work + NB);
+        ws.lr = ws.w + NB * NB;
+        ws.wr = ws.lr + (size_t)(n - NB) * NB;
+    }
+    if constexpr (sizeof(T) == 16) {
+        ProfScope ps(h, HUB_K_CHOLESKY);
+        k_mirror<<<(unsigned)(((size_t)n * n + 255) / 256), 256, 0, h->stream>>>(A, n);
+        HUB_CUDA_TRY(h, cudaGetLastError());
+    }
     for (int j0 = 0; j0 < n; j0 += NB) {
-        const int jb = std::min(NB, n - j0);
-        { ProfScope ps(h, HUB_K_CHOLESKY); k_potf2<T><<<1, 256, 0, h->stream>>>(A, n, j0, jb, h->d_flags, diag, n); }
+        const int jb = std::min(NB, n - j0), rest = n - j0 - jb;
+        { ProfScope ps(h, HUB_K_CHOLESKY); k_potf2<T><<<1, 256, 0, h->stream>>>(A, n, j0, jb, h->d_flags, ws, rest > 0); }
         HUB_CUDA_TRY(h, cudaGetLastError());
-        const int rest = n - j0 - jb;
         if (rest <= 0) continue;
-        { ProfScope ps(h, HUB_K_CHOLESKY); k_trsm_rows<T><<<(rest + 127) / 128, 128, 0, h->stream>>>(A, n, j0, jb, n); }
+        { ProfScope ps(h, HUB_K_CHOLESKY); k_panel<T><<<(rest + 127) / 128, 128, 0, h->stream>>>(A, n, j0, n, ws); }
         HUB_CUDA_TRY(h, cudaGetLastError());
-        T* A21 = A + (size_t)(j0 + jb) * n + j0;
-        T* A22 = A + (size_t)(j0 + jb) * n + (j0 + jb);
-        int rc = gemm_t<T>(h, false, true, rest, rest, jb, -1.0, A21, n, A21, n, 1.0, A22, n);
-        if (rc) return rc;
+        const unsigned tiles = (rest + NB - 1) / NB;
+        { ProfScope ps(h, HUB_K_CHOLESKY); k_trail<T><<<dim3(tiles, tiles), 256, 0, h->stream>>>(A, n, j0 + jb, n, ws); }
+        HUB_CUDA_TRY(h, cudaGetLastError());
     }
     return HUB_OK;
 }
@@ -627,8 +691,8 @@ int dense_gemm(hub_t h, bool ta, bool tb, int m, int n, int k, double alpha, con
     return gemm_t<double>(h, ta, tb, m, n, k, alpha, A, lda, B, ldb, beta, C, ldc);
 }
 
-int dense_cholesky(hub_t h, double* A, int n, double* diag) {
-    return h->cplx ? cholesky_t<double2>(h, (double2*)A, n, diag) : cholesky_t<double>(h, A, n, diag);
+int dense_cholesky(hub_t h, double* A, int n, double* work) {
+    return h->cplx ? cholesky_t<double2>(h, (double2*)A, n, work) : cholesky_t<double>(h, A, n, work);
 }
 
 int dense_tri_inverse(hub_t h, const double* L, double* Linv, int n) {

@@ -368,7 +368,8 @@ int launch_rotate_bf16(hub_t h, const void* X, int ldx, const double* Q, int k, 
                        void* Y, int ldy);
 
 // dense.cu (double, n x n, row-major)
-int dense_cholesky(hub_t h, double* A, int n, double* diag);   // lower L in place; diag: n doubles of workspace
+// lower L in place; work (16-byte aligned): up to three times A's size, none of it for n <= 32
+int dense_cholesky(hub_t h, double* A, int n, double* work);
 int dense_tri_inverse(hub_t h, const double* L, double* Linv, int n);
 // C = alpha op(A) op(B) + beta C ; row-major n x n style small matrices
 int dense_gemm(hub_t h, bool ta, bool tb, int m, int n, int k, double alpha, const double* A,
