@@ -6,9 +6,10 @@
 //   Yout = alpha * (-1/2 Lap_h Y + V .* Y - shift * Y) + beta * Yprev        (Sec. II.B)
 //
 // Number format.  Every column has one power-of-two scale: with E the biased exponent of its
-// largest |x| (colmax.cu), X = x * 2^(1081 - E) rounded to an integer, |X| <= 2^59, so an
-// element keeps all 53 bits down to 2^-6 of the column's maximum and is never off by more
-// than 2^-60 of it (one FP64 rounding of the sum, which holds terms of ~300 x, is larger).
+// largest |x| (colmax.cu), X = x * 2^(1081 - E) rounded to nearest, 2^58 <= |X| < 2^59 for that
+// x.  An element keeps all 53 bits down to 2^-6 of the column's maximum and is never off by more
+// than 2^-59 of it: one FP64 rounding of the sum, which holds terms of ~300 x, is larger, but an
+// element far below the maximum (the tail of a localized column) has fewer than 53 bits.
 // X is kept as two signed limbs, X = xh 2^30 + xl: pair sums of limbs need no carry.
 // The Laplacian weights of order 2 n0 are rational: c_p = k_p / lcd with integers k_p of 22
 // bits, so A_a = k_0 X + sum_p k_p (X_{+p} + X_{-p}) of each axis is exact, and only
@@ -17,16 +18,19 @@
 // one 64-bit integer per point, converted once; alpha and beta enter in FP64 (three FP64
 // operations per point).  sf fixes the binary points: Fq = F 2^sf, Z counts x-units of
 // 2^(81 - sf), (V - shift)q = (V - shift) 2^(sf - 25); it is as large as the sums' 64 bits
-// allow, 59 bits of F or fewer where |V| exceeds 256 Ha and the sum of F's terms (k_fx_veff).
+// allow: 57 to 59 bits of the largest F, fewer where |V| would pass 2^(83 - sf) (k_fx_veff).  F is
+// rounded at 2^-54 of itself or less, as the weights of the FP64 form are, and V at 2^-54 of the
+// largest kinetic energy or 2^-58 of the largest |V|.
 // Columns that the format does not cover (zero, non-finite or outside 2^+-900), potentials
-// that would leave F under 51 bits and shifts beyond 2^(83 - sf) Ha (the largest kinetic
-// energy of the grid, at least) are computed by fx_slow in plain FP64.
+// that would leave F under 53 bits (8192 Ha at 0.3 bohr, 8 Ha at 10) and shifts beyond
+// 2^(83 - sf) Ha (the largest kinetic energy of the grid, at least) are computed by fx_slow in
+// plain FP64.
 //
 // Kernel: one CTA owns a tile of the x-y plane of one column and marches along z.  A ring of 8
 // planes (with a halo of 6 in x and y) in shared memory holds the limbs; plane z + 7 is
 // converted and stored while plane z is computed, and plane z + 8 is in flight in registers, so
 // there is one barrier per plane.  The 13 z-neighbours live in registers.  Bound: the integer
-// pipes (50 multiply-adds at half rate and ~300 other instructions per point); 17.15 -> 4.12 ms
+// pipes (50 multiply-adds at half rate and ~310 other instructions per point); 17.15 -> 4.25 ms
 // on 88 x 88 x 84 x 348 (DRAM floor 0.80 ms), plus 0.27 ms for the column maxima.
 #include <algorithm>
 #include <cmath>
@@ -70,16 +74,17 @@ __device__ __forceinline__ int wrap(int i, int n) {      // i is at most a few n
     return i;
 }
 
-// x as limbs, cut towards zero; e20 the biased exponent of the column's maximum << 20 (at least
-// 123, so that a denormal x shifts to zero whatever its hidden bit)
+// x to nearest as limbs; e20 the biased exponent of the column's maximum << 20 (at least 123, so
+// that a denormal x shifts to zero whatever its hidden bit).  (Cut towards zero, elements are off by
+// up to twice as much and all to one side; the rounding costs 3 of a point's ~25 instructions.)
 __device__ __forceinline__ int2 to_limbs(double v, int e20) {
     const unsigned hi = (unsigned)__double2hiint(v), lo = (unsigned)__double2loint(v);
-    const int s = min((e20 - (int)(hi & 0x7ff00000u)) >> 20, 61) + 2;
-    // the significand times 2^8, 61 bits: X = t >> s
+    const int s = min((e20 - (int)(hi & 0x7ff00000u)) >> 20, 61) + 1;
+    // the significand times 2^8, 61 bits: X = (t >> s, to half a unit) / 2 up
     const unsigned th = __funnelshift_l(lo, (hi & 0xfffffu) | 0x100000u, 8), tl = lo << 8;
-    const unsigned xl = (unsigned)((((unsigned long long)th << 32) | tl) >> s) & 0x3fffffffu;
-    const unsigned xh = __funnelshift_rc(th, 0u, s - 2);
-    return (int)hi < 0 ? make_int2(-(int)xh, -(int)xl) : make_int2((int)xh, (int)xl);
+    const unsigned long long t = ((((unsigned long long)th << 32) | tl) >> s) + 1;
+    const int xl = (int)((unsigned)(t >> 1) & 0x3fffffffu), xh = (int)(t >> 31);
+    return (int)hi < 0 ? make_int2(-xh, -xl) : make_int2(xh, xl);
 }
 
 // the plain FP64 form of one tile and chunk, straight from global memory; returns this thread's sum
@@ -342,11 +347,11 @@ __global__ void k_fx_vmax(const double* __restrict__ V, int* __restrict__ info, 
     if ((threadIdx.x & 31) == 0) atomicMax(info, (int)m);
 }
 
-// limbs of V 2^(sf - 25) with |V| < 2^(83 - sf), sf <= sf0
-__global__ void k_fx_veff(const double* __restrict__ V, int2* __restrict__ Vq, int* __restrict__ info, long n, int sf0) {
+// limbs of V 2^(sf - 25) with |V| < 2^(83 - sf), sfmin <= sf <= sf0
+__global__ void k_fx_veff(const double* __restrict__ V, int2* __restrict__ Vq, int* __restrict__ info, long n, int sf0, int sfmin) {
     const long t = (long)blockIdx.x * blockDim.x + threadIdx.x;
     const int sf = min(sf0, 83 - ((info[0] >> 20) - 1022));       // |V| < 2^(exponent - 1022)
-    const bool bad = sf < sf0 - 8;                               // non-finite values included
+    const bool bad = sf < sfmin;                                 // non-finite values included
     if (t == 0) { info[1] = bad; info[2] = bad ? sf0 : sf; }
     if (t >= n) return;
     const long long q = bad ? 0 : __double2ll_rn(scalbn(V[t], sf - 25));
@@ -356,7 +361,7 @@ __global__ void k_fx_veff(const double* __restrict__ V, int2* __restrict__ Vq, i
 // c_p = k_p / lcd of the centred second derivative of order 2 n0, and sf
 struct FxSetup {
     int k[FXH + 1];
-    int lcd, sf;
+    int lcd, sf, sfmin;       // sfmin: F of 53 bits
 };
 FxSetup fx_setup(hub_t h) {
     static const int lcds[FXH + 1] = {1, 1, 12, 180, 5040, 25200, 831600};
@@ -378,10 +383,14 @@ FxSetup fx_setup(hub_t h) {
     }
     double fmax = 0.0;
     for (int a = 0; a < 3; ++a) fmax = std::max(fmax, 0.5 / (s.lcd * h->h[a] * h->h[a]));
-    // |Fq| < 2^59 keeps the three products of Z in 64 bits; sf <= 75 leaves 256 Ha for V
+    // |Fq| < 2^59 keeps the three products of Z in 64 bits; sf <= 75 leaves 256 Ha for V and the shift.
+    // On coarse grids (above 0.4 bohr) that would cut off bits of F (beyond 4 bohr) and of V, which is rounded
+    // at 2^(24 - sf): 57 - e keeps that under 2^-54 of the largest kinetic energy (2^22.5 F on every
+    // axis) and leaves 2^(26 + e) Ha, four times that energy
     int e;
-    std::frexp(fmax, &e);                         // fmax < 2^e
-    s.sf = std::min(75, 59 - e);
+    std::frexp(fmax, &e);                         // 2^(e - 1) <= fmax < 2^e
+    s.sf = std::max(std::min(75, 59 - e), 57 - e);
+    s.sfmin = 53 - e;
     return s;
 }
 
@@ -401,7 +410,7 @@ int launch_fx_veff(hub_t h, const void* V) {
         k_fx_vmax<<<h->num_sms, 256, 0, h->stream>>>((const double*)V, info, n);
     }
     ProfScope ps(h, HUB_K_COPY);
-    k_fx_veff<<<(unsigned)((n + 255) / 256), 256, 0, h->stream>>>((const double*)V, Vq, info, n, s.sf);
+    k_fx_veff<<<(unsigned)((n + 255) / 256), 256, 0, h->stream>>>((const double*)V, Vq, info, n, s.sf, s.sfmin);
     HUB_CUDA_TRY(h, cudaGetLastError());
     return HUB_OK;
 }
@@ -490,7 +499,8 @@ static int run_fx(hub_t h, const StencilArgs& s, int variant, const StencilDot* 
     return HUB_OK;
 }
 
-// CTA shapes (hub_set_tuning; 0 is the default), on 88 x 88 x 84 x 348: 4.12, 4.25 and 4.40 ms.
+// CTA shapes (hub_set_tuning; 0 is the default), on 88 x 88 x 84 x 348 of normal deviates: 4.14, 4.15
+// and 4.12 ms.
 // Four CTAs of 192 threads hide the barriers of one another's planes; two rows per thread need
 // fewer instructions (382 against ~450 per point) but leave 16 warps per SM.
 int launch_stencil_fx(hub_t h, const StencilArgs& s) {
