@@ -6,10 +6,21 @@
 // magnitude of the group, of 54 bits (double) or 30 bits (float), written as S = 7 or 4
 // signed base-256 digits d_1 .. d_S in [-128, 127] (|d_1| <= 64).  FP16 holds every digit
 // exactly, a product of two digits is an integer of at most 14 bits and the FP32 accumulator
-// of the tensor core holds integers up to 2^24, so a sum over at most 256 terms of the products
-// of one level l = i + j - 1 (digits i and j; at most l products) is exact for l <= 4 in any
-// case and for the others short of 2^24, which needs digits of nearly full size and equal sign
-// throughout.  Levels above S are dropped (2^-56 and 2^-32 of the largest product).
+// of the tensor core holds integers up to 2^24.  A level l = i + j - 1 (digits i and j) has l
+// products, of at most (l - 2) 2^14 + 2 x 2^13 together (2^12 for l = 1):
+//
+//   terms    sums within 2^24 whatever the digits
+//   256      levels 1 - 5 (6 and 7 can pass it by a quarter and a half)
+//   512      levels 1 - 3
+//
+// and an accumulator beyond 2^24 drops the odd unit of an addition.  The double forms (S = 7) sum at
+// most 256 terms: what levels 6 and 7 can lose is under 2^-54 of a sum of products that are all
+// that large.  With 512 it would be 2^-40 (level 4).  The float forms (S = 4, in Gram products
+// and rotations 5 levels) sum up to 512, with at most 2^-37.  Levels beyond are dropped (2^-56 and
+// 2^-32 of the largest product; 2^-40 with 5 levels).
+//
+// The bits are relative to the largest magnitude of the group: a number 2^-k of it has k bits
+// fewer, down to none, where a floating-point operand would keep all of its own.
 #pragma once
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>

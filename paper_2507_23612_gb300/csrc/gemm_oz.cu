@@ -6,9 +6,10 @@
 //
 // On CUDA cores the FP64 pipe (2 multiply-adds per clock and SM) bounds both: 80.1 and 140.4 ms on
 // 650,496 x 348.  Here every operand is split into 7 (double) or 4 (float) 8-bit digits, the
-// digit products are summed exactly in FP32 accumulators, read out every 512 terms and added up
-// in 64-bit integers: the result carries the rounding of the operands to 54 (30) bits of their
-// column's largest magnitude and one rounding of the sum.
+// digit products are summed in FP32 accumulators, read out every 256 (512) terms, up to which the
+// sums are exact where it counts (digits.cuh), and added up in 64-bit integers: the result carries
+// the rounding of the operands to 54 (30) bits of their column's largest magnitude and one rounding
+// of the sum.  (Every 512 terms the double forms took 0.5 ms less, of 4.5 and 3.2.)
 //
 // Both are D[128 x 64] = sum_k A[128, k] B[64, k]: rows and columns are orbitals and k the grid
 // for the Gram product (k split over CTAs), rows are grid points, columns the new and k the old
@@ -39,7 +40,6 @@ namespace hub {
 namespace {
 
 constexpr int MZ_M = 128, MZ_N = 64;
-constexpr int MZ_GROUP = 32;                        // 16-k steps per read-out of the accumulators
 constexpr int MZ_THREADS = 320;
 constexpr size_t MZ_PANEL = (size_t)1 << 30;        // bytes of one operand's digits per panel
 
@@ -49,6 +49,7 @@ struct MCfg {
     static constexpr int AB = S * MZ_M * 32, BB = S * MZ_N * 32;      // bytes of 16 k of a tile
     static constexpr int STAGE = AB + BB;
     static constexpr int NS = S == 7 ? 5 : 8;
+    static constexpr int GROUP = S == 7 ? 16 : 32;      // 16-k steps per read-out of the accumulators
     // levels kept: one more than digits for float, because the first dropped level must not hold
     // squares (digit 3 times digit 3 of a column with itself adds up over the grid)
     static constexpr int L = S == 7 ? 7 : 5;
@@ -127,7 +128,7 @@ k_mm_oz(const __grid_constant__ MzArgs a) {
         const int u = (int)blockIdx.x + uu * (int)gridDim.x;
         return make_int2(u / a.ct, u % a.ct);
     };
-    const int nk = ks1 - ks0, ngr = (nk + MZ_GROUP - 1) / MZ_GROUP;   // groups per unit
+    const int nk = ks1 - ks0, ngr = (nk + C::GROUP - 1) / C::GROUP;   // groups per unit
 
     if (threadIdx.x == 0) {
         abort_flag = 0;
@@ -179,10 +180,10 @@ k_mm_oz(const __grid_constant__ MzArgs a) {
         int s = 0, ph = 0, gi = 0;
         bool stop = false;
         for (int uu = 0; uu < nu && !stop; ++uu)
-            for (int c0 = 0; c0 < nk && !stop; c0 += MZ_GROUP, ++gi) {
+            for (int c0 = 0; c0 < nk && !stop; c0 += C::GROUP, ++gi) {
                 if (gi >= 1 && !wait(&tempty_bar, (gi - 1) & 1)) { stop = true; break; }
                 tc_fence_after();
-                const int c1 = min(nk, c0 + MZ_GROUP);
+                const int c1 = min(nk, c0 + C::GROUP);
                 for (int c = c0; c < c1; ++c) {
                     if (!wait(&full_bar[s], ph)) { stop = true; break; }
                     tc_fence_after();

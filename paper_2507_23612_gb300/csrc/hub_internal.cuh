@@ -100,6 +100,7 @@ struct Table {
     // without the brick tables above.  A function has one slot (real) or two (complex)
     int oz = 0;                       // 1 when the arrays below are built
     int oz_ngroups = 0, oz_nbricks = 0;
+    bool oz_wide = false;             // a brick has more than 256 slots
     long oz_npart = 0;                // (function, brick) pairs: partial rows of the gather
     int4* d_ozg = nullptr;            // per group: brick, slots, 16-byte offset of its values, first slot
     int2* d_ozg_row = nullptr;        // per slot: partial row (x slots per function; -1 padding), exponent

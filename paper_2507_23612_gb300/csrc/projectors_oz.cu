@@ -6,9 +6,10 @@
 // point-major form ran at its limit (gather 9.09 ms, scatter 8.99 ms on 88 x 88 x 84 x 348; now
 // 1.09 and 1.37 ms).  Both are small dense products per brick of 8 x 8 x 4 points, and here they run on the FP16
 // tensor cores with operands split into 7 (double) or 4 (float) 8-bit digits (digits.cuh):
-// every digit product and sum is exact, so the result carries the rounding of the operands to
-// 54 (30) bits below the largest magnitude of their column or function and one rounding of the
-// sum, below the rounding of the sums it replaces.
+// digit products and, where it counts, their sums are exact, so the result carries the rounding of
+// the operands to 54 (30) bits below the largest magnitude of their column or function and one
+// rounding of the sum.  Over a column that is below the rounding of the sums it replaces; where the
+// column is far below its own maximum, inner products and updates have fewer bits than those had.
 //
 // Complex blocks are real ones of twice the points and functions: a brick's 256 complex points
 // are 512 reals (re, im alternating), a function has slot a = (phi_r, phi_i) (real part of
@@ -65,7 +66,10 @@ struct GCfg {
     // 115: 0.173 -> 0.158 ms); double has no room for the stages
     static constexpr int CH = S == 7 ? 2 : 4;
     static constexpr int NP = S == 7 ? 64 : 128;                  // slots per group at most
-    static constexpr int SLICES = BRP * CW / (8 * CH);
+    // A brick of complex double is two units of 256 reals: the sums of 512 products of digits could
+    // pass 2^24 (digits.cuh).  88 x 88 x 56 x 230: 2.08 ms against 1.54 for whole bricks.
+    static constexpr int PARTS = S == 7 ? CW : 1;
+    static constexpr int SLICES = BRP * CW / (8 * CH) / PARTS;
     static constexpr int CB = 8 * (int)sizeof(R), PC = CB / 16;   // a raw chunk, its 16-byte pieces
     static constexpr int PPP = 16 / (int)sizeof(R) / CW;          // points per piece (complex double: 1)
     static constexpr int XB = S * CH * OZ_M * 16;              // digits of one X slice
@@ -92,6 +96,7 @@ struct SCfg {
     static constexpr int NS = S == 7 ? 3 : 5;                     // chunks of values in flight or resident
     static constexpr int NB = 8;                                  // chunks of W digits
     static constexpr int BW = S == 7 ? 2 : 4;                     // warps that build the digits of W
+    static constexpr int PCH = 16;                                // chunks per read-out of the wide form
     static constexpr int THREADS = 32 * (2 + BW + 16);
     static constexpr int ACC = S * NT;
     static constexpr size_t SMEM = (size_t)NS * AB + NB * BB + 1024;
@@ -112,6 +117,7 @@ struct OzGather {
     double* part;
     const unsigned* cmax;
     int* wmax;                // cleared for the reduction
+    long part_rows;           // rows of one part of the bricks
     long ld;                  // in reals
     int n1, n2, n3, ncol, nbx, nby, nunits, ctiles, vec;
     int* flags;
@@ -167,14 +173,15 @@ k_gather_oz(OzGather a) {
         if (lane == 0) {
             int i = 0;
             for (int uu = 0; uu < nu && !abort_flag; ++uu) {
-                const int4 G = a.grp[((int)blockIdx.x + uu * (int)gridDim.x) / a.ctiles];
+                const int u = (int)blockIdx.x + uu * (int)gridDim.x, part = (u / a.ctiles) % C::PARTS;
+                const int4 G = a.grp[u / (a.ctiles * C::PARTS)];
                 const uint32_t units = (uint32_t)(C::CH * S * G.y);
                 bool stop = false;
                 for (int q = 0; q < C::SLICES; ++q, ++i) {
                     const int s = i % C::NV;
                     if (i >= C::NV && !mbar_wait(&vempty_bar[s], ((i / C::NV) - 1) & 1, &abort_flag)) { stop = true; break; }
                     mbar_expect_tx(&full_bar[s], units * 16);
-                    bulk_load(vring + (size_t)s * C::VB, a.val + (size_t)G.z + (size_t)q * units, units * 16,
+                    bulk_load(vring + (size_t)s * C::VB, a.val + (size_t)G.z + (size_t)(part * C::SLICES + q) * units, units * 16,
                               &full_bar[s]);
                     issued_sh = i + 1;
                 }
@@ -189,7 +196,7 @@ k_gather_oz(OzGather a) {
         bool stop = false;
         uint32_t before = 0;                        // slots of the unit before
         for (int uu = 0; uu < nu && !stop; ++uu) {
-            const uint32_t np = (uint32_t)__shfl_sync(0xffffffffu, a.grp[((int)blockIdx.x + uu * (int)gridDim.x) / a.ctiles].y, 0);
+            const uint32_t np = (uint32_t)__shfl_sync(0xffffffffu, a.grp[((int)blockIdx.x + uu * (int)gridDim.x) / (a.ctiles * C::PARTS)].y, 0);
             const int buf = uu & 1;
             if (uu >= 2 && !wait(&tempty_bar[buf], ((uu >> 1) - 1) & 1)) break;
             // the unit before has to be read out first where the two don't fit
@@ -249,13 +256,15 @@ k_gather_oz(OzGather a) {
         const R* cb[NJ];
         bool cok[NJ];
         int gx = 0, gy = 0, gz = 0;                      // brick corner
+        int chunk0 = 0;                                  // first chunk of the unit's part of the brick
         bool more = false;                               // the warp has orbitals in this unit
         auto issue = [&](int j) {                        // the set's j-th slice
             const int i = set + OZ_SETS * j, nq = i % C::SLICES;
             if (i < nsl) {
                 if (nq == set) {
                     const int u = (int)blockIdx.x + (i / C::SLICES) * (int)gridDim.x;
-                    const int brick = a.grp[u / a.ctiles].x, c0 = (u % a.ctiles) * OZ_M + 16 * w;
+                    const int brick = a.grp[u / (a.ctiles * C::PARTS)].x, c0 = (u % a.ctiles) * OZ_M + 16 * w;
+                    chunk0 = (u / a.ctiles) % C::PARTS * (C::SLICES * C::CH);
                     gx = 8 * (brick % a.nbx) + C::PPP * lp;
                     gy = 8 * ((brick / a.nbx) % a.nby);
                     gz = 4 * (brick / (a.nbx * a.nby));
@@ -271,7 +280,7 @@ k_gather_oz(OzGather a) {
                 if (more)
 #pragma unroll
                 for (int r = 0; r < C::CH; ++r) {
-                    const int row = (nq * C::CH + r) / CW, x = gx + (CW == 2 ? 4 * (r & 1) : 0);
+                    const int row = (chunk0 + nq * C::CH + r) / CW, x = gx + (CW == 2 ? 4 * (r & 1) : 0);
                     const int y = gy + (row & 7), z = gz + (row >> 3);
                     const size_t off = ((size_t)x + (size_t)a.n1 * (y + (size_t)a.n2 * z)) * CW;
                     const bool rin = y < a.n2 && z < a.n3;
@@ -358,7 +367,8 @@ k_gather_oz(OzGather a) {
         for (int uu = 0; uu < nu; ++uu) {
             const int u = (int)blockIdx.x + uu * (int)gridDim.x;
             const int buf = uu & 1;
-            const int4 G = a.grp[u / a.ctiles];
+            const int4 G = a.grp[u / (a.ctiles * C::PARTS)];
+            const size_t row0 = (size_t)((u / a.ctiles) % C::PARTS) * a.part_rows;
             const int col = (u % a.ctiles) * OZ_M + 32 * quad + lane;
             int E = col < a.ncol ? (int)(column_max(a.cmax, col) >> (sizeof(R) == 8 ? 20 : 23)) : 0;
             const bool ok = mbar_wait(&tfull_bar[buf], (uu >> 1) & 1, &abort_flag);
@@ -398,7 +408,7 @@ k_gather_oz(OzGather a) {
                         k += 24;
                     }
                     r = scale2(r, k);
-                    if (row >= 0 && col < a.ncol) a.part[(size_t)row * a.ncol + col] = r;
+                    if (row >= 0 && col < a.ncol) a.part[(row0 + row) * a.ncol + col] = r;
                 }
             }
             tc_fence_before();
@@ -444,6 +454,7 @@ struct OzReduce {
     const void* X;
     const int* idx;
     const void* vals;
+    long part_rows;
     long ld;                  // in elements
     double dV;
     int ncol, want_W;
@@ -461,6 +472,13 @@ k_reduce_oz(OzReduce a) {
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int n = blockIdx.y * 32 + lane;
     const int nr = S.nproj * CW;
+    auto partial = [&](int e, int c) {
+        const size_t row = (size_t)a.rent[e] * CW + c;
+        double v = a.part[row * a.ncol + n];
+#pragma unroll
+        for (int k = 1; k < GCfg<R, CW>::PARTS; ++k) v += a.part[(row + k * a.part_rows) * a.ncol + n];
+        return v;
+    };
     for (int p = 0; p < S.nproj; ++p) {
         const int e0 = a.roff[S.proj_off + p], e1 = a.roff[S.proj_off + p + 1];
         double acc[CW] = {};
@@ -471,7 +489,7 @@ k_reduce_oz(OzReduce a) {
 #pragma unroll
                 for (int k = 0; k < 4; ++k)
 #pragma unroll
-                    for (int c = 0; c < CW; ++c) v[k][c] = a.part[((size_t)a.rent[e + 8 * k] * CW + c) * a.ncol + n];
+                    for (int c = 0; c < CW; ++c) v[k][c] = partial(e + 8 * k, c);
 #pragma unroll
                 for (int k = 0; k < 4; ++k)
 #pragma unroll
@@ -479,7 +497,7 @@ k_reduce_oz(OzReduce a) {
             }
             for (; e < e1; e += 8)
 #pragma unroll
-                for (int c = 0; c < CW; ++c) acc[c] += a.part[((size_t)a.rent[e] * CW + c) * a.ncol + n];
+                for (int c = 0; c < CW; ++c) acc[c] += partial(e, c);
         }
 #pragma unroll
         for (int c = 0; c < CW; ++c) red[w][p * CW + c][lane] = acc[c];
@@ -607,7 +625,10 @@ __device__ __noinline__ double oz_plain(const OzScatter& a, long g, int comp, in
     return s;
 }
 
-template <typename R, int CW>
+// WIDE: double, with more than 256 slots on some brick, which are read out every 256: the sums of more
+// products of digits could pass 2^24 (digits.cuh).  A form of its own: the loops of the read-outs
+// cost the others 5 % (88 x 88 x 84 x 348: 1.35 against 1.42 ms).
+template <typename R, int CW, bool WIDE>
 __global__ void __launch_bounds__(SCfg<R, CW>::THREADS, 1)
 k_scatter_oz(OzScatter a) {
     using C = SCfg<R, CW>;
@@ -681,27 +702,36 @@ k_scatter_oz(OzScatter a) {
         auto wait = [&](uint64_t* bar, int parity) { return __all_sync(0xffffffffu, mbar_wait(bar, parity, &abort_flag)) != 0; };
         const uint32_t a0 = desc_lo(ring, OZ_M * 16), b0 = desc_lo(wring, S * NT * 16);
         int ia = 0, sb = 0, pb = 0, uu = 0;         // value chunks so far, W stage and its phase, units so far
+        int used0 = 0, used1 = 0;                   // read-outs so far of either buffer (WIDE)
         bool stop = false;
         for (int q = 0; q < np && !stop; ++q) {
             const int nk = __shfl_sync(0xffffffffu, a.brick[pair_of(q) / C::PASSES].y, 0) / 16;
             const bool keep = nk <= C::NS;
             for (int ct = 0; ct < a.ctiles && !stop; ++ct, ++uu) {
                 const int buf = uu & 1;
-                if (uu >= 2 && !wait(&tempty_bar[buf], ((uu >> 1) - 1) & 1)) { stop = true; break; }
-                tc_fence_after();
                 const uint32_t d0 = tmem + (uint32_t)(buf * 2 * C::ACC);
                 int s = (keep ? ia : ia + ct * nk) % C::NS, ph = ((keep ? ia : ia + ct * nk) / C::NS) & 1;
+                int used = WIDE ? (buf ? used1 : used0) : uu >> 1;
+                if (used >= 1 && !wait(&tempty_bar[buf], (used - 1) & 1)) { stop = true; break; }
+                tc_fence_after();
                 for (int c = 0; c < nk; ++c) {
+                    if (WIDE && c > 0 && c % C::PCH == 0) {            // read out in between
+                        if (el) mma_commit(&tfull_bar[buf]);
+                        ++used;
+                        if (!wait(&tempty_bar[buf], (used - 1) & 1)) { stop = true; break; }
+                        tc_fence_after();
+                    }
                     if (!wait(&full_bar[s], ph) || !wait(&w_bar[sb], pb)) { stop = true; break; }
                     tc_fence_after();
                     if (el) {
                         const uint32_t ao = a0 + (uint32_t)(s * (C::AB / 16)), bo = b0 + (uint32_t)(sb * (C::BB / 16));
+                        const uint32_t more = (WIDE ? c % C::PCH : c) > 0 ? 1u : 0u;
 #pragma unroll
                         for (int t = 0; t < 2; ++t)
 #pragma unroll
                             for (int d = 0; d < S; ++d)
                                 mma_f16_lo(d0 + (uint32_t)(t * C::ACC + d * NT), ao + (uint32_t)((t * S + d) * (2 * OZ_M)), bo, kDescHi,
-                                           instr_desc_f16(OZ_M, (S - d) * NT), (c > 0 || d > 0) ? 1u : 0u);
+                                           instr_desc_f16(OZ_M, (S - d) * NT), d > 0 ? 1u : more);
                         mma_commit(&wempty_bar[sb]);
                         if (!keep || ct == a.ctiles - 1) mma_commit(&empty_bar[s]);
                     }
@@ -710,6 +740,7 @@ k_scatter_oz(OzScatter a) {
                     if (++sb == C::NB) { sb = 0; pb ^= 1; }
                 }
                 if (el && !stop) mma_commit(&tfull_bar[buf]);
+                if (WIDE) (buf ? used1 : used0) = used + 1;
             }
             ia += keep ? nk : nk * a.ctiles;
         }
@@ -775,10 +806,10 @@ k_scatter_oz(OzScatter a) {
         constexpr int F = S == 7 ? 4 : 8;          // columns at a time: the registers allow no more
         const uint32_t lane_base = (uint32_t)(32 * quad) << 16;
         const double alpha = a.alpha_dev ? a.alpha_dev[0] : a.alpha;
-        int uu = 0;
+        int uu = 0, used = 0;                      // units so far; read-outs so far of this set's buffer (WIDE)
         bool stop = false;
         for (int q = 0; q < np && !stop; ++q) {
-            const int pr = pair_of(q), brick = a.brick[pr / C::PASSES].x;
+            const int pr = pair_of(q), brick = a.brick[pr / C::PASSES].x, nk = WIDE ? a.brick[pr / C::PASSES].y / 16 : 0;
             const int k = (pr % C::PASSES) * 256 + t * 128 + 32 * quad + lane;
             const int p = k / CW, comp = k % CW;
             const int x = 8 * (brick % a.nbx) + (p & 7), y = 8 * ((brick / a.nbx) % a.nby) + ((p >> 3) & 7);
@@ -796,33 +827,40 @@ k_scatter_oz(OzScatter a) {
                 const int wm = lane < NT && c0 + lane < a.ncol ? a.wmax[c0 + lane] : 0;
                 const int E = wm == 0 ? Digits<R>::kBias : wm - kWOff;
                 const unsigned odd = __ballot_sync(0xffffffffu, wm >= kWBad || E < Digits<R>::kEmin || E > Digits<R>::kEmax);
-                const bool ok = mbar_wait(&tfull_bar[buf], (uu >> 1) & 1, &abort_flag);
-                if (__any_sync(0xffffffffu, !ok)) { stop = true; break; }
-                tc_fence_after();
+                auto read_out = [&]() {
+                    const bool ok = mbar_wait(&tfull_bar[buf], (WIDE ? used : uu >> 1) & 1, &abort_flag);
+                    if (__any_sync(0xffffffffu, !ok)) { stop = true; return; }
+                    tc_fence_after();
 #pragma unroll
-                for (int o0 = 0; o0 < NT; o0 += F) {
-                    uint32_t v[S * F];
-                    tmem_levels<S, NT, F>(tmem + lane_base + (uint32_t)(buf * 2 * C::ACC + t * C::ACC + o0), v);
+                    for (int o0 = 0; o0 < NT; o0 += F) {
+                        uint32_t v[S * F];
+                        tmem_levels<S, NT, F>(tmem + lane_base + (uint32_t)(buf * 2 * C::ACC + t * C::ACC + o0), v);
 #pragma unroll
-                    for (int f = 0; f < F; ++f) {
-                        const int Ef = __shfl_sync(0xffffffffu, E, o0 + f);
-                        long long lo;
-                        const long long hi = level_sum<R, F>(v + f, &lo);
-                        if constexpr (S == 7) {
-                            // (hi 2^24 + lo) 256^6 with the low 10 bits rounded off; at least 2^-800 or zero
-                            const double r = (double)((hi << 14) + ((lo + 512) >> 10));
-                            const int up = (10 + 48 + Ef + Digits<R>::kBias - 2 * Digits<R>::kUnit) << 20;
-                            yv[o0 + f] = fma(alpha, r == 0.0 ? r : __hiloint2double(__double2hiint(r) + up, __double2loint(r)),
-                                             yv[o0 + f]);
-                        } else {
-                            // hi 2^(24 + Ef + bias - 2 unit) in two factors within the range of float
-                            const float sc = __int_as_float((24 + Ef + Digits<R>::kBias - 2 * Digits<R>::kUnit + 40 + 127) << 23);
-                            yv[o0 + f] = fmaf((float)alpha * sc, (float)hi * 9.094947017729282e-13f, yv[o0 + f]);   // 2^-40
+                        for (int f = 0; f < F; ++f) {
+                            const int Ef = __shfl_sync(0xffffffffu, E, o0 + f);
+                            long long lo;
+                            const long long hi = level_sum<R, F>(v + f, &lo);
+                            if constexpr (S == 7) {
+                                // (hi 2^24 + lo) 256^6 with the low 10 bits rounded off; at least 2^-800 or zero
+                                const double r = (double)((hi << 14) + ((lo + 512) >> 10));
+                                const int up = (10 + 48 + Ef + Digits<R>::kBias - 2 * Digits<R>::kUnit) << 20;
+                                yv[o0 + f] = fma(alpha, r == 0.0 ? r : __hiloint2double(__double2hiint(r) + up, __double2loint(r)),
+                                                 yv[o0 + f]);
+                            } else {
+                                // hi 2^(24 + Ef + bias - 2 unit) in two factors within the range of float
+                                const float sc = __int_as_float((24 + Ef + Digits<R>::kBias - 2 * Digits<R>::kUnit + 40 + 127) << 23);
+                                yv[o0 + f] = fmaf((float)alpha * sc, (float)hi * 9.094947017729282e-13f, yv[o0 + f]);   // 2^-40
+                            }
                         }
                     }
-                }
-                tc_fence_before();
-                mbar_arrive(&tempty_bar[buf]);
+                    tc_fence_before();
+                    mbar_arrive(&tempty_bar[buf]);
+                    ++used;
+                };
+                read_out();
+                if constexpr (WIDE)
+                    for (int c = C::PCH; c < nk && !stop; c += C::PCH) read_out();
+                if (stop) break;
 #pragma unroll
                 for (int o = 0; o < NT; ++o)
                     if (o < nc && !((odd >> o) & 1u)) Y[(size_t)o * a.ld] = yv[o];
@@ -1004,6 +1042,7 @@ int build_oz(hub_t h, Table& t, const std::vector<std::vector<int>>& site_pts) {
         for (int q = bs; q < K; ++q) { bslot.push_back(make_int2(-1, 0)); bfn.push_back(-1); }
         brk.push_back(make_int4((int)b, K, (int)boff, bfirst));
         boff += (size_t)SC::PASSES * (K / 16) * SC::AU;
+        t.oz_wide |= K > 256;
         if (K > OZ_MAXK || goff >= (1ull << 31) || boff >= (1ull << 31) || prow * CW >= (1L << 31)) return HUB_OK;
     }
     // on a device without room for both layouts the point-major form does all products
@@ -1051,7 +1090,7 @@ int gather_oz(hub_t h, const void* X, int ncol, int ld, int spin, bool want_W) {
     Table& t = h->proj;
     int rc;
     if ((rc = launch_colmax(h, X, ncol, ld))) return rc;
-    if ((rc = ensure(h, &h->d_part, &h->part_bytes, std::max(h->part_bytes, (size_t)t.oz_npart * CW * ncol * sizeof(double))))) return rc;
+    if ((rc = ensure(h, &h->d_part, &h->part_bytes, std::max(h->part_bytes, (size_t)t.oz_npart * CW * C::PARTS * ncol * sizeof(double))))) return rc;
     if ((rc = ensure(h, &h->d_C, &h->C_bytes, std::max(h->C_bytes, (size_t)t.nproj * ncol * CW * sizeof(double))))) return rc;
     if ((rc = ensure(h, &h->d_W, &h->W_bytes, std::max(h->W_bytes, (size_t)t.nproj * ncol * CW * sizeof(R))))) return rc;
     if ((rc = ensure(h, (void**)&h->d_wmax, &h->wmax_bytes, std::max(h->wmax_bytes, (size_t)ncol * sizeof(int))))) return rc;
@@ -1068,8 +1107,9 @@ int gather_oz(hub_t h, const void* X, int ncol, int ld, int spin, bool want_W) {
     a.ncol = ncol;
     a.nbx = t.nbx; a.nby = t.nby;
     a.ctiles = (ncol + OZ_M - 1) / OZ_M;
-    if ((long)t.oz_ngroups * a.ctiles > 0x7fffffffL / C::SLICES) return fail(h, HUB_EINVAL, "gather: too many tiles");
-    a.nunits = t.oz_ngroups * a.ctiles;
+    if ((long)t.oz_ngroups * C::PARTS * a.ctiles > 0x7fffffffL / C::SLICES) return fail(h, HUB_EINVAL, "gather: too many tiles");
+    a.nunits = t.oz_ngroups * C::PARTS * a.ctiles;
+    a.part_rows = t.oz_npart * CW;
     // 16-byte copies need whole pieces within a row and 16-byte row starts
     a.vec = h->n1 % C::PPP == 0 && ((size_t)a.ld * sizeof(R)) % 16 == 0 && (uintptr_t)X % 16 == 0;
     a.flags = h->d_flags;
@@ -1094,6 +1134,7 @@ int gather_oz(hub_t h, const void* X, int ncol, int ld, int spin, bool want_W) {
     r.X = X;
     r.idx = t.d_idx;
     r.vals = t.d_vals;
+    r.part_rows = t.oz_npart * CW;
     r.ld = ld;
     r.dV = h->dV;
     r.ncol = ncol;
@@ -1135,9 +1176,17 @@ int scatter_oz(hub_t h, void* Y, int ncol, int ld, double alpha, const double* a
     a.ctiles = (ncol + C::NT - 1) / C::NT;
     a.flags = h->d_flags;
     const int npair = t.oz_nbricks * C::PASSES;
-    HUB_CUDA_TRY(h, cudaFuncSetAttribute(k_scatter_oz<R, CW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM));
-    ProfScope ps(h, HUB_K_SCATTER);
-    k_scatter_oz<R, CW><<<std::max(1, std::min(npair, h->num_sms)), C::THREADS, C::SMEM, h->stream>>>(a);
+    auto run = [&](auto kernel) -> int {
+        HUB_CUDA_TRY(h, cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM));
+        ProfScope ps(h, HUB_K_SCATTER);
+        kernel<<<std::max(1, std::min(npair, h->num_sms)), C::THREADS, C::SMEM, h->stream>>>(a);
+        return HUB_OK;
+    };
+    if constexpr (C::S == 7) {
+        if ((rc = t.oz_wide ? run(k_scatter_oz<R, CW, true>) : run(k_scatter_oz<R, CW, false>))) return rc;
+    } else {
+        if ((rc = run(k_scatter_oz<R, CW, false>))) return rc;
+    }
     HUB_CUDA_TRY(h, cudaGetLastError());
     return HUB_OK;
 }
@@ -1165,7 +1214,8 @@ bool gather_digits(hub_t h, int ncol) {
     const double c = d ? (h->cplx ? 7.1e-6 : 1.96e-6) : (h->cplx ? 5.5e-7 : 1.7e-7);
     const double plain = t.nvals * (c * ncol + (h->cplx ? 8e-6 : 4e-6)) + 10.0;
     // digits: full tiles and the last one
-    const double rounds = (double)((t.oz_ngroups + h->num_sms - 1) / h->num_sms) * 16 * cw;
+    const int parts = d ? cw : 1;
+    const double rounds = (double)((t.oz_ngroups * parts + h->num_sms - 1) / h->num_sms) * 16 * cw / parts;
     const int last = ncol - ncol / OZ_M * OZ_M;
     const double full = d ? 1.04 : 0.88, part = d ? 0.60 + 0.44 * last / OZ_M : 0.42 + 0.46 * last / OZ_M;
     const double digits = rounds * (ncol / OZ_M * full + (last ? part : 0.0));
