@@ -38,8 +38,8 @@ template <> struct Digits<double> {
     static constexpr I kZero = 0x80808080808080ull;
     static __device__ __forceinline__ int exponent(double v) { return (__double2hiint(v) >> 20) & 0x7ff; }
     // integer with the digits as its bytes (offset by 128 each), for a value of biased exponent
-    // e = exponent(v) + de in a group whose largest is E (E >= e, E >= kEmin; a zero or denormal
-    // v shifts to zero, whatever its hidden bit)
+    // e = exponent(v) + de in a group whose largest is E (E >= e, E >= kEmin).  With de = 0 a zero or
+    // denormal v shifts to zero whatever its hidden bit; with another de the caller leaves it out
     static __device__ __forceinline__ I bytes(double v, int E, int de = 0) {
         const unsigned hi = (unsigned)__double2hiint(v), lo = (unsigned)__double2loint(v);
         const int sh = min(E - de - ((int)(hi >> 20) & 0x7ff), 63);

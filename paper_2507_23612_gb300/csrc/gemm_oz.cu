@@ -404,7 +404,8 @@ k_digits_q(const double* __restrict__ Q, int k, int n, int ct, const unsigned* _
             const int c = 8 * u + i;
             const double q = c < k && col < n ? Q[(size_t)c * n + col] : 0.0;
             const int E = c < k ? column_exponent<R>(cmax, c) : 0;
-            const unsigned long long w = q != 0.0 && E > 0 && top > 0 ? Digits<double>::bytes(q, top, E) : Digits<double>::kZero;
+            const unsigned long long w = Digits<double>::exponent(q) > 0 && E > 0 && top > 0 ?    // a denormal q has no part in top
+                                              Digits<double>::bytes(q, top, E) : Digits<double>::kZero;
             if constexpr (S == 7) b[i] = w;
             else b[i] = (unsigned)(((long long)(w - Digits<double>::kZero) + (1 << 23)) >> 24) + Digits<float>::kZero;
         }

@@ -777,7 +777,8 @@ k_scatter_oz(OzScatter a) {
                         de[2 * k + 1] = q4.w - Digits<R>::kBias;
                     }
 #pragma unroll
-                    for (int k = 0; k < 8; ++k) v[it][k] = x[k] != R(0) ? Digits<R>::bytes(x[k], E, de[k]) : Digits<R>::kZero;
+                    for (int k = 0; k < 8; ++k)      // denormal coefficients are zero: they have no part in the maximum
+                        v[it][k] = Digits<R>::exponent(x[k]) > 0 ? Digits<R>::bytes(x[k], E, de[k]) : Digits<R>::kZero;
                 }
                 const bool ok = i < C::NB || mbar_wait(&wempty_bar[s], ((i / C::NB) - 1) & 1, &abort_flag);
                 if (__any_sync(0xffffffffu, !ok)) { stop = true; break; }
@@ -841,7 +842,7 @@ k_scatter_oz(OzScatter a) {
                             long long lo;
                             const long long hi = level_sum<R, F>(v + f, &lo);
                             if constexpr (S == 7) {
-                                // (hi 2^24 + lo) 256^6 with the low 10 bits rounded off; at least 2^-800 or zero
+                                // (hi 2^24 + lo) 256^6 with the low 10 bits rounded off; zero or at least 2^-948
                                 const double r = (double)((hi << 14) + ((lo + 512) >> 10));
                                 const int up = (10 + 48 + Ef + Digits<R>::kBias - 2 * Digits<R>::kUnit) << 20;
                                 yv[o0 + f] = fma(alpha, r == 0.0 ? r : __hiloint2double(__double2hiint(r) + up, __double2loint(r)),
