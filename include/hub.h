@@ -120,6 +120,18 @@ int hub_num_hubbard_atoms(hub_t h, int* nhub);
  * that spin (Eq. DerED; coefficient of phi_m' is sum_m M_m'm <phi_m|psi>). */
 int hub_set_occupation_matrix(hub_t h, int spin, const double* D_re, const double* D_im);
 
+/* Device memory.  Besides its tables a handle holds workspaces that grow with the largest block it
+ * has seen, and memory that only makes products faster: the projectors' values a second and a third
+ * time as digits (FP64 and complex handles; some 0.8 GB for 72 atoms on 88 x 88 x 84 points in FP64,
+ * 1 GB for 48 at a Bloch point) and up to 2 GB of digits per Gram product or rotation of a real
+ * block.  Where there is no room for these, or where room is needed for something else, the products
+ * take slower forms that do without.
+ * hub_set_memory_limit: the workspaces and digits together may take this many bytes (0, the default:
+ * what the device has).  What is held already stays.  A call whose workspace does not fit in any
+ * form returns HUB_ENOMEM.  hub_memory_held: the bytes they take now.  Errors: HUB_EINVAL. */
+int hub_set_memory_limit(hub_t h, long long bytes);
+int hub_memory_held(hub_t h, long long* bytes);
+
 /* Mixed handles (HUB_MIXED_BF16, HUB_MIXED_F16): how the Rayleigh-Ritz block products
  * are taken.  t16 is the handle's 16-bit type (BF16: 8 significand bits; FP16: 11, after
  * the power-of-two scaling of each operand block described at HUB_MIXED_F16).

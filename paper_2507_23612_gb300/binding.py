@@ -68,6 +68,8 @@ _SIGS = {
     "hub_scf_density": [_P, _P],
     "hub_scf_set_density": [_P, _P],
     "hub_num_projectors": [_P, _PI],
+    "hub_set_memory_limit": [_P, C.c_longlong],
+    "hub_memory_held": [_P, C.POINTER(C.c_longlong)],
     "hub_project": [_P, _P, _I, _I, _PD],
     "hub_expand": [_P, _PD, _I, _P, _I, _D],
     "hub_scf_forces": [_P, _PD, _PD],
@@ -246,6 +248,14 @@ class Hub:
     # ------------------------------------------------------------------ setup
     def set_bf16_terms(self, terms: int):
         self._check(self.lib.hub_set_bf16_terms(self.h, int(terms)), "hub_set_bf16_terms")
+
+    def set_memory_limit(self, nbytes: int):
+        self._check(self.lib.hub_set_memory_limit(self.h, nbytes), "hub_set_memory_limit")
+
+    def memory_held(self) -> int:
+        n = C.c_longlong()
+        self._check(self.lib.hub_memory_held(self.h, C.byref(n)), "hub_memory_held")
+        return n.value
 
     def set_veff(self, veff):
         import torch

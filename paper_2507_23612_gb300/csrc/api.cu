@@ -17,23 +17,83 @@ int fail(hub_t h, int code, const std::string& msg) {
     return code;
 }
 
+bool device_alloc(hub_t h, void** p, size_t bytes) {
+    *p = nullptr;
+    if (h->mem_limit > 0 && h->mem_held + bytes > h->mem_limit) return false;
+    if (cudaMalloc(p, bytes) != cudaSuccess) {
+        cudaGetLastError();               // the failed allocation's, which later launches would report
+        *p = nullptr;
+        return false;
+    }
+    h->mem_held += bytes;
+    return true;
+}
+
+void device_free(hub_t h, void** p, size_t bytes) {
+    if (!*p) return;
+    cudaFree(*p);
+    *p = nullptr;
+    h->mem_held -= bytes;
+}
+
+// What only makes products faster: the digit tables of the projectors and the digits of Gram products
+// and rotations (on mixed handles that buffer holds operands of the 16-bit products too)
+static bool give_back(hub_t h, void** but) {
+    if (h->capturing) return false;
+    const size_t held = h->mem_held;
+    cudaStreamSynchronize(h->stream);     // the digits may be in use
+    free_oz(h, h->proj);
+    if (but != &h->d_bf16 && !tensor_mixed_prec(h)) {
+        device_free(h, &h->d_bf16, h->bf16_bytes);
+        h->bf16_bytes = 0;
+    }
+    h->mem_gen++;
+    return h->mem_held < held;
+}
+
+int table_alloc(hub_t h, void** p, size_t bytes) {
+    cudaError_t e = cudaMalloc(p, bytes);
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        if (give_back(h, nullptr)) e = cudaMalloc(p, bytes);
+    }
+    if (e == cudaSuccess) return HUB_OK;
+    cudaGetLastError();
+    *p = nullptr;
+    return fail(h, HUB_ENOMEM, "no device memory for projector tables");
+}
+
 int ensure(hub_t h, void** p, size_t* have, size_t need) {
     if (*have >= need && *p) return HUB_OK;
     h->mem_gen++;
     if (*p) {
         cudaStreamSynchronize(h->stream);
-        cudaFree(*p);
-        *p = nullptr;
+        device_free(h, p, *have);
         *have = 0;
     }
     if (need == 0) return HUB_OK;
-    cudaError_t e = cudaMalloc(p, need);
-    if (e != cudaSuccess) {
-        *p = nullptr;
-        return fail(h, HUB_ENOMEM, std::string("cudaMalloc of workspace failed: ") + cudaGetErrorString(e));
-    }
+    if (!device_alloc(h, p, need) && !(give_back(h, p) && device_alloc(h, p, need)))
+        return fail(h, HUB_ENOMEM, "no device memory for a workspace of " + std::to_string(need) + " bytes");
     *have = need;
     return HUB_OK;
+}
+
+bool claim(hub_t h, void** p, size_t* have, size_t need) {
+    if (*have >= need && *p) return true;
+    if (h->capturing || need >= h->refused) return false;
+    void* q;
+    if (!device_alloc(h, &q, need)) {
+        h->refused = need;
+        return false;
+    }
+    if (*p) {
+        cudaStreamSynchronize(h->stream);
+        device_free(h, p, *have);
+    }
+    *p = q;
+    *have = need;
+    h->mem_gen++;
+    return true;
 }
 
 int check_flags(hub_t h) {
@@ -78,8 +138,9 @@ static void fd_gradient_weights(hub_t h, double w[3][kMaxHalf]) {
 int apply_H_internal(hub_t h, int spin, const void* X, int ld, void* Y, int ncol, double alpha,
                      double shift, const void* Yprev, double beta, const double* coef_dev) {
     int rc;
+    bool digits = false;
     if (h->proj.nsites > 0)
-        if ((rc = launch_gather(h, X, ncol, ld, spin, true))) return rc;
+        if ((rc = launch_gather(h, X, ncol, ld, spin, true, &digits))) return rc;
     StencilArgs a{};
     a.Y = X;
     a.Yprev = Yprev;
@@ -105,10 +166,10 @@ int apply_H_internal(hub_t h, int spin, const void* X, int ld, void* Y, int ncol
     a.shift = shift;
     a.beta = beta;
     a.coef = coef_dev;
-    a.cmax_ready = h->proj.nsites > 0 && gather_digits(h, ncol);
+    a.cmax_ready = digits;
     if ((rc = launch_stencil(h, a))) return rc;
     if (h->proj.nsites > 0)
-        if ((rc = launch_scatter(h, Y, ncol, ld, alpha, coef_dev))) return rc;
+        if ((rc = launch_scatter(h, Y, ncol, ld, alpha, coef_dev, digits))) return rc;
     return HUB_OK;
 }
 
@@ -205,6 +266,7 @@ int hub_destroy(hub_t h) {
     if (!h) return HUB_OK;
     cudaStreamSynchronize(h->stream);
     for (auto& e : h->prof) { cudaEventDestroy(e.a); cudaEventDestroy(e.b); }
+    free_oz(h, h->proj);
     free_table(h->proj);
     void* ptrs[] = {h->d_veff, h->d_work, h->d_work2, h->d_part, h->d_C, h->d_W, h->d_small,
                     h->d_gpart, h->d_bf16, h->d_aux, h->d_flags, h->d_bar, h->d_scal, h->d_tcmax, h->d_cmax, h->d_wmax, h->d_dens,
@@ -288,6 +350,20 @@ int hub_set_occupation_matrix(hub_t h, int spin, const double* D_re, const doubl
                                     cudaMemcpyHostToDevice, h->stream));
     HUB_CUDA_TRY(h, cudaStreamSynchronize(h->stream));
     h->D_set[spin] = true;
+    return HUB_OK;
+}
+
+int hub_set_memory_limit(hub_t h, long long bytes) {
+    if (!h) return HUB_EINVAL;
+    if (bytes < 0) return fail(h, HUB_EINVAL, "negative memory limit");
+    h->mem_limit = (size_t)bytes;
+    h->refused = ~(size_t)0;
+    return HUB_OK;
+}
+
+int hub_memory_held(hub_t h, long long* bytes) {
+    if (!h || !bytes) return HUB_EINVAL;
+    *bytes = (long long)h->mem_held;
     return HUB_OK;
 }
 
@@ -530,7 +606,7 @@ int hub_expand(hub_t h, const double* W_host, int ncol, void* Y, int ld, double 
         HUB_CUDA_TRY(h, cudaMemcpyAsync(h->d_W, wf.data(), n * sizeof(float), cudaMemcpyHostToDevice, h->stream));
         HUB_CUDA_TRY(h, cudaStreamSynchronize(h->stream));     // wf goes out of scope
     }
-    return launch_scatter(h, Y, ncol, ld, alpha, nullptr, false);
+    return launch_scatter(h, Y, ncol, ld, alpha);
 }
 
 int hub_hubbard_forces(hub_t h, int spin, const void* X, int ncol, int ld, const double* f_host,
@@ -810,8 +886,7 @@ static int density_setup(hub_t h, ScfState& st) {
         st.hist_r[i] = v; v += ns * Nd;
     }
     for (int s = 0; s < ns; ++s)
-        if (!h->d_veff_spin[s])
-            HUB_CUDA_TRY(h, cudaMalloc(&h->d_veff_spin[s], veff_bytes(h)));
+        if ((rc = ensure(h, &h->d_veff_spin[s], &h->veff_spin_bytes[s], veff_bytes(h)))) return rc;
     const double vol = h->dV * (double)h->Nd;
     for (int s = 0; s < ns; ++s)
         if ((rc = density_fill(h, st.rho_in[s], st.p.n_elec / ns / vol))) return rc;

@@ -110,6 +110,15 @@ void filter_coefficients(int degree, double a, double b, double a_low, double* o
 
 using namespace hub;
 
+// the tuning of a batched system; memory that it took from the digit tables changes the forms of the
+// products, whose workspaces have to be there before the capture
+static int tune_and_settle(hub_t h, int spin, void* X, int ld, int ncol) {
+    const bool digits = h->proj.oz != 0;
+    int rc = hub_autotune(h, spin, X, ncol, ld, nullptr);
+    if (!rc && digits && !h->proj.oz) rc = apply_H_internal(h, spin, X, ld, h->d_work, ncol, 1.0, 0.0, nullptr, 0.0);
+    return rc;
+}
+
 #define BATCH_TRY(expr)                                                                    \
     do {                                                                                   \
         cudaError_t _e = (expr);                                                           \
@@ -326,7 +335,7 @@ int hub_batch_filter(int nsys, const hub_t* sys, const int* spin, void* const* X
             // may skip the autotuner's own application for shapes seen before)
             if ((rc = ensure(h, &h->d_work, &h->work_bytes, std::max(h->work_bytes, (size_t)ld[i] * ncol[i] * es))) ||
                 (rc = apply_H_internal(h, spin[i], X[i], ld[i], h->d_work, ncol[i], 1.0, 0.0, nullptr, 0.0)) ||
-                (rc = hub_autotune(h, spin[i], X[i], ncol[i], ld[i], nullptr))) {
+                (rc = tune_and_settle(h, spin[i], X[i], ld[i], ncol[i]))) {
                 if (h != sys[0]) sys[0]->last_error = "system " + std::to_string(i) + ": " + h->last_error;
                 return rc;
             }

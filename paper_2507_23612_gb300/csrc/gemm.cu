@@ -403,13 +403,8 @@ static bool gram_digits(hub_t h) {
 static bool rotate_digits(hub_t h, int k, int n) {
     return !h->cplx && h->Nd <= (1L << 25) && (h->esize == 8 || (k > 128 && (double)k * n * h->Nd >= 1.5e9));
 }
-// The digits take up to 2 GB of workspace, claimed before the first launch: on a full device the
-// product is left to the CUDA cores, which need little.
-static bool no_memory(int rc) {
-    if (rc != HUB_ENOMEM) return false;
-    cudaGetLastError();               // the failed allocation's, which later launches would report
-    return true;
-}
+// The digits take up to 2 GB of workspace, claimed before the first launch, or less where there is not
+// that much: without room (HUB_ENOMEM) the product is left to the CUDA cores, which need little.
 
 int launch_gram(hub_t h, const void* A, int lda, const void* B, int ldb, int m, int n,
                 double alpha, bool sym, double* G) {
@@ -420,7 +415,7 @@ int launch_gram(hub_t h, const void* A, int lda, const void* B, int ldb, int m, 
     }
     if (gram_digits(h)) {
         const int rc = launch_gram_oz(h, A, lda, B, ldb, m, n, alpha, sym, G);
-        if (!no_memory(rc)) return rc;
+        if (rc != HUB_ENOMEM) return rc;
     }
     if (h->esize == 8) return gram_t<double>(h, A, lda, B, ldb, m, n, alpha, sym, G);
     if (lda % 4 == 0 && ldb % 4 == 0 && (uintptr_t)A % 16 == 0 && (uintptr_t)B % 16 == 0)
@@ -432,7 +427,7 @@ int launch_rotate(hub_t h, const void* X, int ldx, const double* Q, int k, int n
     if (n == 0) return HUB_OK;
     if (rotate_digits(h, k, n)) {
         const int rc = launch_rotate_oz(h, X, ldx, Q, k, n, Y, ldy);
-        if (!no_memory(rc)) return rc;
+        if (rc != HUB_ENOMEM) return rc;
     }
     dim3 grid((unsigned)((h->Nd + BM - 1) / BM), (n + BN - 1) / BN);
     ProfScope ps(h, HUB_K_ROTATE);

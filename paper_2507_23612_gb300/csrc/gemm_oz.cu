@@ -42,6 +42,7 @@ namespace {
 constexpr int MZ_M = 128, MZ_N = 64;
 constexpr int MZ_THREADS = 320;
 constexpr size_t MZ_PANEL = (size_t)1 << 30;        // bytes of one operand's digits per panel
+constexpr size_t MZ_LEAST = (size_t)1 << 24;
 
 template <typename R>
 struct MCfg {
@@ -478,10 +479,19 @@ k_gram_oz_reduce(const longlong2* __restrict__ part, int tiles, int splits, int 
 }
 
 // ---------------------------------------------------------------------------- host
+// room for the digits of `per` steps or, where there is less, of fewer (panels of 8 MB are the least
+// that are tried)
+bool claim_panel(hub_t h, long& per, size_t step, size_t fixed) {
+    while (!claim(h, &h->d_bf16, &h->bf16_bytes, (size_t)per * step + fixed)) {
+        if (per == 1 || (size_t)per * step < MZ_LEAST) return false;
+        per = (per + 1) / 2;
+    }
+    return true;
+}
+
 template <typename R>
 int gram_oz(hub_t h, const void* A, int lda, const void* B, int ldb, int m, int n, double alpha, bool sym, double* G) {
     using C = MCfg<R>;
-    constexpr int S = C::S;
     int rc;
     const long Nd = h->Nd;
     const bool same = A == B && lda == ldb && m == n;
@@ -492,13 +502,11 @@ int gram_oz(hub_t h, const void* A, int lda, const void* B, int ldb, int m, int 
     // panels of whole 16-point steps
     const size_t stepA = (size_t)rt * C::AB, stepB = (size_t)ct * C::BB;
     const long steps = (Nd + 15) / 16;
-    const long per = std::max<long>(1, std::min<long>(steps, (long)(MZ_PANEL / std::max(stepA, stepB))));
+    long per = std::max<long>(1, std::min<long>(steps, (long)(MZ_PANEL / std::max(stepA, stepB))));
     // column maxima: A's, then B's
-    const size_t cm = (size_t)(m + n) * kColParts * sizeof(unsigned);
-    if ((rc = ensure(h, (void**)&h->d_cmax, &h->cmax_bytes, std::max(h->cmax_bytes, cm)))) return rc;
-    const size_t npart = (size_t)splits * tiles * MZ_M * MZ_N * sizeof(longlong2);
-    if ((rc = ensure(h, &h->d_gpart, &h->gpart_bytes, std::max(h->gpart_bytes, npart)))) return rc;
-    if ((rc = ensure(h, &h->d_bf16, &h->bf16_bytes, std::max(h->bf16_bytes, (size_t)per * (stepA + stepB))))) return rc;
+    if (!claim(h, (void**)&h->d_cmax, &h->cmax_bytes, (size_t)(m + n) * kColParts * sizeof(unsigned)) ||
+        !claim(h, &h->d_gpart, &h->gpart_bytes, (size_t)splits * tiles * MZ_M * MZ_N * sizeof(longlong2)) ||
+        !claim_panel(h, per, stepA + stepB, 0)) return HUB_ENOMEM;
     unsigned* cmB = h->d_cmax + (same ? 0 : (size_t)m * kColParts);
     if ((rc = launch_colmax(h, A, m, lda))) return rc;
     if (!same && (rc = launch_colmax_at(h, B, n, ldb, cmB))) return rc;
@@ -539,7 +547,6 @@ int gram_oz(hub_t h, const void* A, int lda, const void* B, int ldb, int m, int 
     k_gram_oz_reduce<R><<<(unsigned)(((long)m * n + 31) / 32), 256, 0, h->stream>>>(
         a.part, tiles, splits, ct, sym, m, n, alpha, h->d_cmax, cmB, (const R*)A, lda, (const R*)B, ldb, Nd, G);
     HUB_CUDA_TRY(h, cudaGetLastError());
-    (void)S;
     return HUB_OK;
 }
 
@@ -551,9 +558,10 @@ int rotate_oz(hub_t h, const void* X, int ldx, const double* Q, int k, int n, vo
     const int ct = (n + MZ_N - 1) / MZ_N, ks = (k + 15) / 16;
     const size_t perTile = (size_t)ks * C::AB, nB = (size_t)ks * ct * C::BB;
     const long tilesAll = (Nd + MZ_M - 1) / MZ_M;
-    const long per = std::max<long>(1, std::min<long>(tilesAll, (long)(MZ_PANEL / perTile)));
+    long per = std::max<long>(1, std::min<long>(tilesAll, (long)(MZ_PANEL / perTile)));
     const size_t nE = ((size_t)(n + 1) * sizeof(int) + 255) / 256 * 256;
-    if ((rc = ensure(h, &h->d_bf16, &h->bf16_bytes, std::max(h->bf16_bytes, (size_t)per * perTile + nB + nE)))) return rc;
+    if (!claim(h, (void**)&h->d_cmax, &h->cmax_bytes, (size_t)k * kColParts * sizeof(unsigned)) ||
+        !claim_panel(h, per, perTile, nB + nE)) return HUB_ENOMEM;
     if ((rc = launch_colmax(h, X, k, ldx))) return rc;
     uint4* dA = (uint4*)h->d_bf16;
     uint4* dB = dA + (size_t)per * perTile / 16;

@@ -101,6 +101,7 @@ struct Table {
     int oz = 0;                       // 1 when the arrays below are built
     int oz_ngroups = 0, oz_nbricks = 0;
     bool oz_wide = false;             // a brick has more than 256 slots
+    size_t oz_bytes = 0;              // of the arrays below
     long oz_npart = 0;                // (function, brick) pairs: partial rows of the gather
     int4* d_ozg = nullptr;            // per group: brick, slots, 16-byte offset of its values, first slot
     int2* d_ozg_row = nullptr;        // per slot: partial row (x slots per function; -1 padding), exponent
@@ -159,6 +160,9 @@ struct hub_ctx {
     int gather_dense = 0;         // real float: gather in the brick form (else point-major)
     int gemm_split = 2;           // tensor-core split-K: CTAs per SM of the Gram products
     int capturing = 0;            // work is being captured into a CUDA graph
+    size_t mem_limit = 0;         // of mem_held (0: none)
+    size_t mem_held = 0;          // bytes of the workspaces and of the digit tables
+    size_t refused = ~(size_t)0;  // smallest optional workspace that was refused (claim)
     long long mem_gen = 0;        // bumped whenever a workspace or table is reallocated
     cudaStream_t stream = nullptr;
     int device = 0;
@@ -185,6 +189,7 @@ struct hub_ctx {
     // density SCF: per-spin V_eff in the working type (used by apply_H when veff_per_spin),
     // and the double buffers of the density model (V_loc, rho, V_H, v_x, Pulay history)
     void* d_veff_spin[2] = {nullptr, nullptr};
+    size_t veff_spin_bytes[2] = {0, 0};
     int veff_per_spin = 0;
     double* d_rho_ws = nullptr;   size_t rho_ws_bytes = 0;
     double* d_vloc = nullptr;     size_t vloc_bytes = 0;    // double copy of the set V_eff
@@ -227,7 +232,18 @@ struct ProfScope {
         h->prof.push_back(ProfEvt{kind, a, b});
     }
 };
+// Device memory of a workspace or of the digit tables: false past the handle's limit or without room
+bool device_alloc(hub_t h, void** p, size_t bytes);
+void device_free(hub_t h, void** p, size_t bytes);
+// Device memory of the tables themselves, which are not counted
+int table_alloc(hub_t h, void** p, size_t bytes);
+// A workspace that a product cannot do without: where there is no room, the memory that only makes
+// products faster is given back first
 int ensure(hub_t h, void** p, size_t* have, size_t need);
+// ... or that a faster form wants: the buffer at hand stays where there is no room for a larger one,
+// and that size is not tried again (until the tables or the limit are set anew).  No allocation
+// during capture, so a captured call takes the form of the call before.
+bool claim(hub_t h, void** p, size_t* have, size_t need);
 
 // An NVTX range around one ABI call (visible to Nsight tools; without a tool attached the
 // calls return at once; compiled out where the toolkit has no NVTX headers)
@@ -306,11 +322,12 @@ int build_tables(hub_t h, int natoms, const double* pos, const int* kb_nchan, co
 void free_table(Table& t);
 // C[P x ncol] (double, x2 complex) = dV * <proj_p|x_n>; with want_W also W = transform(C)
 // in the working type (gamma .* C for KB rows, M_spin C for Hubbard rows).
-int launch_gather(hub_t h, const void* X, int ncol, int ld, int spin, bool want_W);
+// *digits: the digit form ran (d_cmax holds the column maxima of X and d_wmax those of W)
+int launch_gather(hub_t h, const void* X, int ncol, int ld, int spin, bool want_W, bool* digits = nullptr);
 // Y[g, n] += alpha * sum_e vals_e . W[rows_e, n]   (W from the last launch_gather); with
-// alpha_dev != nullptr alpha is read on the device
+// alpha_dev != nullptr alpha is read on the device; wmax_ready: d_wmax holds the maxima of this W
 int launch_scatter(hub_t h, void* Y, int ncol, int ld, double alpha, const double* alpha_dev = nullptr,
-                   bool w_from_gather = true);
+                   bool wmax_ready = false);
 // D per Hubbard atom (double, [nhub*50] re/im pairs) and E_U into d_scal[0] from the C of
 // the last launch_gather; f_dev [ncol] double.
 int launch_occupation(hub_t h, int ncol, const double* f_dev, double kweight, double* D_dev);
@@ -329,8 +346,10 @@ int launch_scatter_tc(hub_t h, void* Y, int ncol, int ld, double alpha, const do
 
 // projectors_oz.cu: digit form of the gather and scatter; launch_gather and launch_scatter take it
 // where these say so.  site_pts: grid points of each site, ascending
+// (and their workspace could be claimed)
 bool gather_digits(hub_t h, int ncol);
-bool scatter_digits(hub_t h, int ncol);
+bool scatter_digits(hub_t h, int ncol, bool wmax_ready);
+void free_oz(hub_t h, Table& t);
 int build_oz_tables(hub_t h, Table& t, const std::vector<std::vector<int>>& site_pts);
 int launch_gather_oz(hub_t h, const void* X, int ncol, int ld, int spin, bool want_W);
 // wmax_ready: d_wmax holds the maxima of W (both written by launch_gather_oz)
@@ -353,16 +372,16 @@ int launch_gram(hub_t h, const void* A, int lda, const void* B, int ldb, int m, 
 // Y[K x n] = X[K x k] Q[k x n]; Q double column-major [k x n] (ldq = k)
 int launch_rotate(hub_t h, const void* X, int ldx, const double* Q, int k, int n, void* Y,
                   int ldy);
-// gemm_oz.cu: the same for real blocks as exact digit products on the tensor cores
+// gemm_oz.cu: the same for real blocks as digit products on the tensor cores; HUB_ENOMEM, before any
+// launch, where there is no room for the digits
 int launch_gram_oz(hub_t h, const void* A, int lda, const void* B, int ldb, int m, int n,
                    double alpha, bool sym, double* G);
 int launch_rotate_oz(hub_t h, const void* X, int ldx, const double* Q, int k, int n, void* Y, int ldy);
 // mixed-precision variants (tcgen05 path; 16-bit operand type from h->prec)
 // true when the Rayleigh-Ritz block products of this handle run on the tensor cores: a mixed
 // handle (BF16 or FP16 operands), real blocks, and a product form with 1 or 3 terms
-inline bool tensor_mixed(const hub_ctx* h) {
-    return (h->prec == HUB_MIXED_BF16 || h->prec == HUB_MIXED_F16) && h->bf16_terms > 0 && !h->cplx;
-}
+inline bool tensor_mixed_prec(const hub_ctx* h) { return h->prec == HUB_MIXED_BF16 || h->prec == HUB_MIXED_F16; }
+inline bool tensor_mixed(const hub_ctx* h) { return tensor_mixed_prec(h) && h->bf16_terms > 0 && !h->cplx; }
 int launch_gram_bf16(hub_t h, const void* A, int lda, const void* B, int ldb, int m, int n,
                      double alpha, bool sym, double* G);
 int launch_rotate_bf16(hub_t h, const void* X, int ldx, const double* Q, int k, int n,

@@ -733,7 +733,8 @@ template <typename Tp>
 int upload(hub_t h, Tp** dptr, const std::vector<Tp>& v) {
     if (*dptr) { cudaFree(*dptr); *dptr = nullptr; }
     if (v.empty()) return HUB_OK;
-    HUB_CUDA_TRY(h, cudaMalloc((void**)dptr, v.size() * sizeof(Tp)));
+    const int rc = table_alloc(h, (void**)dptr, v.size() * sizeof(Tp));
+    if (rc) return rc;
     HUB_CUDA_TRY(h, cudaMemcpy(*dptr, v.data(), v.size() * sizeof(Tp), cudaMemcpyHostToDevice));
     return HUB_OK;
 }
@@ -747,8 +748,7 @@ void free_table(Table& t) {
                     t.d_csr_ent, t.d_order, t.d_gamma, t.d_hub_sites, t.d_U,
                     t.d_M[0], t.d_M[1], t.d_bent, t.d_bfirst, t.d_phi, t.d_frow, t.d_roff,
                     t.d_rent, t.d_tcg, t.d_tcg_row, t.d_tchi, t.d_tclo, t.d_tcs_brick, t.d_tcs_frow, t.d_tcs_hi,
-                    t.d_tcs_lo, t.d_ozg, t.d_ozg_row, t.d_ozg_val, t.d_ozb, t.d_ozb_row, t.d_ozb_val, t.d_oz_exp,
-                    t.d_oz_roff, t.d_oz_rent};
+                    t.d_tcs_lo};
     for (void* p : ptrs)
         if (p) cudaFree(p);
     t = Table();
@@ -1030,7 +1030,7 @@ int build_tables(hub_t h, int natoms, const double* pos, const int* kb_nchan, co
     if ((rc = upload(h, &t.d_U, t.h_U))) return rc;
     const size_t vbytes = (size_t)t.nvals * h->esize * (h->cplx ? 2 : 1);
     if (vbytes) {
-        HUB_CUDA_TRY(h, cudaMalloc(&t.d_vals, vbytes));
+        if ((rc = table_alloc(h, &t.d_vals, vbytes))) return rc;
         dim3 grid(t.nitems);
         const double* kp = h->kpt;
         ProfScope ps(h, HUB_K_TABLE);
@@ -1051,13 +1051,15 @@ int build_tables(hub_t h, int natoms, const double* pos, const int* kb_nchan, co
         HUB_CUDA_TRY(h, cudaStreamSynchronize(h->stream));     // values are ready
         if ((rc = build_bricks(h, t, site_pts))) return rc;
     }
+    h->refused = ~(size_t)0;
     if (!t.dense && t.nsites > 0) {
-        HUB_CUDA_TRY(h, cudaStreamSynchronize(h->stream));     // values are ready
+        HUB_CUDA_TRY(h, cudaStreamSynchronize(h->stream));     // values are ready, the old digits not in use
+        free_oz(h, h->proj);                                   // one set of digits at a time
         if ((rc = build_oz_tables(h, t, site_pts))) return rc;
     }
     const size_t mbytes = (size_t)std::max(t.nhub, 1) * 25 * sizeof(double) * (h->cplx ? 2 : 1);
     for (int s = 0; s < 2; ++s) {
-        HUB_CUDA_TRY(h, cudaMalloc((void**)&t.d_M[s], mbytes));
+        if ((rc = table_alloc(h, (void**)&t.d_M[s], mbytes))) return rc;
         HUB_CUDA_TRY(h, cudaMemsetAsync(t.d_M[s], 0, mbytes, h->stream));
     }
     // the D = 0 coefficients M = (U/2) I
@@ -1070,6 +1072,7 @@ int build_tables(hub_t h, int natoms, const double* pos, const int* kb_nchan, co
         HUB_CUDA_TRY(h, cudaStreamSynchronize(h->stream));
         t.h_M[s] = M;                  // host copy of the coefficients in use
     }
+    free_oz(h, h->proj);
     free_table(h->proj);
     h->proj = std::move(t);
     h->mem_gen++;
@@ -1080,8 +1083,6 @@ static int gather_dense(hub_t h, const void* X, int ncol, int ld, int spin, bool
     Table& t = h->proj;
     int rc;
     if ((rc = ensure(h, &h->d_part, &h->part_bytes, (size_t)t.npart_rows * ncol * sizeof(float)))) return rc;
-    if ((rc = ensure(h, &h->d_C, &h->C_bytes, (size_t)t.nproj * ncol * sizeof(double)))) return rc;
-    if ((rc = ensure(h, &h->d_W, &h->W_bytes, (size_t)t.nproj * ncol * sizeof(float)))) return rc;
     if (h->gather_dense >= 2 && t.tc) {
         if ((rc = launch_gather_tc(h, X, ncol, ld))) return rc;
     } else {
@@ -1130,8 +1131,6 @@ static int gather_t(hub_t h, const void* X, int ncol, int ld, int spin, bool wan
     Table& t = h->proj;
     int rc;
     if ((rc = ensure(h, &h->d_part, &h->part_bytes, (size_t)t.nitems * kMaxProj * ncol * sizeof(D)))) return rc;
-    if ((rc = ensure(h, &h->d_C, &h->C_bytes, (size_t)t.nproj * ncol * sizeof(D)))) return rc;
-    if ((rc = ensure(h, &h->d_W, &h->W_bytes, (size_t)t.nproj * ncol * sizeof(T)))) return rc;
     // columns per warp (the value table is re-read once per column group): 16 bytes of each
     // point's row, except complex float, which takes four columns (32 bytes) with two points
     // per lane and iteration (rutile, 348 columns: 4.28 -> 2.66 ms; eight columns 2.58 ms at
@@ -1156,9 +1155,17 @@ static int gather_t(hub_t h, const void* X, int ncol, int ld, int spin, bool wan
     return HUB_OK;
 }
 
-int launch_gather(hub_t h, const void* X, int ncol, int ld, int spin, bool want_W) {
+int launch_gather(hub_t h, const void* X, int ncol, int ld, int spin, bool want_W, bool* digits) {
+    if (digits) *digits = false;
     if (ncol == 0 || h->proj.nsites == 0) return HUB_OK;
-    if (gather_digits(h, ncol)) return launch_gather_oz(h, X, ncol, ld, spin, want_W);
+    const size_t rows = (size_t)h->proj.nproj * ncol * (h->cplx ? 2 : 1);
+    int rc;
+    if ((rc = ensure(h, &h->d_C, &h->C_bytes, std::max(h->C_bytes, rows * sizeof(double))))) return rc;
+    if ((rc = ensure(h, &h->d_W, &h->W_bytes, std::max(h->W_bytes, rows * h->esize)))) return rc;
+    if (gather_digits(h, ncol)) {
+        if (digits) *digits = true;
+        return launch_gather_oz(h, X, ncol, ld, spin, want_W);
+    }
     if (h->gather_dense && use_dense(h, X, ld)) return gather_dense(h, X, ncol, ld, spin, want_W);
     if (h->esize == 8) return h->cplx ? gather_t<double, true>(h, X, ncol, ld, spin, want_W)
                                       : gather_t<double, false>(h, X, ncol, ld, spin, want_W);
@@ -1181,10 +1188,9 @@ static int scatter_t(hub_t h, void* Y, int ncol, int ld, double alpha, const dou
     return HUB_OK;
 }
 
-int launch_scatter(hub_t h, void* Y, int ncol, int ld, double alpha, const double* alpha_dev, bool w_from_gather) {
+int launch_scatter(hub_t h, void* Y, int ncol, int ld, double alpha, const double* alpha_dev, bool wmax_ready) {
     if (ncol == 0 || h->proj.nsites == 0) return HUB_OK;
-    if (scatter_digits(h, ncol))
-        return launch_scatter_oz(h, Y, ncol, ld, alpha, alpha_dev, w_from_gather && gather_digits(h, ncol));
+    if (scatter_digits(h, ncol, wmax_ready)) return launch_scatter_oz(h, Y, ncol, ld, alpha, alpha_dev, wmax_ready);
     if (use_dense(h, Y, ld)) {
         if (h->gather_dense == 3 && h->proj.tc) return launch_scatter_tc(h, Y, ncol, ld, alpha, alpha_dev);
         return scatter_dense(h, Y, ncol, ld, alpha, alpha_dev);

@@ -957,11 +957,13 @@ __global__ void k_oz_slots(int n, int cw, const int* __restrict__ exps, int2* __
     if (i < n) slots[i].y = fn[i] >= 0 ? exps[fn[i]] : 0;
 }
 
+// a device copy of v, counted in bytes: false without room
 template <typename Tp>
-int put(hub_t h, Tp** d, const std::vector<Tp>& v) {
-    HUB_CUDA_TRY(h, cudaMalloc((void**)d, std::max<size_t>(v.size(), 1) * sizeof(Tp)));
-    if (!v.empty()) HUB_CUDA_TRY(h, cudaMemcpy(*d, v.data(), v.size() * sizeof(Tp), cudaMemcpyHostToDevice));
-    return HUB_OK;
+bool put(hub_t h, Tp** d, const std::vector<Tp>& v, size_t* bytes) {
+    const size_t n = std::max<size_t>(v.size(), 1) * sizeof(Tp);
+    if (!device_alloc(h, (void**)d, n)) return false;
+    *bytes += n;
+    return v.empty() || cudaMemcpy(*d, v.data(), v.size() * sizeof(Tp), cudaMemcpyHostToDevice) == cudaSuccess;
 }
 
 template <typename R, int CW>
@@ -1047,22 +1049,24 @@ int build_oz(hub_t h, Table& t, const std::vector<std::vector<int>>& site_pts) {
         if (K > OZ_MAXK || goff >= (1ull << 31) || boff >= (1ull << 31) || prow * CW >= (1L << 31)) return HUB_OK;
     }
     // on a device without room for both layouts the point-major form does all products
-    if (cudaMalloc((void**)&t.d_ozg_val, goff * 16) != cudaSuccess || cudaMalloc((void**)&t.d_ozb_val, boff * 16) != cudaSuccess) {
-        cudaGetLastError();
-        cudaFree(t.d_ozg_val);
-        t.d_ozg_val = nullptr;
-        return HUB_OK;
-    }
-    int rc;
+    size_t tmp = 0;
     int *d_row_pair = nullptr, *d_gfn = nullptr, *d_bfn = nullptr;
     int4* d_pairs = nullptr;
-    if ((rc = put(h, &t.d_ozg, grp)) || (rc = put(h, &t.d_ozg_row, gslot)) || (rc = put(h, &t.d_ozb, brk)) ||
-        (rc = put(h, &t.d_ozb_row, bslot)) || (rc = put(h, &t.d_oz_roff, roff)) || (rc = put(h, &t.d_oz_rent, rent))) return rc;
-    HUB_CUDA_TRY(h, cudaMalloc((void**)&t.d_oz_exp, std::max(t.nproj, 1) * sizeof(int)));
-    HUB_CUDA_TRY(h, cudaMemsetAsync(t.d_ozg_val, 0, goff * 16, h->stream));
-    HUB_CUDA_TRY(h, cudaMemsetAsync(t.d_ozb_val, 0, boff * 16, h->stream));
-    if (!(rc = put(h, &d_row_pair, row_pair)) && !(rc = put(h, &d_pairs, pairs)) && !(rc = put(h, &d_gfn, gfn)) &&
-        !(rc = put(h, &d_bfn, bfn))) {
+    auto room = [&](void** p, size_t n) {
+        if (!device_alloc(h, p, n)) return false;
+        t.oz_bytes += n;
+        return true;
+    };
+    const bool ok = room((void**)&t.d_ozg_val, goff * 16) && room((void**)&t.d_ozb_val, boff * 16) &&
+                    room((void**)&t.d_oz_exp, std::max(t.nproj, 1) * sizeof(int)) && put(h, &t.d_ozg, grp, &t.oz_bytes) &&
+                    put(h, &t.d_ozg_row, gslot, &t.oz_bytes) && put(h, &t.d_ozb, brk, &t.oz_bytes) &&
+                    put(h, &t.d_ozb_row, bslot, &t.oz_bytes) && put(h, &t.d_oz_roff, roff, &t.oz_bytes) &&
+                    put(h, &t.d_oz_rent, rent, &t.oz_bytes) && put(h, &d_row_pair, row_pair, &tmp) &&
+                    put(h, &d_pairs, pairs, &tmp) && put(h, &d_gfn, gfn, &tmp) && put(h, &d_bfn, bfn, &tmp);
+    cudaError_t e = cudaGetLastError(), es = cudaSuccess;
+    if (ok) {
+        cudaMemsetAsync(t.d_ozg_val, 0, goff * 16, h->stream);
+        cudaMemsetAsync(t.d_ozb_val, 0, boff * 16, h->stream);
         ProfScope ps(h, HUB_K_TABLE);
         const R* vals = (const R*)t.d_vals;
         k_oz_exponents<R, CW><<<t.nsites, 256, 0, h->stream>>>(t.d_sites, vals, t.d_oz_exp);
@@ -1071,13 +1075,16 @@ int build_oz(hub_t h, Table& t, const std::vector<std::vector<int>>& site_pts) {
         k_oz_fill<R, CW><<<t.nitems, 256, 0, h->stream>>>(t.d_items, t.d_sites, t.d_idx, vals, t.d_oz_exp, d_row_pair, d_pairs,
                                                           t.d_ozg, t.d_ozb, n1, n2, (unsigned short*)t.d_ozg_val,
                                                           (unsigned short*)t.d_ozb_val);
+        e = cudaGetLastError();
+        es = cudaStreamSynchronize(h->stream);
     }
-    const cudaError_t e = cudaGetLastError(), es = cudaStreamSynchronize(h->stream);
     for (void* p : {(void*)d_row_pair, (void*)d_pairs, (void*)d_gfn, (void*)d_bfn})
         if (p) cudaFree(p);
-    if (rc) return rc;
+    h->mem_held -= tmp;
+    if (!ok) free_oz(h, t);
     HUB_CUDA_TRY(h, e);
     HUB_CUDA_TRY(h, es);
+    if (!ok) return HUB_OK;
     t.oz_ngroups = (int)grp.size();
     t.oz_nbricks = (int)brk.size();
     t.oz_npart = prow;
@@ -1091,10 +1098,6 @@ int gather_oz(hub_t h, const void* X, int ncol, int ld, int spin, bool want_W) {
     Table& t = h->proj;
     int rc;
     if ((rc = launch_colmax(h, X, ncol, ld))) return rc;
-    if ((rc = ensure(h, &h->d_part, &h->part_bytes, std::max(h->part_bytes, (size_t)t.oz_npart * CW * C::PARTS * ncol * sizeof(double))))) return rc;
-    if ((rc = ensure(h, &h->d_C, &h->C_bytes, std::max(h->C_bytes, (size_t)t.nproj * ncol * CW * sizeof(double))))) return rc;
-    if ((rc = ensure(h, &h->d_W, &h->W_bytes, std::max(h->W_bytes, (size_t)t.nproj * ncol * CW * sizeof(R))))) return rc;
-    if ((rc = ensure(h, (void**)&h->d_wmax, &h->wmax_bytes, std::max(h->wmax_bytes, (size_t)ncol * sizeof(int))))) return rc;
     OzGather a{};
     a.X = X;
     a.grp = t.d_ozg;
@@ -1108,7 +1111,6 @@ int gather_oz(hub_t h, const void* X, int ncol, int ld, int spin, bool want_W) {
     a.ncol = ncol;
     a.nbx = t.nbx; a.nby = t.nby;
     a.ctiles = (ncol + OZ_M - 1) / OZ_M;
-    if ((long)t.oz_ngroups * C::PARTS * a.ctiles > 0x7fffffffL / C::SLICES) return fail(h, HUB_EINVAL, "gather: too many tiles");
     a.nunits = t.oz_ngroups * C::PARTS * a.ctiles;
     a.part_rows = t.oz_npart * CW;
     // 16-byte copies need whole pieces within a row and 16-byte row starts
@@ -1152,7 +1154,6 @@ int scatter_oz(hub_t h, void* Y, int ncol, int ld, double alpha, const double* a
     Table& t = h->proj;
     int rc;
     if (!wmax_ready) {
-        if ((rc = ensure(h, (void**)&h->d_wmax, &h->wmax_bytes, std::max(h->wmax_bytes, (size_t)ncol * sizeof(int))))) return rc;
         ProfScope ps(h, HUB_K_SCATTER);
         k_wmax_oz<R, CW><<<(ncol + 31) / 32, 256, 0, h->stream>>>((const R*)h->d_W, t.d_oz_exp, t.nproj, ncol, h->d_wmax);
         HUB_CUDA_TRY(h, cudaGetLastError());
@@ -1194,6 +1195,20 @@ int scatter_oz(hub_t h, void* Y, int ncol, int ld, double alpha, const double* a
 
 }  // namespace
 
+void free_oz(hub_t h, Table& t) {
+    for (void* p : {(void*)t.d_ozg, (void*)t.d_ozg_row, (void*)t.d_ozg_val, (void*)t.d_ozb, (void*)t.d_ozb_row, (void*)t.d_ozb_val,
+                    (void*)t.d_oz_exp, (void*)t.d_oz_roff, (void*)t.d_oz_rent})
+        if (p) cudaFree(p);
+    t.d_ozg = t.d_ozb = nullptr;
+    t.d_ozg_row = t.d_ozb_row = nullptr;
+    t.d_ozg_val = t.d_ozb_val = nullptr;
+    t.d_oz_exp = t.d_oz_roff = t.d_oz_rent = nullptr;
+    h->mem_held -= t.oz_bytes;
+    t.oz_bytes = 0;
+    if (t.oz) h->mem_gen++;
+    t.oz = 0;
+}
+
 int build_oz_tables(hub_t h, Table& t, const std::vector<std::vector<int>>& site_pts) {
     if (t.nsites == 0) return HUB_OK;
     if (h->esize == 8) return h->cplx ? build_oz<double, 2>(h, t, site_pts) : build_oz<double, 1>(h, t, site_pts);
@@ -1220,10 +1235,14 @@ bool gather_digits(hub_t h, int ncol) {
     const int last = ncol - ncol / OZ_M * OZ_M;
     const double full = d ? 1.04 : 0.88, part = d ? 0.60 + 0.44 * last / OZ_M : 0.42 + 0.46 * last / OZ_M;
     const double digits = rounds * (ncol / OZ_M * full + (last ? part : 0.0));
-    return digits < plain;
+    if (digits >= plain || (long)t.oz_ngroups * parts * (ncol / OZ_M + 1) > 0x7fffffffL / 64) return false;
+    // the gather's workspace (the point-major form takes over without it)
+    return claim(h, (void**)&h->d_cmax, &h->cmax_bytes, (size_t)ncol * kColParts * sizeof(unsigned)) &&
+           claim(h, (void**)&h->d_wmax, &h->wmax_bytes, (size_t)ncol * sizeof(int)) &&
+           claim(h, &h->d_part, &h->part_bytes, (size_t)t.oz_npart * cw * parts * ncol * sizeof(double));
 }
 
-bool scatter_digits(hub_t h, int ncol) {
+bool scatter_digits(hub_t h, int ncol, bool wmax_ready) {
     const Table& t = h->proj;
     if (!t.oz) return false;
     const bool d = h->esize == 8;
@@ -1232,7 +1251,7 @@ bool scatter_digits(hub_t h, int ncol) {
                            : (h->cplx ? 6.8e-7 : 3.7e-7) * t.nvals * std::max(ncol, 12);
     const long pairs = (long)t.oz_nbricks * cw;
     const double digits = (double)((pairs + h->num_sms - 1) / h->num_sms) * ((ncol + nt - 1) / nt) * (d ? 4.2 : 5.5) + 12.0;
-    return digits < plain + 10.0;
+    return digits < plain + 10.0 && (wmax_ready || claim(h, (void**)&h->d_wmax, &h->wmax_bytes, (size_t)ncol * sizeof(int)));
 }
 
 int launch_gather_oz(hub_t h, const void* X, int ncol, int ld, int spin, bool want_W) {
