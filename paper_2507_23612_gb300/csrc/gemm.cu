@@ -390,21 +390,34 @@ int gram_t(hub_t h, const void* A, int lda, const void* B, int ldb, int m, int n
 }  // namespace
 
 // Real blocks as digit products on the tensor cores (gemm_oz.cu; complex blocks stay here).  The
-// digit sums hold 2^25 grid points.  Doubles always: the Gram product is level with the FP64 pipe at
-// 14^3 x 6 (54 us) and ahead from there on (88x88x84 x 348, symmetric: 83.0 -> 3.6 ms; the rotation
-// 140.4 -> 4.0).  Floats: the conversions have to be earned.  The Gram product is ahead from some
-// thousand points on (14^3 x 24: 23 against 29 us; 24^3 x 24: 63 against 33; 88x88x84 x 348: 4.4
-// against 1.9 ms), the rotation only over many columns (with its conversions, 88x88x84 x 96: 0.49
-// against 0.75 ms, x 130: 1.06 against 1.0, x 348: 5.1 against 2.2; 28x30x56 x 130: 0.09 against
-// 0.10, x 200: 0.16 against 0.13).
-static bool gram_digits(hub_t h) {
-    return !h->cplx && h->Nd <= (1L << 25) && (h->esize == 8 || h->Nd >= 8192);
+// digit sums hold 2^25 grid points.  Doubles always, 88x88x84 x 348: symmetric Gram product 83.0 -> 4.5
+// ms, rotation 140.4 -> 5.0 ms (and 1 column 1.28 -> 0.60 ms, 14^3 x 8: 58 -> 35 us, 4^3 x 2: 53 -> 41).
+// The digits take up to 2 GB of workspace, claimed before the first launch, or less where there is not
+// that much: without room (HUB_ENOMEM) the product is left to the CUDA cores, which need little.
+//
+// Floats: the conversions have to be earned.  Their cost goes by whole tiles of 128 and 64 columns (0.5
+// to 0.7 ns a point for one), so that a few columns of a large grid, which fill one tile of the
+// CUDA-core form and are read in 0.2 ns a point, stay there (gram_f32x8; microseconds, CUDA cores
+// against digits, A^T A / A^T B):
+//   1 column     24^3  40 / 40   44 / 55     60x60x64  148 / 148  149 / 163    88x88x84 221 / 221  350 / 385
+//   2 columns    72^3 279 / 279 224 / 243    88x88x84  331 / 330  352 / 388    100^3   385 / 386  514 / 562
+//   8 columns    72^3 356 / 355 222 / 244    88x88x84  407 / 406  356 / 396    100^3   468 / 466  523 / 577
+//   64 columns   72^3 428 / 501 251 / 312    88x88x84  563 / 595  405 / 500    100^3   673 / 703  594 / 727
+//   65 columns   24^3 112 /  96  46 /  56    88x88x84  691 / 744  490 / 596    160^3 x 96: 3870 / 5470, 3090 / 4300
+// The rotation takes them over many columns only (with its conversions, 88x88x84 x 96: 0.49 against
+// 0.75 ms, x 130: 1.06 against 1.0, x 348: 5.1 against 2.2; 28x30x56 x 130: 0.09 against 0.10, x 200:
+// 0.16 against 0.13).
+static bool gram_digits(hub_t h, int m, int n, bool f32x8) {
+    if (h->cplx || h->Nd > (1L << 25)) return false;
+    if (h->esize == 8) return true;
+    const int c = std::max(m, n);
+    if (!f32x8 || c > 64) return h->Nd >= 8192;
+    if (c == 1) return h->Nd >= 20000 && h->Nd <= 200000;
+    return h->Nd >= 8192 && h->Nd <= (c < 4 ? 480000 : 700000);
 }
 static bool rotate_digits(hub_t h, int k, int n) {
     return !h->cplx && h->Nd <= (1L << 25) && (h->esize == 8 || (k > 128 && (double)k * n * h->Nd >= 1.5e9));
 }
-// The digits take up to 2 GB of workspace, claimed before the first launch, or less where there is not
-// that much: without room (HUB_ENOMEM) the product is left to the CUDA cores, which need little.
 
 int launch_gram(hub_t h, const void* A, int lda, const void* B, int ldb, int m, int n,
                 double alpha, bool sym, double* G) {
@@ -413,12 +426,13 @@ int launch_gram(hub_t h, const void* A, int lda, const void* B, int ldb, int m, 
         if (h->esize == 8) return gram_t<double2>(h, A, lda, B, ldb, m, n, alpha, sym, G);
         return gram_t<float2>(h, A, lda, B, ldb, m, n, alpha, sym, G);
     }
-    if (gram_digits(h)) {
+    const bool f32x8 = h->esize == 4 && lda % 4 == 0 && ldb % 4 == 0 && (uintptr_t)A % 16 == 0 && (uintptr_t)B % 16 == 0;
+    if (gram_digits(h, m, n, f32x8)) {
         const int rc = launch_gram_oz(h, A, lda, B, ldb, m, n, alpha, sym, G);
         if (rc != HUB_ENOMEM) return rc;
     }
     if (h->esize == 8) return gram_t<double>(h, A, lda, B, ldb, m, n, alpha, sym, G);
-    if (lda % 4 == 0 && ldb % 4 == 0 && (uintptr_t)A % 16 == 0 && (uintptr_t)B % 16 == 0)
+    if (f32x8)
         return gram_f32x8(h, (const float*)A, lda, (const float*)B, ldb, m, n, alpha, sym, G);
     return gram_t<float>(h, A, lda, B, ldb, m, n, alpha, sym, G);
 }
