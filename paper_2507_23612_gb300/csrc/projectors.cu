@@ -924,6 +924,7 @@ int build_tables(hub_t h, int natoms, const double* pos, const int* kb_nchan, co
                             if (hi[ax] < lo[ax]) empty = true;
                         }
                         if (empty) continue;
+                        const size_t before = pts.size();
                         bool any = false;
                         for (int k3 = lo[2]; k3 <= hi[2]; ++k3) {
                             const double dz = k3 * h->h[2] - c[2];
@@ -938,13 +939,15 @@ int build_tables(hub_t h, int natoms, const double* pos, const int* kb_nchan, co
                                 }
                             }
                         }
+                        // ascending within an image; images are merged
+                        if (before > 0 && pts.size() > before && pts[before] <= pts[before - 1])
+                            std::inplace_merge(pts.begin(), pts.begin() + before, pts.end());
                         if (any)
                             for (int ax = 0; ax < 3; ++ax) {
                                 tmin[ax] = std::min(tmin[ax], tt[ax]);
                                 tmax[ax] = std::max(tmax[ax], tt[ax]);
                             }
                     }
-            std::sort(pts.begin(), pts.end());
             pts.erase(std::unique(pts.begin(), pts.end()), pts.end());
             if (pts.empty()) continue;   // cannot happen for rc > 0 and a grid inside the cell
             for (int ax = 0; ax < 3; ++ax) { S.tlo[ax] = tmin[ax]; S.thi[ax] = tmax[ax]; }

@@ -982,15 +982,17 @@ int build_oz(hub_t h, Table& t, const std::vector<std::vector<int>>& site_pts) {
     std::vector<int> row_pair(t.npts), stamp(nb, -1), count(nb + 1, 0);
     for (int s = 0; s < t.nsites; ++s) {
         const int first = (int)pl.size();
-        int yz = -1, by = 0;
-        long zb = 0;
-        int r = t.h_sites[s].pt_off;
+        int r = t.h_sites[s].pt_off, pair = 0;
+        long end = -1;                               // of the run of points in this row and brick
         for (int g : site_pts[s]) {
-            const int q = g / n1, x = g - q * n1;
-            if (q != yz) { yz = q; by = (q % n2) / BRY; zb = (long)t.nby * (q / n2 / BRZ); }
-            const long b = x / BRX + t.nbx * (by + zb);
-            if (stamp[b] < first) { stamp[b] = (int)pl.size(); pl.push_back({s, (int)b}); count[b + 1]++; }
-            row_pair[r++] = stamp[b];
+            if (g >= end) {
+                const int q = g / n1, x = g - q * n1;
+                const long b = x / BRX + t.nbx * ((q % n2) / BRY + (long)t.nby * (q / n2 / BRZ));
+                if (stamp[b] < first) { stamp[b] = (int)pl.size(); pl.push_back({s, (int)b}); count[b + 1]++; }
+                pair = stamp[b];
+                end = (long)q * n1 + std::min(n1, (x / BRX + 1) * BRX);
+            }
+            row_pair[r++] = pair;
         }
     }
     for (long b = 0; b < nb; ++b) count[b + 1] += count[b];
