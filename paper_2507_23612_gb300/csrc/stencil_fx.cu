@@ -325,7 +325,9 @@ k_stencil_fx(const __grid_constant__ FxArgs a) {
 #pragma unroll
         for (int r = 0; r < ROWS; ++r) {
             const int2 c = q[r][FXH];
-            long long M3 = 1 << 25;
+            long long M3 = 1 << 29;                    // the low limbs' product, then the mixed ones
+            mad(M3, c.y, vc[r].y);
+            M3 = (M3 >> 30) + (1 << 25);
             mad(M3, c.x, vc[r].y);
             mad(M3, c.y, vc[r].x);
             const long long Z = H[r] + (M1[r] >> 30) + (M2[r] >> 31) + (((long long)c.x * vc[r].x) << 4) + (M3 >> 26);

@@ -90,3 +90,15 @@ def test_potential_keeps_its_bits(h):
     lam = float(largest_kinetic(n, L))
     for y in apply(n, L, veff, x):
         assert np.all(np.abs(y - veff) <= 2.0 ** -53 * (lam + np.abs(veff)))
+
+
+@pytest.mark.parametrize("h", [0.3, 1.0, 4.1, 12.9])
+def test_products_with_the_potential_keep_their_bits(h):
+    """x = 1/3 everywhere, whose low limb is not zero: H x = V / 3, to one rounding at 2^-53 of the row sum."""
+    n = (12, 14, 10)
+    L = tuple(h * m for m in n)
+    x = np.full(n[0] * n[1] * n[2], 1.0 / 3.0)
+    veff = np.random.default_rng(4).uniform(-0.9, 0.9, x.size)
+    lam = float(largest_kinetic(n, L))
+    for y in apply(n, L, veff, x):
+        assert np.all(np.abs(y - veff * x) <= 2.0 ** -53 * (lam + np.abs(veff)) * x)
