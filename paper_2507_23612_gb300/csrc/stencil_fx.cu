@@ -59,7 +59,7 @@ struct FxArgs {
     int tx, ty, tilesx, tiles;    // tile shape and count
     int zchunk, nzc;
     int k[FXH + 1];               // integer weights, k[0] the centre
-    double F[3];
+    double F[3], Flo[3];          // F = F + Flo
     double alpha, beta, shift;
     const double* coef;           // device {alpha, beta, shift} or nullptr
     double w[3][FXH], cen;        // FP64 weights (alpha = 1) of the slow form
@@ -112,6 +112,9 @@ __device__ __noinline__ double fx_slow(const FxArgs& a, const double* __restrict
     return dot;
 }
 
+// 2^k, |k| < 1023 (scalbn's cases cost a small grid's launch 5 us)
+__device__ __forceinline__ double pow2(int k) { return __hiloint2double((k + 1023) << 20, 0); }
+
 __device__ __forceinline__ void mad(long long& acc, int s, int w) { acc += (long long)s * w; }
 
 // the product for a conjugate-gradient step: dot[1] = sum, dot[0] = dot[2], dot[6] = dot[0] / dot[1] or 0
@@ -148,19 +151,19 @@ k_stencil_fx(const __grid_constant__ FxArgs a) {
 
     const int emax = (int)(column_max(a.cmax, col) >> 20), e20 = emax << 20;
     const int sf = a.vinfo[2];
-    const bool fits = fabs(shift) < scalbn(1.0, 83 - sf);       // NaN: false
+    const bool fits = fabs(shift) < pow2(83 - sf);              // NaN: false
     if (emax < kFxEmin || emax > kFxEmax || !fits || a.vinfo[1]) {    // the same for the whole CTA
         const double sum = fx_slow(a, Y, Yp, Yo, gx0, gy0, z0, z1, alpha, beta, shift);
         if constexpr (DOT) finish_dot(a, sum);
         return;
     }
-    const double scale = scalbn(alpha, 81 - sf + emax - 1081);
-    const long long shq = __double2ll_rn(scalbn(shift, sf - 25));
+    const double scale = alpha * pow2(81 - sf + emax - 1081);
+    const long long shq = __double2ll_rn(shift * pow2(sf - 25));
     const int shh = (int)(shq >> 30), shl = (int)(shq & 0x3fffffff);
     int fh[3], fl[3];                             // F 2^sf as limbs of 30 bits
 #pragma unroll
     for (int ax = 0; ax < 3; ++ax) {
-        const long long fq = __double2ll_rn(scalbn(a.F[ax], sf));
+        const long long fq = __double2ll_rn(a.F[ax] * pow2(sf)) + __double2ll_rn(a.Flo[ax] * pow2(sf));
         fh[ax] = (int)(fq >> 30);
         fl[ax] = (int)(fq & 0x3fffffff);
     }
@@ -434,7 +437,13 @@ static int run_fx(hub_t h, const StencilArgs& s, int variant, const StencilDot* 
     double wb = 0.0;
     for (int p = 0; p <= FXH; ++p) a.k[p] = f.k[p];
     for (int ax = 0; ax < 3; ++ax) {
-        a.F[ax] = -0.5 / (f.lcd * h->h[ax] * h->h[ax]);
+        // to more than 53 bits: a rounding at 2^-53 is one and the same error of the kinetic energy at every
+        // point, where the rounded weights of the FP64 form average out
+        const int n = ax == 0 ? h->n1 : ax == 1 ? h->n2 : h->n3;
+        const long double ih = (long double)n / (long double)h->L[ax];
+        const long double F = -0.5L * ih * ih / f.lcd;
+        a.F[ax] = (double)F;
+        a.Flo[ax] = (double)(F - a.F[ax]);
         for (int p = 0; p < FXH; ++p) {
             a.w[ax][p] = p < s.n0 ? s.wbase[ax][p] : 0.0;
             wb += a.w[ax][p];

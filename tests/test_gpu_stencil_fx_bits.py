@@ -1,6 +1,9 @@
 """How many bits the fixed-point stencil keeps: elements are rounded to nearest (2^-59 of the column's
 maximum), and the Laplacian's factors keep theirs on grids of any spacing.  Alternating signs add
 every point's error up: H x = lambda x with lambda the largest kinetic energy."""
+import math
+from fractions import Fraction
+
 import numpy as np
 import pytest
 
@@ -102,3 +105,25 @@ def test_products_with_the_potential_keep_their_bits(h):
     lam = float(largest_kinetic(n, L))
     for y in apply(n, L, veff, x):
         assert np.all(np.abs(y - veff * x) <= 2.0 ** -53 * (lam + np.abs(veff)) * x)
+
+
+@pytest.mark.parametrize("h", [(0.36, 0.36, 0.36), (0.1973, 0.1973, 0.1973), (0.6, 0.7, 0.8)])
+def test_factors_do_not_shift_the_kinetic_energy(h):
+    """256 amplitudes of the alternating column: the roundings of the results average to 2^-58 of lambda
+    (2^-54.3 / 16), an error of the factors stays: at most 2^-55 together.  (The sum of the weights of
+    order 12 that alternate, 4 sum over odd p, exactly.)"""
+    n = (12, 14, 10)
+    L = tuple(h[a] * n[a] for a in range(3))
+    hb = Hub(n, L, 6, prec=HUB_F64)
+    hb.set_veff(torch.zeros(12 * 14 * 10, dtype=torch.float64, device="cuda"))
+    hb.set_atoms([])
+    amp = np.random.default_rng(6).uniform(1.0, 2.0, 256)
+    X = torch.tensor(amp[:, None] * alternating(n)[None], device="cuda")
+    Y = torch.empty_like(X)
+    hb.apply_H(0, X, Y)
+    x, y = X.cpu().numpy().astype(np.longdouble), Y.cpu().numpy().astype(np.longdouble)
+    f = math.factorial
+    odd = sum(Fraction(2 * f(6) ** 2, p * p * f(6 - p) * f(6 + p)) for p in (1, 3, 5))
+    lam = sum(np.longdouble(2) * np.longdouble(odd.numerator) / np.longdouble(odd.denominator) *
+              (np.longdouble(n[a]) / np.longdouble(L[a])) ** 2 for a in range(3))
+    assert abs(float(np.mean(y / x) / lam - 1)) <= 2.0 ** -55
