@@ -20,7 +20,8 @@
 // 2^-32 of the largest product; 2^-40 with 5 levels).
 //
 // The bits are relative to the largest magnitude of the group: a number 2^-k of it has k bits
-// fewer, down to none, where a floating-point operand would keep all of its own.
+// fewer, down to none, where a floating-point operand would keep all of its own.  So groups are
+// small where the results are local: the values of X around a brick (gather).
 #pragma once
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>

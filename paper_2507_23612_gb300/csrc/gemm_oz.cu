@@ -508,7 +508,7 @@ int gram_oz(hub_t h, const void* A, int lda, const void* B, int ldb, int m, int 
         !claim(h, &h->d_gpart, &h->gpart_bytes, (size_t)splits * tiles * MZ_M * MZ_N * sizeof(longlong2)) ||
         !claim_panel(h, per, stepA + stepB, 0)) return HUB_ENOMEM;
     unsigned* cmB = h->d_cmax + (same ? 0 : (size_t)m * kColParts);
-    if ((rc = launch_colmax(h, A, m, lda))) return rc;
+    if ((rc = launch_colmax_at(h, A, m, lda, h->d_cmax))) return rc;
     if (!same && (rc = launch_colmax_at(h, B, n, ldb, cmB))) return rc;
     uint4* dA = (uint4*)h->d_bf16;
     uint4* dB = dA + (size_t)per * stepA / 16;
@@ -562,7 +562,7 @@ int rotate_oz(hub_t h, const void* X, int ldx, const double* Q, int k, int n, vo
     const size_t nE = ((size_t)(n + 1) * sizeof(int) + 255) / 256 * 256;
     if (!claim(h, (void**)&h->d_cmax, &h->cmax_bytes, (size_t)k * kColParts * sizeof(unsigned)) ||
         !claim_panel(h, per, perTile, nB + nE)) return HUB_ENOMEM;
-    if ((rc = launch_colmax(h, X, k, ldx))) return rc;
+    if ((rc = launch_colmax_at(h, X, k, ldx, h->d_cmax))) return rc;
     uint4* dA = (uint4*)h->d_bf16;
     uint4* dB = dA + (size_t)per * perTile / 16;
     int* esc = (int*)((char*)dB + nB);

@@ -278,16 +278,25 @@ struct StencilArgs {
     int n0;
     double phase[3][2];     // exp(i k_a L_a) (re, im), complex only
     const double* coef;     // device {alpha, beta, shift} or nullptr (then w/center/alpha/beta)
-    bool cmax_ready;        // d_cmax holds the column maxima of Y
+    bool cmax_ready;        // d_cmax holds the maxima of Y (launch_colmax)
     double wbase[3][kMaxHalf];  // (-1/2) c_p / h_a^2 (alpha = 1)
 };
 int launch_stencil(hub_t h, const StencilArgs& a);
 int stencil_variants(hub_t h);
-// colmax.cu: h->d_cmax[col * kColParts + i], the largest leading word of |x| over slice i of
-// each column (biased exponent on top)
+// colmax.cu: d_cmax[col * kColParts + i], the largest leading word of |x| over z part i of each column
+// (biased exponent on top), and behind the ncol columns of a launch_colmax the pieces of 32 x 8 points
+// (2^xlog x 2^ylog on planes of millions of points) of every part: [col][part][y >> ylog][x >> xlog]
 constexpr int kColParts = 8;
+constexpr int kColPieces = 12000;     // per part at most
+struct BlockMap {
+    const unsigned* m;
+    int nbx, nby, zper;           // pieces along x and y, planes per part
+    int xlog, ylog;
+};
+BlockMap block_map(const hub_ctx* h, const unsigned* cmax, int ncol);
+size_t colmax_bytes(const hub_ctx* h, int ncol);
 int launch_colmax(hub_t h, const void* X, int ncol, int ld);
-int launch_colmax_at(hub_t h, const void* X, int ncol, int ld, unsigned* cmax);   // into cmax
+int launch_colmax_at(hub_t h, const void* X, int ncol, int ld, unsigned* cmax);   // into cmax, columns alone
 #ifdef __CUDACC__
 __device__ __forceinline__ unsigned column_max(const unsigned* cmax, int col) {
     unsigned m = 0;
@@ -295,11 +304,19 @@ __device__ __forceinline__ unsigned column_max(const unsigned* cmax, int col) {
     for (int i = 0; i < kColParts; ++i) m = max(m, cmax[(size_t)col * kColParts + i]);
     return m;
 }
+// of the pieces that the brick of 8 x 8 x 4 points at x, y, z (multiples of these) lies in
+__device__ __forceinline__ unsigned brick_max(const BlockMap& b, int col, int x, int y, int z, int n3) {
+    const int nblk = b.nbx * b.nby, p0 = z / b.zper, end = min(z + 4, n3);
+    const unsigned* m = b.m + ((size_t)col * kColParts + p0) * nblk + (y >> b.ylog) * b.nbx + (x >> b.xlog);
+    unsigned v = *m;
+    for (int e = (p0 + 1) * b.zper; e < end; e += b.zper) v = max(v, *(m += nblk));
+    return v;
+}
 #endif
 // stencil_fx.cu: the real FP64 stencil in fixed point.  A potential of Nd doubles is followed
 // by its fixed-point form (fx_veff_bytes bytes), written by launch_fx_veff
 int launch_stencil_fx(hub_t h, const StencilArgs& a);
-// ... of one column without Yprev, on a handle of any type, with d_cmax set: dot[0] = dot[2], dot[1] = sum
+// ... of one column without Yprev, on a handle of any type, with the column's d_cmax set: dot[0] = dot[2], dot[1] = sum
 // of Y * Yout, dot[6] = dot[0] / dot[1] (0 unless dot[1] > 0); part: one double per CTA (at most one per
 // 32 points of a row), counter: zero
 struct StencilDot {

@@ -115,13 +115,24 @@ struct OzGather {
     const int2* slot;         // partial row (-1: padding), exponent of the function
     const uint4* val;
     double* part;
-    const unsigned* cmax;
+    BlockMap bmax;            // maxima of X
     int* wmax;                // cleared for the reduction
     long part_rows;           // rows of one part of the bricks
     long ld;                  // in reals
     int n1, n2, n3, ncol, nbx, nby, nunits, ctiles, vec;
     int* flags;
 };
+
+// scale of a column's digits on a brick: the largest exponent of the pieces around it, at least the
+// smallest of the format; a brick with non-finite or larger values has zero digits (its column is
+// summed in the reduction)
+template <typename R, int CW>
+__device__ __forceinline__ int oz_exponent(const OzGather& a, int x, int y, int z, int col) {
+    if (col >= a.ncol) return 1 << 14;
+    const unsigned m = brick_max(a.bmax, col, x, y, z, a.n3);
+    const int E = max((int)(m >> (sizeof(R) == 8 ? 20 : 23)), Digits<R>::kEmin);
+    return E > Digits<R>::kEmax ? 1 << 14 : E;
+}
 
 template <typename R, int CW>
 __global__ void __launch_bounds__(OZ_GTHREADS, 1)
@@ -258,6 +269,9 @@ k_gather_oz(OzGather a) {
         int gx = 0, gy = 0, gz = 0;                      // brick corner
         int chunk0 = 0;                                  // first chunk of the unit's part of the brick
         bool more = false;                               // the warp has orbitals in this unit
+        int E = 0, Enext = 0;                            // exponent of this lane's orbital: of the unit converted and of the
+                                                         // one whose copies begin (ND slices ahead, within the unit)
+        static_assert(C::SLICES / OZ_SETS >= C::ND, "one unit ahead at most");
         auto issue = [&](int j) {                        // the set's j-th slice
             const int i = set + OZ_SETS * j, nq = i % C::SLICES;
             if (i < nsl) {
@@ -269,6 +283,7 @@ k_gather_oz(OzGather a) {
                     gy = 8 * ((brick / a.nbx) % a.nby);
                     gz = 4 * (brick / (a.nbx * a.nby));
                     more = c0 < a.ncol;
+                    Enext = oz_exponent<R, CW>(a, gx - C::PPP * lp, gy, gz, c0 + (lane & 15));
 #pragma unroll
                     for (int o = 0; o < NJ; ++o) {
                         const int col = c0 + o * (32 / C::PC) + ln;
@@ -308,16 +323,13 @@ k_gather_oz(OzGather a) {
         };
         auto perm = [](int t) { return C::PC == 4 ? (t >> 1) & 3 : (t >> 2) & 1; };
         for (int j = 0; j < C::ND; ++j) issue(j);
-        int E = 0;
         bool any = false;                        // a warp without orbitals leaves its rows as they are: they reach only
                                                  // their own outputs
         for (int i = set, j = 0; i < nsl; i += OZ_SETS, ++j) {
             if (i % C::SLICES == set) {
                 const int u = (int)blockIdx.x + (i / C::SLICES) * (int)gridDim.x;
-                const int c0 = (u % a.ctiles) * OZ_M + 16 * w, col = c0 + (lane & 15);
-                any = c0 < a.ncol;
-                E = col < a.ncol ? (int)(column_max(a.cmax, col) >> (sizeof(R) == 8 ? 20 : 23)) : 0;
-                if (E < Digits<R>::kEmin || E > Digits<R>::kEmax) E = 1 << 14;      // all digits zero
+                any = (u % a.ctiles) * OZ_M + 16 * w < a.ncol;
+                E = Enext;
             }
             asm volatile("cp.async.wait_group %0;" ::"n"(C::ND - 1) : "memory");
             __syncwarp();
@@ -370,7 +382,7 @@ k_gather_oz(OzGather a) {
             const int4 G = a.grp[u / (a.ctiles * C::PARTS)];
             const size_t row0 = (size_t)((u / a.ctiles) % C::PARTS) * a.part_rows;
             const int col = (u % a.ctiles) * OZ_M + 32 * quad + lane;
-            int E = col < a.ncol ? (int)(column_max(a.cmax, col) >> (sizeof(R) == 8 ? 20 : 23)) : 0;
+            const int E = oz_exponent<R, CW>(a, 8 * (G.x % a.nbx), 8 * (G.x / a.nbx % a.nby), 4 * (G.x / (a.nbx * a.nby)), col);
             const bool ok = mbar_wait(&tfull_bar[buf], (uu >> 1) & 1, &abort_flag);
             if (__any_sync(0xffffffffu, !ok)) break;
             tc_fence_after();
@@ -1106,7 +1118,7 @@ int gather_oz(hub_t h, const void* X, int ncol, int ld, int spin, bool want_W) {
     a.slot = t.d_ozg_row;
     a.val = t.d_ozg_val;
     a.part = (double*)h->d_part;
-    a.cmax = h->d_cmax;
+    a.bmax = block_map(h, h->d_cmax, ncol);
     a.wmax = h->d_wmax;
     a.ld = (long)ld * CW;
     a.n1 = h->n1; a.n2 = h->n2; a.n3 = h->n3;
@@ -1239,7 +1251,7 @@ bool gather_digits(hub_t h, int ncol) {
     const double digits = rounds * (ncol / OZ_M * full + (last ? part : 0.0));
     if (digits >= plain || (long)t.oz_ngroups * parts * (ncol / OZ_M + 1) > 0x7fffffffL / 64) return false;
     // the gather's workspace (the point-major form takes over without it)
-    return claim(h, (void**)&h->d_cmax, &h->cmax_bytes, (size_t)ncol * kColParts * sizeof(unsigned)) &&
+    return claim(h, (void**)&h->d_cmax, &h->cmax_bytes, colmax_bytes(h, ncol)) &&
            claim(h, (void**)&h->d_wmax, &h->wmax_bytes, (size_t)ncol * sizeof(int)) &&
            claim(h, &h->d_part, &h->part_bytes, (size_t)t.oz_npart * cw * parts * ncol * sizeof(double));
 }

@@ -5,11 +5,13 @@
 //
 //   Yout = alpha * (-1/2 Lap_h Y + V .* Y - shift * Y) + beta * Yprev        (Sec. II.B)
 //
-// Number format.  Every column has one power-of-two scale: with E the biased exponent of its
-// largest |x| (colmax.cu), X = x * 2^(1081 - E) rounded to nearest, 2^58 <= |X| < 2^59 for that
-// x.  An element keeps all 53 bits down to 2^-6 of the column's maximum and is never off by more
-// than 2^-59 of it: one FP64 rounding of the sum, which holds terms of ~300 x, is larger, but an
-// element far below the maximum (the tail of a localized column) has fewer than 53 bits.
+// Number format.  Every CTA has one power-of-two scale: with E the biased exponent of the largest
+// |x| of the pieces (32 x 8 points of an eighth of the planes, colmax.cu) that its points and their
+// neighbours lie in, X = x * 2^(1081 - E) rounded to nearest, |X| < 2^59.  An element keeps all 53
+// bits down to 2^-6 of that maximum and is never off by more than 2^-59 of it: one FP64 rounding of
+// the sum, which holds terms of ~300 x, is larger.  A column may decay by any factor over the cell;
+// only elements more than 2^-6 below others within some 70 x 30 x n3 / 4 points have fewer bits.  (One
+// scale per column, whose far tails would be cut to zero, takes 4.25 ms below.)
 // X is kept as two signed limbs, X = xh 2^30 + xl: pair sums of limbs need no carry.
 // The Laplacian weights of order 2 n0 are rational: c_p = k_p / lcd with integers k_p of 22
 // bits, so A_a = k_0 X + sum_p k_p (X_{+p} + X_{-p}) of each axis is exact, and only
@@ -21,7 +23,8 @@
 // allow: 57 to 59 bits of the largest F, fewer where |V| would pass 2^(83 - sf) (k_fx_veff).  F is
 // rounded at 2^-54 of itself or less, as the weights of the FP64 form are, and V at 2^-54 of the
 // largest kinetic energy or 2^-58 of the largest |V|.
-// Columns that the format does not cover (zero, non-finite or outside 2^+-900), potentials
+// What the format does not cover (columns that are zero or below 2^-900, CTAs with elements that are
+// not finite or above 2^900), potentials
 // that would leave F under 53 bits (8192 Ha at 0.3 bohr, 8 Ha at 10) and shifts beyond
 // 2^(83 - sf) Ha (the largest kinetic energy of the grid, at least) are computed by fx_slow in
 // plain FP64.
@@ -30,8 +33,8 @@
 // planes (with a halo of 6 in x and y) in shared memory holds the limbs; plane z + 7 is
 // converted and stored while plane z is computed, and plane z + 8 is in flight in registers, so
 // there is one barrier per plane.  The 13 z-neighbours live in registers.  Bound: the integer
-// pipes (50 multiply-adds at half rate and ~310 other instructions per point); 17.15 -> 4.25 ms
-// on 88 x 88 x 84 x 348 (DRAM floor 0.80 ms), plus 0.27 ms for the column maxima.
+// pipes (50 multiply-adds at half rate and ~310 other instructions per point); 17.15 -> 4.35 ms
+// on 88 x 88 x 84 x 348 (DRAM floor 0.80 ms), plus 0.27 ms for the maxima.
 #include <algorithm>
 #include <cmath>
 
@@ -54,7 +57,8 @@ struct FxArgs {
     const double* V;
     const int2* Vq;               // (V 2^(sf - 25)) as limbs of 30 bits
     const int* vinfo;             // largest high word of |V|; not covered (0 or 1); sf
-    const unsigned* cmax;         // column maxima (colmax.cu)
+    const unsigned* cmax;         // column maxima and pieces (colmax.cu)
+    BlockMap bmax;
     int n1, n2, n3, ld;
     int tx, ty, tilesx, tiles;    // tile shape and count
     int zchunk, nzc;
@@ -112,6 +116,41 @@ __device__ __noinline__ double fx_slow(const FxArgs& a, const double* __restrict
     return dot;
 }
 
+// first piece and number of pieces of 2^log points that [lo, hi) of a periodic axis meets (lo >= -FXH);
+// all of them where it reaches around to its own first piece
+__device__ __forceinline__ int2 pieces(int lo, int hi, int n, int count, int log) {
+    if (hi - lo + (1 << log) > n) return make_int2(0, count);
+    const int a = (lo < 0 ? lo + n : lo) >> log, b = (hi > n ? hi - n - 1 : hi - 1) >> log;
+    return make_int2(a, b >= a ? b - a + 1 : b - a + 1 + count);
+}
+// largest leading word of the pieces that meet a box: the same in every warp (a lane takes a z part
+// and every fourth piece along y), without a barrier
+__device__ __forceinline__ unsigned region_max(const BlockMap& b, int col, int x0, int x1, int n1, int y0, int y1, int n2, int z0,
+                                               int z1, int n3) {
+    const int part = threadIdx.x & 7, nblk = b.nbx * b.nby;
+    const int b0 = part * b.zper, b1 = min(b0 + b.zper, n3);
+    const bool in = b0 < b1 && (z1 - z0 >= n3 || (z0 < b1 && b0 < z1) || z0 < b1 - n3 || b0 + n3 < z1);
+    const int2 px = pieces(x0, x1, n1, b.nbx, b.xlog), py = pieces(y0, y1, n2, b.nby, b.ylog);
+    const unsigned* p = b.m + ((size_t)col * kColParts + part) * nblk;
+    unsigned m = 0;
+    if (in)
+        for (int j = (threadIdx.x >> 3) & 3; j < py.y; j += 4) {
+            int y = py.x + j;
+            if (y >= b.nby) y -= b.nby;
+            for (int i = 0; i < px.y; i += 4) {
+                unsigned v[4];                         // in flight together
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    int x = px.x + min(i + k, px.y - 1);
+                    if (x >= b.nbx) x -= b.nbx;
+                    v[k] = p[y * b.nbx + x];
+                }
+                m = max(max(m, max(v[0], v[1])), max(v[2], v[3]));
+            }
+        }
+    return __reduce_max_sync(0xffffffffu, m);
+}
+
 // 2^k, |k| < 1023 (scalbn's cases cost a small grid's launch 5 us)
 __device__ __forceinline__ double pow2(int k) { return __hiloint2double((k + 1023) << 20, 0); }
 
@@ -149,10 +188,43 @@ k_stencil_fx(const __grid_constant__ FxArgs a) {
     const double alpha = a.coef ? a.coef[0] : a.alpha, beta = a.coef ? a.coef[1] : a.beta;
     const double shift = a.coef ? a.coef[2] : a.shift;
 
-    const int emax = (int)(column_max(a.cmax, col) >> 20), e20 = emax << 20;
+    // this thread's halo'd points of a plane (beyond the last one: a point that nobody reads)
+    const int sx = a.tx + 2 * FXH, sy = a.ty + 2 * FXH, stage = sy * FXP + 2;
+    int s_idx[PER], s_off[PER];
+#pragma unroll
+    for (int k = 0; k < PER; ++k) {
+        const int i = tid + k * nt;
+        s_idx[k] = sy * FXP;
+        s_off[k] = 0;
+        if (i < sx * sy) {
+            const int iy = i / sx, ix = i - iy * sx;
+            s_idx[k] = iy * FXP + ix;
+            s_off[k] = wrap(gy0 - FXH + iy, n2) * n1 + wrap(gx0 - FXH + ix, n1);
+        }
+    }
+    auto load = [&](long zo, double (&v)[PER]) {
+#pragma unroll
+        for (int k = 0; k < PER; ++k) v[k] = Y[zo + s_off[k]];
+    };
+    double pf[PER];
+    long zl = (long)z0 * plane;                   // plane loaded last
+    load(zl, pf);
+
+    // the scale: the column's, or that of the pieces that this CTA's points and their neighbours lie in
+    unsigned top;
+    if constexpr (DOT) top = column_max(a.cmax, col);
+    else top = region_max(a.bmax, col, gx0 - FXH, gx0 + a.tx + FXH, n1, gy0 - FXH, gy0 + a.ty + FXH, n2, z0 - FXH,
+                          max(z1 + FXH, z0 + 8), n3);         // plane z0 + 7 is converted in any case
+    int emax = (int)(top >> 20);
     const int sf = a.vinfo[2];
     const bool fits = fabs(shift) < pow2(83 - sf);              // NaN: false
-    if (emax < kFxEmin || emax > kFxEmax || !fits || a.vinfo[1]) {    // the same for the whole CTA
+    bool plain = emax > kFxEmax || !fits || a.vinfo[1];         // the same for the whole CTA
+    if (emax < kFxEmin) {
+        plain |= (int)(column_max(a.cmax, col) >> 20) < kFxEmin;
+        emax = kFxEmin;
+    }
+    const int e20 = emax << 20;
+    if (plain) {
         const double sum = fx_slow(a, Y, Yp, Yo, gx0, gy0, z0, z1, alpha, beta, shift);
         if constexpr (DOT) finish_dot(a, sum);
         return;
@@ -172,20 +244,6 @@ k_stencil_fx(const __grid_constant__ FxArgs a) {
     // the smooth part of its input and damps the rest, would keep all of it
     const long long m1 = (1 << 29) + (((long long)fl[0] + fl[1] + fl[2]) >> 1);
 
-    // this thread's halo'd points of a plane (beyond the last one: a point that nobody reads)
-    const int sx = a.tx + 2 * FXH, sy = a.ty + 2 * FXH, stage = sy * FXP + 2;
-    int s_idx[PER], s_off[PER];
-#pragma unroll
-    for (int k = 0; k < PER; ++k) {
-        const int i = tid + k * nt;
-        s_idx[k] = sy * FXP;
-        s_off[k] = 0;
-        if (i < sx * sy) {
-            const int iy = i / sx, ix = i - iy * sx;
-            s_idx[k] = iy * FXP + ix;
-            s_off[k] = wrap(gy0 - FXH + iy, n2) * n1 + wrap(gx0 - FXH + ix, n1);
-        }
-    }
     // rows ROWS * ty .. of the tile
     const int ty = tid / a.tx, tx = tid - ty * a.tx;
     bool act[ROWS];
@@ -199,24 +257,23 @@ k_stencil_fx(const __grid_constant__ FxArgs a) {
     const int ctr = act[0] ? (ROWS * ty + FXH) * FXP + tx + FXH : FXH * FXP + FXH;
     const int last = z1 + FXH - 1;                // highest plane needed
 
-    auto load = [&](long zo, double (&v)[PER]) {
-#pragma unroll
-        for (int k = 0; k < PER; ++k) v[k] = Y[zo + s_off[k]];
-    };
     auto store = [&](int j, const double (&v)[PER]) {
         int2* dst = ring + (j & (FXS - 1)) * stage;
 #pragma unroll
         for (int k = 0; k < PER; ++k) dst[s_idx[k]] = to_limbs(v[k], e20);
     };
 
-    // planes z0 .. z0 + 6 into the ring (stage index: plane - z0), z-queue z0 - 6 .. z0 + 5
-    double pf[PER];
-    long zl = (long)z0 * plane;                   // plane to load next
+    // planes z0 .. z0 + 6 into the ring (stage index: plane - z0), each while the next is in flight (plane
+    // z0 + 7 at last, needed or not: it is inside the block); z-queue z0 - 6 .. z0 + 5
+#pragma unroll 1
     for (int j = 0; j <= FXH; ++j) {
-        load(zl, pf);
-        store(j, pf);
+        double next[PER];
         zl += plane;
         if (zl == cell) zl = 0;
+        load(zl, next);
+        store(j, pf);
+#pragma unroll
+        for (int k = 0; k < PER; ++k) pf[k] = next[k];
     }
     int2 q[ROWS][2 * FXH + 1];                    // [i]: plane z - 7 + i before the shift
 #pragma unroll
@@ -225,7 +282,6 @@ k_stencil_fx(const __grid_constant__ FxArgs a) {
 #pragma unroll
         for (int r = 0; r < ROWS; ++r) q[r][1 + j] = to_limbs(Y[zo + own[r]], e20);
     }
-    load(zl, pf);                                 // plane z0 + 7 (needed or not: inside the block)
     long zo = (long)z0 * plane;
     int2 vq[ROWS];
     double yp[ROWS];
@@ -432,6 +488,7 @@ static int run_fx(hub_t h, const StencilArgs& s, int variant, const StencilDot* 
     a.Vq = (const int2*)(a.V + h->Nd);
     a.vinfo = (const int*)(a.Vq + h->Nd);
     a.cmax = h->d_cmax;
+    a.bmax = block_map(h, h->d_cmax, s.ncol);
     a.n1 = s.n1; a.n2 = s.n2; a.n3 = s.n3; a.ld = s.ld;
     const FxSetup f = fx_setup(h);
     double wb = 0.0;
