@@ -112,6 +112,8 @@ struct Table {
     int* d_oz_exp = nullptr;          // [nproj] biased exponent of each function's largest value
     int* d_oz_roff = nullptr;         // [nproj + 1] partial rows of each projector row (CSR)
     int* d_oz_rent = nullptr;
+    int* d_oz_sfirst = nullptr;       // [nsites + 1] bricks of each site (CSR, indexes of d_ozb)
+    int* d_oz_sbrick = nullptr;
     // tensor-core form of the brick gather (built with the bricks when n1 % 4 == 0): the
     // entries of each brick packed into groups of at most 64 functions, per group its values
     // in the 128-byte-swizzled K-major layout of tcgen05 operands, split as TF32 hi + lo,
@@ -197,7 +199,7 @@ struct hub_ctx {
     unsigned int* d_bar = nullptr;  // [4] grid-barrier state
     double* d_scal = nullptr;     // [256] device scalars (Lanczos, reductions)
     unsigned* d_cmax = nullptr;   size_t cmax_bytes = 0;    // column maxima (colmax.cu)
-    int* d_wmax = nullptr;        size_t wmax_bytes = 0;    // column maxima of W (projectors_oz.cu)
+    int* d_wmax = nullptr;        size_t wmax_bytes = 0;    // maxima of W by brick and column (projectors_oz.cu)
     unsigned* d_tcmax = nullptr;  // [4] max |x| bit patterns of the FP16 operands (scales)
 
     hub::ScfState* scf = nullptr;

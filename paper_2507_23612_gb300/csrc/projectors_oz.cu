@@ -7,9 +7,9 @@
 // 1.09 and 1.37 ms).  Both are small dense products per brick of 8 x 8 x 4 points, and here they run on the FP16
 // tensor cores with operands split into 7 (double) or 4 (float) 8-bit digits (digits.cuh):
 // digit products and, where it counts, their sums are exact, so the result carries the rounding of
-// the operands to 54 (30) bits below the largest magnitude of their column or function and one
-// rounding of the sum.  Over a column that is below the rounding of the sums it replaces; where the
-// column is far below its own maximum, inner products and updates have fewer bits than those had.
+// the operands to 54 (30) bits below the largest magnitude of the values of X, or of the coefficients,
+// around the brick and of the function, and one rounding of the sum, below the rounding of the sums it
+// replaces.
 //
 // Complex blocks are real ones of twice the points and functions: a brick's 256 complex points
 // are 512 reals (re, im alternating), a function has slot a = (phi_r, phi_i) (real part of
@@ -56,8 +56,10 @@ constexpr int OZ_M = 128;                     // orbitals (gather) or reals (sca
 constexpr int OZ_MAXK = 512;                  // slots per brick at most
 constexpr int OZ_SETS = 2;                     // sets of 8 converter warps, on alternate slices
 constexpr int OZ_GTHREADS = 32 * (2 + 8 * OZ_SETS + 8);
-constexpr int kWOff = 4096;                   // d_wmax: biased exponent + kWOff, 0 for a zero column
-constexpr int kWBad = 1 << 20;                // d_wmax of a column with non-finite values
+// d_wmax [brick][column]: biased exponent of the largest coefficient of the brick's functions times
+// the function's, + kWOff, or 0 (all zero) or kWBad (with non-finite values)
+constexpr int kWOff = 4096;
+constexpr int kWBad = 1 << 20;
 
 template <typename R, int CW>
 struct GCfg {
@@ -116,7 +118,8 @@ struct OzGather {
     const uint4* val;
     double* part;
     BlockMap bmax;            // maxima of X
-    int* wmax;                // cleared for the reduction
+    int* wmax;                // cleared for the reduction: nw values
+    long nw;
     long part_rows;           // rows of one part of the bricks
     long ld;                  // in reals
     int n1, n2, n3, ncol, nbx, nby, nunits, ctiles, vec;
@@ -150,7 +153,7 @@ k_gather_oz(OzGather a) {
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int nu = (a.nunits - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;
-    for (int i = blockIdx.x * OZ_GTHREADS + threadIdx.x; i < a.ncol; i += gridDim.x * OZ_GTHREADS) a.wmax[i] = 0;
+    for (long i = (long)blockIdx.x * OZ_GTHREADS + threadIdx.x; i < a.nw; i += (long)gridDim.x * OZ_GTHREADS) a.wmax[i] = 0;
 
     if (threadIdx.x == 0) {
         abort_flag = 0;
@@ -462,6 +465,8 @@ struct OzReduce {
     double* C;
     void* W;
     int* wmax;
+    const int* sfirst;        // bricks of every site
+    const int* sbrick;
     const unsigned* cmax;
     const void* X;
     const int* idx;
@@ -471,6 +476,30 @@ struct OzReduce {
     double dV;
     int ncol, want_W;
 };
+
+// A site's coefficients of column n (per lane; written by warp 0, which takes their maximum) into the
+// maxima of the bricks that its functions reach.  256 threads, 32 columns.
+template <typename R, int CW>
+__device__ __forceinline__ void raise_wmax(const SiteDev& S, const R* W, const int* exps, const int* sfirst, const int* sbrick, int n,
+                                           int ncol, int* wmax) {
+    __shared__ int tops[32];
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (w == 0) {
+        int top = 0;
+        if (n < ncol)
+            for (int p = 0; p < S.nproj; ++p)
+                for (int q = 0; q < CW; ++q) {
+                    const int e = Digits<R>::exponent(W[((size_t)(S.proj_off + p) * ncol + n) * CW + q]);
+                    if (e == (sizeof(R) == 8 ? 0x7ff : 0xff)) top = kWBad;
+                    else if (e > 0) top = max(top, e + exps[S.proj_off + p] - Digits<R>::kBias + kWOff);
+                }
+        tops[lane] = top;
+    }
+    __syncthreads();
+    const int top = tops[lane];
+    if (top == 0) return;
+    for (int e = sfirst[blockIdx.x] + w; e < sfirst[blockIdx.x + 1]; e += 8) atomicMax(wmax + (size_t)sbrick[e] * ncol + n, top);
+}
 
 template <typename R, int CW>
 __global__ void __launch_bounds__(256)
@@ -558,48 +587,24 @@ k_reduce_oz(OzReduce a) {
             __syncthreads();
         }
     }
-    if (w != 0 || n >= a.ncol) return;
-    D c[kMaxProj];
-    for (int p = 0; p < S.nproj; ++p) {
-        if constexpr (CPLX) c[p] = make_double2(red[0][2 * p][lane], red[0][2 * p + 1][lane]);
-        else c[p] = red[0][p][lane];
-        ((D*)a.C)[(size_t)(S.proj_off + p) * a.ncol + n] = c[p];
-    }
-    if (!a.want_W) return;
-    site_transform<R, CPLX>(S, c, a.gamma, a.M, (T*)a.W, n, a.ncol);
-    int top = 0;
-    for (int p = 0; p < S.nproj; ++p)
-        for (int q = 0; q < CW; ++q) {
-            const R v = ((const R*)a.W)[((size_t)(S.proj_off + p) * a.ncol + n) * CW + q];
-            const int e = Digits<R>::exponent(v);
-            if (e == (sizeof(R) == 8 ? 0x7ff : 0xff)) top = kWBad;
-            else if (e > 0) top = max(top, e + a.exps[S.proj_off + p] - Digits<R>::kBias + kWOff);
+    if (w == 0 && n < a.ncol) {
+        D c[kMaxProj];
+        for (int p = 0; p < S.nproj; ++p) {
+            if constexpr (CPLX) c[p] = make_double2(red[0][2 * p][lane], red[0][2 * p + 1][lane]);
+            else c[p] = red[0][p][lane];
+            ((D*)a.C)[(size_t)(S.proj_off + p) * a.ncol + n] = c[p];
         }
-    if (top) atomicMax(a.wmax + n, top);
+        if (a.want_W) site_transform<R, CPLX>(S, c, a.gamma, a.M, (T*)a.W, n, a.ncol);
+    }
+    if (a.want_W) raise_wmax<R, CW>(S, (const R*)a.W, a.exps, a.sfirst, a.sbrick, n, a.ncol, a.wmax);
 }
 
-// column maxima of a W that did not come from the reduction: 32 columns per CTA, its 8 warps on
-// the rows w, w + 8, ...
+// maxima of a W that did not come from the reduction (wmax cleared before): one CTA per (site, 32 columns)
 template <typename R, int CW>
 __global__ void __launch_bounds__(256)
-k_wmax_oz(const R* __restrict__ W, const int* __restrict__ exps, int nproj, int ncol, int* __restrict__ wmax) {
-    __shared__ int red[8][32];
-    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, n = blockIdx.x * 32 + lane;
-    int top = 0;
-    if (n < ncol)
-        for (int p = w; p < nproj; p += 8)
-#pragma unroll
-            for (int q = 0; q < CW; ++q) {
-                const int e = Digits<R>::exponent(W[((size_t)p * ncol + n) * CW + q]);
-                if (e == (sizeof(R) == 8 ? 0x7ff : 0xff)) top = kWBad;
-                else if (e > 0) top = max(top, e + exps[p] - Digits<R>::kBias + kWOff);
-            }
-    red[w][lane] = top;
-    __syncthreads();
-    if (w == 0 && n < ncol) {
-        for (int k = 1; k < 8; ++k) top = max(top, red[k][lane]);
-        wmax[n] = top;
-    }
+k_wmax_oz(const SiteDev* __restrict__ sites, const R* __restrict__ W, const int* __restrict__ exps, const int* __restrict__ sfirst,
+          const int* __restrict__ sbrick, int ncol, int* __restrict__ wmax) {
+    raise_wmax<R, CW>(sites[blockIdx.x], W, exps, sfirst, sbrick, blockIdx.y * 32 + (threadIdx.x & 31), ncol, wmax);
 }
 
 // ---------------------------------------------------------------------------- scatter
@@ -766,6 +771,7 @@ k_scatter_oz(OzScatter a) {
         bool stop = false;
         for (int q = 0; q < np && !stop; ++q) {
             const int4 B = a.brick[pair_of(q) / C::PASSES];
+            const int* wmax = a.wmax + (size_t)(pair_of(q) / C::PASSES) * a.ncol;
             const int nk = B.y / 16;
             for (int l = 0; l < nk * a.ctiles; ++l, ++i) {
                 if (i % C::BW != b) continue;
@@ -775,7 +781,7 @@ k_scatter_oz(OzScatter a) {
                 for (int it = 0; it < NT / 16; ++it) {
                     const int task = it * 32 + lane, o = task % NT, kc = task / NT, col = c0 + o;
                     const int4* sl = reinterpret_cast<const int4*>(a.slot + B.w + c * 16 + kc * 8);
-                    const int wm = col < a.ncol ? a.wmax[col] : 0;
+                    const int wm = col < a.ncol ? wmax[col] : 0;
                     const int E = wm - kWOff;
                     const bool good = wm > 0 && wm < kWBad;
                     R x[8];
@@ -822,6 +828,7 @@ k_scatter_oz(OzScatter a) {
         int uu = 0, used = 0;                      // units so far; read-outs so far of this set's buffer (WIDE)
         bool stop = false;
         for (int q = 0; q < np && !stop; ++q) {
+            const int* wmax = a.wmax + (size_t)(pair_of(q) / C::PASSES) * a.ncol;
             const int pr = pair_of(q), brick = a.brick[pr / C::PASSES].x, nk = WIDE ? a.brick[pr / C::PASSES].y / 16 : 0;
             const int k = (pr % C::PASSES) * 256 + t * 128 + 32 * quad + lane;
             const int p = k / CW, comp = k % CW;
@@ -836,8 +843,8 @@ k_scatter_oz(OzScatter a) {
                 R yv[NT];
 #pragma unroll
                 for (int o = 0; o < NT; ++o) yv[o] = o < nc ? Y[(size_t)o * a.ld] : R(0);
-                // lane o < NT: column c0 + o.  A zero column has zero digits whatever its exponent.
-                const int wm = lane < NT && c0 + lane < a.ncol ? a.wmax[c0 + lane] : 0;
+                // lane o < NT: column c0 + o.  Zero coefficients have zero digits whatever the exponent.
+                const int wm = lane < NT && c0 + lane < a.ncol ? wmax[c0 + lane] : 0;
                 const int E = wm == 0 ? Digits<R>::kBias : wm - kWOff;
                 const unsigned odd = __ballot_sync(0xffffffffu, wm >= kWBad || E < Digits<R>::kEmin || E > Digits<R>::kEmax);
                 auto read_out = [&]() {
@@ -1062,6 +1069,12 @@ int build_oz(hub_t h, Table& t, const std::vector<std::vector<int>>& site_pts) {
         t.oz_wide |= K > 256;
         if (K > OZ_MAXK || goff >= (1ull << 31) || boff >= (1ull << 31) || prow * CW >= (1L << 31)) return HUB_OK;
     }
+    std::vector<int> sfirst(t.nsites + 1, 0), sbrick(pl.size());
+    for (size_t i = 0; i < pl.size(); ++i) {
+        sfirst[pl[i].site + 1]++;
+        sbrick[i] = pairs[i].z;
+    }
+    for (int i = 0; i < t.nsites; ++i) sfirst[i + 1] += sfirst[i];
     // on a device without room for both layouts the point-major form does all products
     size_t tmp = 0;
     int *d_row_pair = nullptr, *d_gfn = nullptr, *d_bfn = nullptr;
@@ -1075,7 +1088,8 @@ int build_oz(hub_t h, Table& t, const std::vector<std::vector<int>>& site_pts) {
                     room((void**)&t.d_oz_exp, std::max(t.nproj, 1) * sizeof(int)) && put(h, &t.d_ozg, grp, &t.oz_bytes) &&
                     put(h, &t.d_ozg_row, gslot, &t.oz_bytes) && put(h, &t.d_ozb, brk, &t.oz_bytes) &&
                     put(h, &t.d_ozb_row, bslot, &t.oz_bytes) && put(h, &t.d_oz_roff, roff, &t.oz_bytes) &&
-                    put(h, &t.d_oz_rent, rent, &t.oz_bytes) && put(h, &d_row_pair, row_pair, &tmp) &&
+                    put(h, &t.d_oz_rent, rent, &t.oz_bytes) && put(h, &t.d_oz_sfirst, sfirst, &t.oz_bytes) &&
+                    put(h, &t.d_oz_sbrick, sbrick, &t.oz_bytes) && put(h, &d_row_pair, row_pair, &tmp) &&
                     put(h, &d_pairs, pairs, &tmp) && put(h, &d_gfn, gfn, &tmp) && put(h, &d_bfn, bfn, &tmp);
     cudaError_t e = cudaGetLastError(), es = cudaSuccess;
     if (ok) {
@@ -1120,6 +1134,7 @@ int gather_oz(hub_t h, const void* X, int ncol, int ld, int spin, bool want_W) {
     a.part = (double*)h->d_part;
     a.bmax = block_map(h, h->d_cmax, ncol);
     a.wmax = h->d_wmax;
+    a.nw = want_W ? (long)t.oz_nbricks * ncol : 0;
     a.ld = (long)ld * CW;
     a.n1 = h->n1; a.n2 = h->n2; a.n3 = h->n3;
     a.ncol = ncol;
@@ -1147,6 +1162,8 @@ int gather_oz(hub_t h, const void* X, int ncol, int ld, int spin, bool want_W) {
     r.C = (double*)h->d_C;
     r.W = h->d_W;
     r.wmax = h->d_wmax;
+    r.sfirst = t.d_oz_sfirst;
+    r.sbrick = t.d_oz_sbrick;
     r.cmax = h->d_cmax;
     r.X = X;
     r.idx = t.d_idx;
@@ -1169,7 +1186,9 @@ int scatter_oz(hub_t h, void* Y, int ncol, int ld, double alpha, const double* a
     int rc;
     if (!wmax_ready) {
         ProfScope ps(h, HUB_K_SCATTER);
-        k_wmax_oz<R, CW><<<(ncol + 31) / 32, 256, 0, h->stream>>>((const R*)h->d_W, t.d_oz_exp, t.nproj, ncol, h->d_wmax);
+        HUB_CUDA_TRY(h, cudaMemsetAsync(h->d_wmax, 0, (size_t)t.oz_nbricks * ncol * sizeof(int), h->stream));
+        k_wmax_oz<R, CW><<<dim3((unsigned)t.nsites, (unsigned)((ncol + 31) / 32)), 256, 0, h->stream>>>(
+            t.d_sites, (const R*)h->d_W, t.d_oz_exp, t.d_oz_sfirst, t.d_oz_sbrick, ncol, h->d_wmax);
         HUB_CUDA_TRY(h, cudaGetLastError());
     }
     OzScatter a{};
@@ -1211,12 +1230,12 @@ int scatter_oz(hub_t h, void* Y, int ncol, int ld, double alpha, const double* a
 
 void free_oz(hub_t h, Table& t) {
     for (void* p : {(void*)t.d_ozg, (void*)t.d_ozg_row, (void*)t.d_ozg_val, (void*)t.d_ozb, (void*)t.d_ozb_row, (void*)t.d_ozb_val,
-                    (void*)t.d_oz_exp, (void*)t.d_oz_roff, (void*)t.d_oz_rent})
+                    (void*)t.d_oz_exp, (void*)t.d_oz_roff, (void*)t.d_oz_rent, (void*)t.d_oz_sfirst, (void*)t.d_oz_sbrick})
         if (p) cudaFree(p);
     t.d_ozg = t.d_ozb = nullptr;
     t.d_ozg_row = t.d_ozb_row = nullptr;
     t.d_ozg_val = t.d_ozb_val = nullptr;
-    t.d_oz_exp = t.d_oz_roff = t.d_oz_rent = nullptr;
+    t.d_oz_exp = t.d_oz_roff = t.d_oz_rent = t.d_oz_sfirst = t.d_oz_sbrick = nullptr;
     h->mem_held -= t.oz_bytes;
     t.oz_bytes = 0;
     if (t.oz) h->mem_gen++;
@@ -1252,7 +1271,7 @@ bool gather_digits(hub_t h, int ncol) {
     if (digits >= plain || (long)t.oz_ngroups * parts * (ncol / OZ_M + 1) > 0x7fffffffL / 64) return false;
     // the gather's workspace (the point-major form takes over without it)
     return claim(h, (void**)&h->d_cmax, &h->cmax_bytes, colmax_bytes(h, ncol)) &&
-           claim(h, (void**)&h->d_wmax, &h->wmax_bytes, (size_t)ncol * sizeof(int)) &&
+           claim(h, (void**)&h->d_wmax, &h->wmax_bytes, (size_t)t.oz_nbricks * ncol * sizeof(int)) &&
            claim(h, &h->d_part, &h->part_bytes, (size_t)t.oz_npart * cw * parts * ncol * sizeof(double));
 }
 
@@ -1265,7 +1284,7 @@ bool scatter_digits(hub_t h, int ncol, bool wmax_ready) {
                            : (h->cplx ? 6.8e-7 : 3.7e-7) * t.nvals * std::max(ncol, 12);
     const long pairs = (long)t.oz_nbricks * cw;
     const double digits = (double)((pairs + h->num_sms - 1) / h->num_sms) * ((ncol + nt - 1) / nt) * (d ? 4.2 : 5.5) + 12.0;
-    return digits < plain + 10.0 && (wmax_ready || claim(h, (void**)&h->d_wmax, &h->wmax_bytes, (size_t)ncol * sizeof(int)));
+    return digits < plain + 10.0 && (wmax_ready || claim(h, (void**)&h->d_wmax, &h->wmax_bytes, (size_t)t.oz_nbricks * ncol * sizeof(int)));
 }
 
 int launch_gather_oz(hub_t h, const void* X, int ncol, int ld, int spin, bool want_W) {

@@ -99,3 +99,35 @@ def test_gather(prec, cplx):
     top = np.array([np.max(near[:, inside[:, p]], axis=1) for p in range(P.shape[1])])
     pts = np.count_nonzero(P, axis=0)[:, None]
     assert np.all(np.abs(C - ref) <= 16 * u * g.dV * top * np.max(np.abs(P), axis=0)[:, None] * pts)
+
+
+@pytest.mark.parametrize("prec,cplx", [(HUB_F64, False), (HUB_F64, True), (HUB_F32, True)])
+def test_scatter(prec, cplx):
+    """Coefficients that decay with the atoms' distance from a centre of each column."""
+    kpt = (0.05, 0.2, -0.3) if cplx else (0.0, 0.0, 0.0)
+    ats = atoms()
+    g, P = tables(ats, kpt)
+    hb = Hub(N, L, 6, prec=prec, complex_=cplx, kpt=kpt if cplx else None)
+    copies = 1 if prec == HUB_F64 else 4
+    hb.set_atoms(ats * copies)
+    rng = np.random.default_rng(3)
+    ncol = 130
+    x = np.repeat([a.pos[0] / L[0] for a in ats], 9)
+    d = np.abs(x[:, None] - rng.uniform(0, 1, ncol)[None])
+    W = rng.uniform(0.5, 1.0, (P.shape[1], ncol)) * (1e-24 if prec == HUB_F64 else 1e-9) ** (2 * np.minimum(d, 1 - d))
+    W = W * np.exp(1j * rng.uniform(0, 6.28, W.shape)) if cplx else W
+    Y = torch.zeros(ncol, ND, dtype=hb.dtype, device="cuda")
+    hb.profile(1)
+    hb.expand(np.concatenate([W] * copies), Y, 1.0)
+    assert hb.profile_read()["scatter"][1] == 2             # maxima of W, then the digit form
+    hb.profile(-1)
+    got = Y.cpu().numpy().reshape(ncol, -1, N[0])
+    W = W.astype({HUB_F64: np.complex128, HUB_F32: np.complex64}[prec]) if cplx else W
+    ref = copies * (P @ W).T.reshape(ncol, -1, N[0])
+    # of the coefficients of functions on the same brick: those whose x planes come within 8 points
+    inside = (np.abs(P) > 0).reshape(-1, N[0], P.shape[1]).any(0)
+    inside = np.any([np.roll(inside, s, axis=0) for s in range(-8, 9)], axis=0)
+    top = np.array([np.max(np.abs(W) * inside[i][:, None], axis=0) for i in range(N[0])]).T
+    u = 2.0 ** -53 if prec == HUB_F64 else 2.0 ** -24
+    terms = copies * np.count_nonzero(inside, axis=1)
+    assert np.all(np.abs(got - ref) <= (16 * u * np.max(np.abs(P)) * terms * top)[:, None])
