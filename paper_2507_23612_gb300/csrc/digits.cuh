@@ -21,7 +21,9 @@
 //
 // The bits are relative to the largest magnitude of the group: a number 2^-k of it has k bits
 // fewer, down to none, where a floating-point operand would keep all of its own.  So groups are
-// small where the results are local: the values of X around a brick (gather).
+// small where the results are local: the values of X around a brick (gather), the coefficients of a
+// brick's functions (scatter), the orbitals at a point (rotation); a Gram product, which is a norm, takes
+// whole columns.
 #pragma once
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>

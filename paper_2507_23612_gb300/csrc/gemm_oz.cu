@@ -14,7 +14,8 @@
 // Both are D[128 x 64] = sum_k A[128, k] B[64, k]: rows and columns are orbitals and k the grid
 // for the Gram product (k split over CTAs), rows are grid points, columns the new and k the old
 // orbitals for the rotation.  In the rotation the column scales of X move into Q (a power of two
-// per row), so that the digits of one grid point share a scale over k.
+// per row), and the digits of one grid point share a scale over k, that of the orbitals there: a point
+// where all of them are small keeps its bits.
 //
 // A conversion pass writes the digits in the order in which the MMAs read them (K-major, no
 // swizzle: 16-byte units of 8 k; per 16 k and row tile one contiguous block), in panels of the
@@ -25,8 +26,8 @@
 // Kernel: warp 0 copies, warp 1 issues the MMAs, warps 2-9 read the accumulators (one TMEM lane
 // quarter and 32 columns each) into 64-bit sums in registers.  Every mbarrier wait is bounded.
 // Bound by the tensor pipe (28 digit products of FP64: 896 clocks per 16 k of a tile): on
-// 650,496 x 348 the symmetric Gram product takes 2.0 ms, the rotation 2.6 ms, the conversions
-// 0.65 ms per operand.
+// 650,496 x 348 the symmetric Gram product takes 2.2 ms, the rotation 3.2 ms, the conversions
+// 0.65 ms per operand (0.9 for the rotation's rows).
 //
 // Columns outside the digit format (non-finite or of extreme magnitude) are summed in plain FP64.
 #include <algorithm>
@@ -73,6 +74,7 @@ struct MzArgs {
     long ldy, row0, rows;     // rows row0 .. row0 + rows of Y
     int n;
     const int* escale;        // per column: exponent of the result; [n]: not covered
+    const int* rexp;          // per row of the panel: its own, to be added
     const void* X;            // plain sums
     const double* Q;
     long ldx;
@@ -257,6 +259,7 @@ k_mm_oz(const __grid_constant__ MzArgs a) {
                 const long r = (long)t.x * MZ_M + row;
                 const bool plain = a.escale[a.n] != 0;
                 if (r < a.rows) {
+                    const int re = a.rexp[r];
                     R* y = (R*)a.Y + a.row0 + r;
 #pragma unroll
                     for (int c = 0; c < 32; ++c) {
@@ -269,10 +272,10 @@ k_mm_oz(const __grid_constant__ MzArgs a) {
                             for (int k = 0; k < a.k; ++k) v = fma((double)x[(size_t)k * a.ldx], a.Q[(size_t)k * a.n + col], v);
                         } else if constexpr (S == 7) {
                             // hs 2^24 + ls, rounded once: |hs| < 2^46 per 512 terms
-                            v = a.k <= 512 ? scale2((double)((hs[c] << 14) + ((ls[c] + 512) >> 10)), a.escale[col] + 10)
-                                           : scale2(fma((double)hs[c], 16777216.0, (double)ls[c]), a.escale[col]);
+                            v = a.k <= 512 ? scale2((double)((hs[c] << 14) + ((ls[c] + 512) >> 10)), a.escale[col] + 10 + re)
+                                           : scale2(fma((double)hs[c], 16777216.0, (double)ls[c]), a.escale[col] + re);
                         } else {
-                            v = scale2((double)((hs[c] << 8) + ls[c]), a.escale[col] - 8);
+                            v = scale2((double)((hs[c] << 8) + ls[c]), a.escale[col] - 8 + re);
                         }
                         y[(size_t)col * a.ldy] = (R)v;
                     }
@@ -351,25 +354,57 @@ k_digits_tall(const R* __restrict__ X, long ld, long Nd, int ncol, long g0, int 
     if (B && col < ct * MZ_N) put_digits<R>(b, B + ((size_t)step * ct + (col >> 6)) * (2 * S * MZ_N) + (size_t)kc * S * MZ_N + (col & 63), MZ_N);
 }
 
-// Rotation: rows r0 .. of X, k = orbital (A form, 128-row tiles); a thread takes 8 orbitals of one
-// row, lanes are neighbouring rows
+// Rotation: rows r0 .. of X, k = orbital (A form, 128-row tiles).  A CTA takes 32 rows: the largest
+// exponent of each relative to its columns' (rexp), then the digits, 8 orbitals per thread (the second
+// read comes from the caches: 32 x 348 doubles are 89 KB)
 template <typename R>
 __global__ void __launch_bounds__(256)
 k_digits_rows(const R* __restrict__ X, long ld, int k, long r0, long rows, int rt, const unsigned* __restrict__ cmax,
-              uint4* __restrict__ A) {
+              uint4* __restrict__ A, int* __restrict__ rexp) {
     constexpr int S = Digits<R>::S;
-    const long r = (long)blockIdx.x * 256 + threadIdx.x;
-    const int u = blockIdx.y;
-    if (r >= (long)rt * MZ_M) return;
-    typename Digits<R>::I b[8];
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        const int c = 8 * u + i;
-        int E = c < k ? column_exponent<R>(cmax, c) : 0;
-        if (!covered<R>(E)) E = 1 << 14;
-        b[i] = Digits<R>::bytes(c < k && r < rows ? X[(size_t)c * ld + r0 + r] : R(0), E);
+    extern __shared__ int cexp[];
+    __shared__ int tops[8][32];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const long r = (long)blockIdx.x * 32 + lane;
+    for (int c = threadIdx.x; c < k; c += 256) {
+        const int E = column_exponent<R>(cmax, c);
+        cexp[c] = covered<R>(E) ? E : 1 << 14;
     }
-    put_digits<R>(b, A + (((size_t)(u >> 1) * rt + (r >> 7)) * S * 2 + (u & 1)) * MZ_M + (r & 127), 2 * MZ_M);
+    __syncthreads();
+    const bool in = r < rows;
+    const R* x = X + r0 + (in ? r : 0);
+    int top = -(1 << 16);
+    int c = warp;
+    for (; c + 24 < k; c += 32) {
+        R v[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) v[i] = x[(size_t)(c + 8 * i) * ld];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int e = Digits<R>::exponent(v[i]);
+            if (e > 0) top = max(top, e - cexp[c + 8 * i]);
+        }
+    }
+    for (; c < k; c += 8) {
+        const int e = Digits<R>::exponent(x[(size_t)c * ld]);
+        if (e > 0) top = max(top, e - cexp[c]);
+    }
+    tops[warp][lane] = top;
+    __syncthreads();
+#pragma unroll
+    for (int w = 0; w < 8; ++w) top = max(top, tops[w][lane]);
+    if (top < -(1 << 13)) top = 0;                                     // nothing but zeros and columns not covered
+    if (warp == 0 && r < (long)rt * MZ_M) rexp[r] = top;
+    for (int u = warp; u < (k + 15) / 16 * 2; u += 8) {
+        R v[8];
+        typename Digits<R>::I b[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) v[i] = 8 * u + i < k && in ? x[(size_t)(8 * u + i) * ld] : R(0);
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+            b[i] = Digits<R>::exponent(v[i]) > 0 ? Digits<R>::bytes(v[i], cexp[8 * u + i] + top) : Digits<R>::kZero;
+        put_digits<R>(b, A + (((size_t)(u >> 1) * rt + (r >> 7)) * S * 2 + (u & 1)) * MZ_M + (r & 127), 2 * MZ_M);
+    }
 }
 
 // Q (double, row-major k x n) times the column scales of X, as B form digits; one warp per column.
@@ -556,16 +591,18 @@ int rotate_oz(hub_t h, const void* X, int ldx, const double* Q, int k, int n, vo
     int rc;
     const long Nd = h->Nd;
     const int ct = (n + MZ_N - 1) / MZ_N, ks = (k + 15) / 16;
-    const size_t perTile = (size_t)ks * C::AB, nB = (size_t)ks * ct * C::BB;
+    const size_t perTile = (size_t)ks * C::AB + MZ_M * sizeof(int), nB = (size_t)ks * ct * C::BB;
     const long tilesAll = (Nd + MZ_M - 1) / MZ_M;
     long per = std::max<long>(1, std::min<long>(tilesAll, (long)(MZ_PANEL / perTile)));
+    if (k > 12000) return HUB_ENOMEM;                 // the columns' exponents in shared memory
     const size_t nE = ((size_t)(n + 1) * sizeof(int) + 255) / 256 * 256;
     if (!claim(h, (void**)&h->d_cmax, &h->cmax_bytes, (size_t)k * kColParts * sizeof(unsigned)) ||
         !claim_panel(h, per, perTile, nB + nE)) return HUB_ENOMEM;
     if ((rc = launch_colmax_at(h, X, k, ldx, h->d_cmax))) return rc;
     uint4* dA = (uint4*)h->d_bf16;
-    uint4* dB = dA + (size_t)per * perTile / 16;
+    uint4* dB = dA + (size_t)per * ks * C::AB / 16;
     int* esc = (int*)((char*)dB + nB);
+    int* rexp = (int*)((char*)esc + nE);
     HUB_CUDA_TRY(h, cudaMemsetAsync(esc + n, 0, sizeof(int), h->stream));
     {
         ProfScope ps(h, HUB_K_COPY);
@@ -581,6 +618,7 @@ int rotate_oz(hub_t h, const void* X, int ldx, const double* Q, int k, int n, vo
     a.ldy = ldy;
     a.n = n;
     a.escale = esc;
+    a.rexp = rexp;
     a.X = X;
     a.Q = Q;
     a.ldx = ldx;
@@ -593,8 +631,8 @@ int rotate_oz(hub_t h, const void* X, int ldx, const double* Q, int k, int n, vo
         a.rows = std::min<long>((long)a.rt * MZ_M, Nd - a.row0);
         {
             ProfScope ps(h, HUB_K_COPY);
-            k_digits_rows<R><<<dim3((unsigned)((a.rt * MZ_M + 255) / 256), 2 * ks), 256, 0, h->stream>>>(
-                (const R*)X, ldx, k, a.row0, a.rows, a.rt, h->d_cmax, dA);
+            k_digits_rows<R><<<(unsigned)(a.rt * (MZ_M / 32)), 256, (size_t)k * sizeof(int), h->stream>>>(
+                (const R*)X, ldx, k, a.row0, a.rows, a.rt, h->d_cmax, dA, rexp);
         }
         HUB_CUDA_TRY(h, cudaGetLastError());
         ProfScope ps(h, HUB_K_ROTATE);

@@ -567,8 +567,8 @@ static int run_fx(hub_t h, const StencilArgs& s, int variant, const StencilDot* 
     return HUB_OK;
 }
 
-// CTA shapes (hub_set_tuning; 0 is the default), on 88 x 88 x 84 x 348 of normal deviates: 4.14, 4.15
-// and 4.12 ms.
+// CTA shapes (hub_set_tuning; 0 is the default), on 88 x 88 x 84 x 348 of normal deviates: 4.19, 4.17
+// and 4.16 ms.
 // Four CTAs of 192 threads hide the barriers of one another's planes; two rows per thread need
 // fewer instructions (382 against ~450 per point) but leave 16 warps per SM.
 int launch_stencil_fx(hub_t h, const StencilArgs& s) {

@@ -131,3 +131,28 @@ def test_scatter(prec, cplx):
     u = 2.0 ** -53 if prec == HUB_F64 else 2.0 ** -24
     terms = copies * np.count_nonzero(inside, axis=1)
     assert np.all(np.abs(got - ref) <= (16 * u * np.max(np.abs(P)) * terms * top)[:, None])
+
+
+@pytest.mark.parametrize("prec,ncol", [(HUB_F64, 12), (HUB_F64, 70), (HUB_F32, 140)])
+def test_rotation(prec, ncol):
+    """Orbitals with a common tail (a molecule and its vacuum): Rayleigh-Ritz returns X Q, and the rows of
+    the tail follow the Q that the rows of the molecule give, to rounding of their own size times the
+    condition of that fit (below 100)."""
+    n = (512, 16, 10)
+    Nd = n[0] * n[1] * n[2]
+    rng = np.random.default_rng(5)
+    d = np.abs(np.arange(512) - 256)
+    env = (1e-24 if prec == HUB_F64 else 1e-9) ** (d / 256.0)
+    hb = Hub(n, tuple(H * m for m in n), 6, prec=prec)
+    hb.set_veff(torch.tensor(rng.uniform(-1, 0, Nd), device="cuda"))
+    hb.set_atoms([])
+    X = torch.tensor((rng.standard_normal((ncol, n[1] * n[2], 512)) * env).reshape(ncol, Nd), device="cuda").to(hb.dtype)
+    X0 = X.double().cpu().numpy().reshape(ncol, -1, 512)
+    hb.rayleigh_ritz(0, X)
+    Y = X.double().cpu().numpy().reshape(ncol, -1, 512)
+    core = slice(236, 276)
+    Q = np.linalg.lstsq(X0[:, :, core].reshape(ncol, -1).T, Y[:, :, core].reshape(ncol, -1).T, rcond=None)[0]
+    err = np.abs(Y - np.einsum("kj,kyx->jyx", Q, X0)).max(axis=(0, 1))
+    size = np.abs(X0).max(axis=(0, 1)) * np.abs(Q).sum(axis=0).max()
+    u = 2.0 ** -53 if prec == HUB_F64 else 2.0 ** -24
+    assert np.all(err <= 100 * 16 * u * size)
