@@ -82,11 +82,6 @@ struct MzArgs {
     int* flags;
 };
 
-__device__ __forceinline__ uint32_t mz_desc(const void* p, uint32_t lbo) {
-    return ((saddr(p) & 0x3FFFF) >> 4) | ((lbo >> 4) << 16);      // high word as in the projector products
-}
-constexpr uint32_t kMzHi = 8u | (1u << 14);
-
 // tile t of the Gram product: rows 128 * i.x, columns 64 * i.y; a symmetric product has only the
 // tiles that reach the diagonal or beyond
 __device__ __forceinline__ int2 gram_tile(int t, int ct, int sym) {
@@ -179,7 +174,7 @@ k_mm_oz(const __grid_constant__ MzArgs a) {
     } else if (warp == 1) {
         const bool el = elect_one();
         auto wait = [&](uint64_t* bar, int parity) { return __all_sync(0xffffffffu, mbar_wait(bar, parity, &abort_flag)) != 0; };
-        const uint32_t a0 = mz_desc(ring, MZ_M * 16), b0 = mz_desc(ring + C::AB, S * MZ_N * 16);
+        const uint32_t a0 = desc_lo(ring, MZ_M * 16), b0 = desc_lo(ring + C::AB, S * MZ_N * 16);
         int s = 0, ph = 0, gi = 0;
         bool stop = false;
         for (int uu = 0; uu < nu && !stop; ++uu)
@@ -201,10 +196,10 @@ k_mm_oz(const __grid_constant__ MzArgs a) {
                             constexpr int kMax = 256;
                             const int n = (S < C::L - d ? S : C::L - d) * MZ_N;
                             const int cut = n > kMax ? kMax : (d == 1 && C::L > S ? n - MZ_N : n);
-                            mma_f16_lo(tmem + (uint32_t)(d * MZ_N), ao + (uint32_t)(d * 2 * MZ_M), bo, kMzHi,
+                            mma_f16_lo(tmem + (uint32_t)(d * MZ_N), ao + (uint32_t)(d * 2 * MZ_M), bo, kDescHi,
                                        instr_desc_f16(MZ_M, cut), d > 0 ? 1u : acc);
                             if (n > cut)
-                                mma_f16_lo(tmem + (uint32_t)(d * MZ_N + cut), ao + (uint32_t)(d * 2 * MZ_M), bo + (uint32_t)cut, kMzHi,
+                                mma_f16_lo(tmem + (uint32_t)(d * MZ_N + cut), ao + (uint32_t)(d * 2 * MZ_M), bo + (uint32_t)cut, kDescHi,
                                            instr_desc_f16(MZ_M, n - cut), d == 0 || C::L > S ? acc : 1u);
                         }
                         mma_commit(&empty_bar[s]);

@@ -106,11 +106,6 @@ struct SCfg {
     static_assert(SMEM <= 227 * 1024, "shared memory");
 };
 
-// descriptor words of a K-major operand without swizzle: 16-byte k units lbo bytes apart, 8-row
-// groups 128 bytes apart
-__device__ __forceinline__ uint32_t desc_lo(const void* p, uint32_t lbo) { return ((saddr(p) & 0x3FFFF) >> 4) | ((lbo >> 4) << 16); }
-constexpr uint32_t kDescHi = 8u | (1u << 14);
-
 struct OzGather {
     const void* X;
     const int4* grp;          // brick, slots, 16-byte offset, first slot

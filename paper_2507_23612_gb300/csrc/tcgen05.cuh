@@ -82,6 +82,10 @@ __device__ __forceinline__ bool elect_one() {
     asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}" : "=r"(p));
     return p != 0;
 }
+// descriptor words of a K-major operand without swizzle: 16-byte k units lbo bytes apart, 8-row
+// groups 128 bytes apart
+__device__ __forceinline__ uint32_t desc_lo(const void* p, uint32_t lbo) { return ((saddr(p) & 0x3FFFF) >> 4) | ((lbo >> 4) << 16); }
+constexpr uint32_t kDescHi = 8u | (1u << 14);
 __device__ __forceinline__ void mma_f16_lo(uint32_t tmem_d, uint32_t a_lo, uint32_t b_lo, uint32_t hi, uint32_t idesc,
                                            uint32_t acc) {
     asm volatile("{\n .reg .pred p;\n .reg .b64 a, b;\n setp.ne.b32 p, %5, 0;\n mov.b64 a, {%1, %3};\n mov.b64 b, {%2, %3};\n"
