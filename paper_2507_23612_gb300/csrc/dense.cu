@@ -245,11 +245,11 @@ __device__ __forceinline__ int exponent_of(double v) { return (__double2hiint(v)
 
 // c and sg = s exp(i arg a_pq) of the rotation that zeroes a_pq: s = t c, t the smaller root of
 // |a_pq| t^2 + (a_qq - a_pp) t = |a_pq|.  t, 1 / sqrt(1 + t^2) and the phase are estimated in float
-// (2^-22) and corrected once in double (t to 2^-43, the others to rounding), so that the coupling
-// falls below the convergence threshold and one step ends a 2 x 2 problem.  (The divisions and
-// square roots of a double angle are some 50 dependent instructions of the FP64 pipe, of about 64
-// clocks each; these are 11.
-// Left at the float estimates, a step costs 0.15 us less and the coupling falls to 2^-22.)
+// (2^-22) and corrected in double to rounding (t twice, 2^-43 and 2^-65), so that the coupling falls to
+// a few ulp and one step ends a 2 x 2 problem.  (The divisions and square roots of a double angle
+// are some 50 dependent instructions of the FP64 pipe, of about 64 clocks each; these are 14.
+// Left at the float estimates, a step costs 0.25 us less and the coupling falls to 2^-22; the second
+// correction of t costs 0.08 us of it.)
 template <typename T>
 __device__ __forceinline__ void jacobi_angle(double app, double aqq, T apq, double& c, T& sg) {
     constexpr bool CPLX = sizeof(T) == 16;
@@ -282,7 +282,8 @@ __device__ __forceinline__ void jacobi_angle(double app, double aqq, T apq, doub
     const float tf = __fdividef(mf, df + sqrtf(fmaf(df, df, mf * mf)));
     const double t0 = (double)tf, y = (double)rsqrtf(fmaf(tf, tf, 1.0f)), y2 = y * y;
     const double g = (double)__fdividef(1.0f, fmaf(mf, tf, df));          // one over the derivative
-    const double t = fma(-fma(fma(a, t0, D), t0, -a), g, t0);
+    const double t1 = fma(-fma(fma(a, t0, D), t0, -a), g, t0);            // 2^-43
+    const double t = fma(-fma(fma(a, t1, D), t1, -a), g, t1);
     const double u = fma(t, t, 1.0), ty = t * y;
     const double h = fma(-u, y2, 1.0), k = fma(0.375, h, 0.5);
     c = fma(y * h, k, y);                                                  // y (1 + h/2 + 3 h^2/8)
@@ -324,7 +325,7 @@ struct JacobiArgs {
 //     shared memory (in global memory if they don't fit) and applies the angles of the step before,
 //     which the CTAs of the diagonal groups leave in memory, between its arrival and the release.
 //     One warp only waits.
-// 348 orbitals: 29.9 -> 14.0 ms (58: 3.3 -> 1.7 ms; complex 348: 53.2 -> 22.6 ms) against every CTA
+// 348 orbitals: 29.9 -> 14.2 ms (58: 3.3 -> 1.7 ms; complex 348: 53.2 -> 21 ms) against every CTA
 // computing every angle in double and V between the loads and the barrier.  Of a step's 8300 clocks
 // 2600 go into loads and angles, 1700 into the update, 1000 into the stores and 1700 into the wait.
 // The rotation of a pair (p, q) is J = [[c, sg], [-conj(sg), c]] with c real and
@@ -650,7 +651,11 @@ int jacobi_t(hub_t h, int nmat, T* const* A, T* const* V, double* const* eig, in
     a.n = n;
     a.N = N;
     a.max_sweeps = 60;
-    a.tol = 1e-13;
+    // A coupling c that is left turns two orbitals by c / gap.  With 1e-13 for doubles, small blocks
+    // (2 to 20 orbitals, 84 blocks) that stopped just below it had D and density wrong by up to 2e-12;
+    // with 1e-15 all are within 3e-14 (median 5e-15 in both), for a sweep more in one block of eight.
+    // Rounding doesn't hold couplings up: a rotation rounds each to an ulp of itself.
+    a.tol = h->esize == 8 ? 1e-15 : 1e-13;
     HUB_CUDA_TRY(h, cudaMemsetAsync(h->d_bar, 0, 4 * sizeof(unsigned int), h->stream));
     HUB_CUDA_TRY(h, cudaMemsetAsync(a.sweeps, 0, 2 * sizeof(int), h->stream));
     if ((size_t)H * RS * sizeof(double) > 48 * 1024) return fail(h, HUB_EINVAL, "subspace too large for the Jacobi solver");
