@@ -274,7 +274,8 @@ def kernel_roofline(name, t_n, wl, prec, function_points):
         out = {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
                "traffic": traffic * pts_orb if traffic else None, "traffic_unit": "DRAM bytes per launch",
                "kernel": name, "ms_per_launch": t_ms / n,
-               "peak_source": "FP64 pipe: 152 SM x 2 FMA/clk x 2.07 GHz (nominal; bench.py --probe-alu measured 1.253)"}
+               "peak_source": "FP64 pipe: 152 SM x 2 FMA/clk x 2.07 GHz (nominal; bench.py --probe-alu measured 1.253)",
+               "runs_on": "integer pipes" if name == "stencil" else "FP16 tensor cores (8-bit digits)"}
         gbs = {"stencil": 24.0, "gather": 8.0, "scatter": 16.0}[name] * pts_orb / per_launch_s / 1e9
         out["hbm_achieved_gbs"], out["hbm_frac"] = gbs, gbs / hbm_peak()[0]
         if name == "stencil":

@@ -56,7 +56,7 @@ typedef enum {
 } hub_status;
 
 typedef enum {
-    HUB_F64 = 0,          /* every step in double */
+    HUB_F64 = 0,          /* blocks, results and dense steps in double; sums: see Accuracy */
     HUB_F32 = 1,          /* filter and Rayleigh-Ritz products in float; dense steps double */
     HUB_MIXED_BF16 = 2,   /* float filter; X^T X (always the hi/lo BF16 split), X^T H X and
                              X Q as BF16 tensor-core products with float accumulation;
@@ -66,6 +66,22 @@ typedef enum {
                              of two so that its largest magnitude lies in [2^14, 2^15) (FP16
                              overflows at 65504), the scale is removed from the FP32 result */
 } hub_prec;
+
+/* Accuracy.  GB300 adds and multiplies doubles at 1/63 of the float rate, so the large sums of products
+ * of HUB_F64 handles are taken in integers, where that is the faster form:
+ *   - H x of a real block: the stencil and the potential in 64-bit fixed point.  An element of x counts
+ *     with an error of at most 2^-59 of the largest |x| of its neighbourhood (at most 70 x 30 points
+ *     along x and y and a chunk of the planes, n3/4 more at both ends);
+ *   - projector products: operands of 54 bits below the largest |x| around a brick of 8 x 8 x 4
+ *     points (hub_project), the largest coefficient of the brick's functions (hub_expand), and the
+ *     function's largest value;
+ *   - rotations in Rayleigh-Ritz (real): 54 bits below the largest orbital at each grid point; Gram
+ *     products (real): 54 bits below each column's largest magnitude.
+ * Every sum is rounded once.  Against 64-bit sums the errors relative to these magnitudes are those of
+ * double arithmetic; an element far below its neighbourhood has fewer significant bits than a sum of
+ * its own would have.  Projector products of complex float blocks, and Gram products and rotations of
+ * large real float blocks, are taken the same way with 30 bits.  Columns with values that are not
+ * finite or beyond 2^+-900 (2^+-87 for float) are summed in floating point. */
 
 /* Create a handle for one grid, one Bloch wavevector and one precision.
  *   n1,n2,n3      grid points per axis (each >= 1)
@@ -164,8 +180,8 @@ int hub_chefsi_filter(hub_t h, int spin, void* X, int ncol, int ld, int degree,
  * 1: S and H^ are Hermitian, L is complex lower triangular with a real diagonal and the
  * eigensolver is a complex Jacobi).  Mixed handles take the block products of a complex
  * block in float on CUDA cores (the 16-bit tensor-core products are real only).
- * Errors: HUB_ENOTSPD (X rank-deficient), HUB_ENOCONV (Jacobi sweep limit),
- * HUB_ETIMEOUT, HUB_EINVAL. */
+ * Errors: HUB_ENOTSPD (a pivot of S is not positive: X rank-deficient), HUB_ENOCONV (Jacobi
+ * sweep limit), HUB_ETIMEOUT, HUB_EINVAL. */
 int hub_rayleigh_ritz(hub_t h, int spin, void* X, int ncol, int ld, double* eig_host,
                       void* work);
 

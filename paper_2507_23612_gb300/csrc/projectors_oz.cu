@@ -4,7 +4,7 @@
 //
 // GB300's FP64 pipe does 2 multiply-adds per clock and SM, so the FP64 products of the
 // point-major form ran at its limit (gather 9.09 ms, scatter 8.99 ms on 88 x 88 x 84 x 348; now
-// 1.09 and 1.37 ms).  Both are small dense products per brick of 8 x 8 x 4 points, and here they run on the FP16
+// 1.12 and 1.33 ms).  Both are small dense products per brick of 8 x 8 x 4 points, and here they run on the FP16
 // tensor cores with operands split into 7 (double) or 4 (float) 8-bit digits (digits.cuh):
 // digit products and, where it counts, their sums are exact, so the result carries the rounding of
 // the operands to 54 (30) bits below the largest magnitude of the values of X, or of the coefficients,
@@ -32,7 +32,9 @@
 // convert and store the digits, and 8 warps add the levels of finished units.  Scatter kernel: units (brick, 256 reals, NT
 // orbitals); 2 (double) or 4 warps build the digits of W and 16 update Y: with 8, in one set, a unit's
 // loads of Y waited for the stores of the one before (1.50 -> 1.37 ms); complex float needs the four
-// builders as well (88 x 88 x 56 x 230: 0.94 -> 0.67 ms; with two 0.97).  Every mbarrier wait is
+// builders as well (88 x 88 x 56 x 230: 0.94 -> 0.67 ms; with two 0.97).  Bounds in FP64 (88 x 88 x 28 x
+// 128): the gather's ALU pipe, 70 % busy with the digits of X (tensor pipe 22 %, DRAM 33 %); the
+// scatter's FP64 pipe, 62 % busy with the conversion and addition of its results (DRAM 39 %).  Every mbarrier wait is
 // bounded: after its limit the CTA raises FLAG_TIMEOUT, stops issuing, drains what it issued,
 // frees its TMEM and returns.
 //

@@ -32,9 +32,11 @@
 // Kernel: one CTA owns a tile of the x-y plane of one column and marches along z.  A ring of 8
 // planes (with a halo of 6 in x and y) in shared memory holds the limbs; plane z + 7 is
 // converted and stored while plane z is computed, and plane z + 8 is in flight in registers, so
-// there is one barrier per plane.  The 13 z-neighbours live in registers.  Bound: the integer
-// pipes (50 multiply-adds at half rate and ~310 other instructions per point); 17.15 -> 4.35 ms
-// on 88 x 88 x 84 x 348 (DRAM floor 0.80 ms), plus 0.27 ms for the maxima.
+// there is one barrier per plane.  The 13 z-neighbours live in registers.  Bound by instruction
+// issue (50 multiply-adds at half rate and ~310 other instructions per point: 62 % of the issue
+// slots, ALU pipe 44 %, multiply-adds 32 %, DRAM 9 % on 88 x 88 x 28 x 128, waits for loads and for
+// the plane barriers between); 17.15 -> 4.35 ms on 88 x 88 x 84 x 348 (DRAM floor 0.80 ms), plus
+// 0.27 ms for the maxima.
 #include <algorithm>
 #include <cmath>
 
