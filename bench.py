@@ -219,13 +219,16 @@ def cpu_oracle_sample(workload: str, seconds: float, cols: int = 2, procs: int =
 # kernel whose source has changed since reports traffic null until it is captured again.
 # Captured on the rutile 2x2x3 workload (348 orbitals, one launch = 226.4 M point-orbitals)
 # with `ncu --metrics dram__bytes_read.sum,dram__bytes_write.sum,gpu__time_duration.sum
-# --clock-control none -k regex:"k_stencil|k_gather|k_scatter" -s 300 -c 6` around `python bench.py
-# --prec f32 --steps 1 --warmup 1 --no-scf-tts --no-e2e --no-cpu-baseline`; the float gather and
-# scatter are the tensor-core brick forms.
+# --clock-control none -k regex:"k_stencil|k_gather|k_scatter" -s 6 -c 6` around one chefsi_filter of
+# degree 4; the FP64 kernels are the fixed-point stencil and the digit products, the float gather
+# and scatter the tensor-core brick forms.
 TRAFFIC_CAPTURES = {
-    ("f32", "stencil"): (12.52, "stencil.cu", "7095f36bbcbc94c0"),
-    ("f32", "gather"): (5.71, "projectors_tc.cu", "c1f826507f2e5e4b"),
-    ("f32", "scatter"): (10.42, "projectors_tc.cu", "c1f826507f2e5e4b"),
+    ("f64", "stencil"): (25.16, "stencil_fx.cu", "0c947dfa451acbd5"),
+    ("f64", "gather"): (11.28, "projectors_oz.cu", "42d64dc68ce5849a"),
+    ("f64", "scatter"): (18.26, "projectors_oz.cu", "42d64dc68ce5849a"),
+    ("f32", "stencil"): (12.53, "stencil.cu", "8be285ea9ac8b708"),
+    ("f32", "gather"): (5.73, "projectors_tc.cu", "94da405c3234112b"),
+    ("f32", "scatter"): (10.13, "projectors_tc.cu", "94da405c3234112b"),
 }
 
 
